@@ -801,8 +801,9 @@ private:
         if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc", __LINE__);
         allocs.push_back(q);
         p = (T *)q;
-        e = cudaMemset(q, 0, std::max<size_t>(n, 1) * sizeof(T));
-        if (e != cudaSuccess) return cuda_fail(e, "cudaMemset", __LINE__);
+        // on the handle's stream, which does not wait for the default one: the uploads that follow come after it
+        e = cudaMemsetAsync(q, 0, std::max<size_t>(n, 1) * sizeof(T), s);
+        if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync", __LINE__);
         return SIM_OK;
     }
 
