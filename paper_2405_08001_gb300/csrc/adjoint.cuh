@@ -266,15 +266,15 @@ __global__ void k_adj_out(Dev<R> D, const double *lam, const double *av, double 
 }
 // dE_e -= lambda_e . d g_e / d E_e: the tet's elastic gradient is linear in E_e (mu and lambda are), so its
 // derivative is the gradient evaluated with E_e = 1 (D carries mu and lambda of E = 1 and no per-tet scale)
-template <typename R>
+template <typename R, bool CO = false>
 __global__ void __launch_bounds__(EB) k_adj_youngs(Dev<R> D, const double *lam, double *dE)
 {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= D.nt) return;
     TetIn<R> in;
-    load_tet_in<R>(D, e, in);
+    load_tet_in<R, CO>(D, e, in);
     R gv[4][3], dv[4][3];
-    if (!tet_grad_eval<R>(D, in, gv, dv)) return;
+    if (!tet_grad_eval<R, CO>(D, in, gv, dv)) return;
     const int vid[4] = {in.tv.x, in.tv.y, in.tv.z, in.tv.w};
     double s = 0.0;
 #pragma unroll

@@ -24,11 +24,17 @@ template <typename R> struct Dev {
     float4 *xh, *xl;                   // FP32 form: float-float copy of x (hi, lo); null in the FP64 form
     float4 *xbh;                       // FP32 form: xh at the last candidate build (displacement check)
     float4 *xth, *xtl;                 // FP32 form: float-float copy of xtil (hi with w = xtil.w, lo)
-    const float *G0;                   // FP32 form: [14][nt] rest metric Dm^T Dm of each tet as float-float (six
-                                       // heads, six tails), then det Dm as float-float
-                                       // (hi of entries 00 01 02 11 12 22, then lo)
-    float4 *tS;                        // FP32 form: [4][nt] of the last gradient pass per tet: S = 2 dPsi/dC and
-                                       // C^-1 (entries 00 01 02 11 12 22 each), k1, k2, 0, 0 (tet_pHp_vec)
+    const float *G0;                   // FP32 corotated densities: [14][nt] rest metric Dm^T Dm of each tet as
+                                       // float-float (six heads, six tails: entries 00 01 02 11 12 22), then det Dm
+                                       // as float-float; null otherwise
+    const float4 *tc;                  // FP32 form: [5][nt] constants of each tet: the 14 values of G0, then h^2 V M
+                                       // (entries 00 01 02 11 12 22), M = Dm^-1 Dm^-T
+    const double4_32a *td;             // FP64 form: [2][nt] constants of each tet: h^2 V M (the six entries), det Dm^-1,
+                                       // h^2 V
+    float4 *tS;                        // FP32 form: [4][nt] record of the last gradient pass per tet for tet_pHp_vec:
+                                       // Z = Ds^-T (row-major), h^2 V Ds^-1 P Dm^-T (00 01 02 11 12 22), h^2 V k2
+    R *tk;                             // the record's scalars: FP32 form [nt] h^2 V k1; FP64 form [2][nt]
+                                       // h^2 V Psi_33 det(Dm^-1)^2 and h^2 V Psi_3 det(Dm^-1)
     R4 *g[2], *dg[2];                  // ping-pong by iteration parity; g.w = plane curvature kappa b'', dg.w = xtil.w
     R4 *p;
     R4 *pg, *pnext;                    // persistent form: P g of the current iteration, the next direction
@@ -399,26 +405,56 @@ template <typename R> __device__ inline void tet_material(const Dev<R> &D, int e
     if (D.escale) { R s = D.escale[e]; mu *= s; lam *= s; }
 }
 
-// The per-tet constants a gradient evaluation streams in (coalesced, structure-of-arrays in memory): indices,
-// D_m^-1, h^2 V, the Young's modulus scale and, in the FP32 form, the float-float rest metric.
+// The per-tet constants a gradient evaluation streams in (coalesced, structure-of-arrays in memory).  The densities
+// without an I1 term work on the edge vectors (tet_grad_edges) and need no D_m^-1; FCR and ARAP do.
 template <typename R> struct TetIn {
     int4 tv;
-    R w[3][3];
-    R hv, es;
+    R w[3][3];      // FCR, ARAP: rows of D_m^-1
+    R m[6];         // h^2 V M, M = D_m^-1 D_m^-T, entries 00 01 02 11 12 22
+    R dw;           // FP64 form: det D_m^-1
+    R hv, es;       // h^2 V, the Young's modulus scale
     float g0[14];   // FP32 form: rest metric entries 00 01 02 11 12 22, heads then tails; det Dm head, tail
 };
-template <typename R> __device__ inline void load_tet_in(const Dev<R> &D, int e, TetIn<R> &in)
+template <typename R, bool CO = false> __device__ inline void load_tet_in(const Dev<R> &D, int e, TetIn<R> &in)
 {
     in.tv = D.tet[e];
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) in.w[r][c] = D.Dm[(3 * r + c) * D.nt + e];
-    in.hv = D.hv[e];
     in.es = D.escale ? D.escale[e] : R(1);
     if constexpr (sizeof(R) == 4) {
+        in.hv = D.hv[e];
+        if constexpr (CO) {
+            load_w<R>(D, e, in.w);
 #pragma unroll
-        for (int q = 0; q < 14; ++q) in.g0[q] = D.G0[q * D.nt + e];
+            for (int q = 0; q < 14; ++q) in.g0[q] = D.G0[q * D.nt + e];
+        } else {
+            const size_t n = (size_t)D.nt;
+            const float4 a = D.tc[e], b = D.tc[n + e], c = D.tc[2 * n + e], d = D.tc[3 * n + e], f = D.tc[4 * n + e];
+            const float g[14] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w, d.x, d.y};
+#pragma unroll
+            for (int q = 0; q < 14; ++q) in.g0[q] = g[q];
+            in.m[0] = d.z; in.m[1] = d.w; in.m[2] = f.x; in.m[3] = f.y; in.m[4] = f.z; in.m[5] = f.w;
+        }
+    } else {
+        if constexpr (CO) {
+            load_w<R>(D, e, in.w);
+            in.hv = D.hv[e];
+        } else {
+            const double4_32a a = D.td[e], b = D.td[(size_t)D.nt + e];
+            in.m[0] = a.x; in.m[1] = a.y; in.m[2] = a.z; in.m[3] = a.w; in.m[4] = b.x; in.m[5] = b.y;
+            in.dw = b.z;
+            in.hv = b.w;
+        }
+    }
+}
+
+// cofactor matrix: columns s1 x s2, s2 x s0, s0 x s1 of the columns s0, s1, s2
+template <typename R> __device__ inline void cof3(const R s[3][3], R c[3][3])
+{
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const int p = (j + 1) % 3, q = (j + 2) % 3;
+        c[0][j] = s[1][p] * s[2][q] - s[2][p] * s[1][q];
+        c[1][j] = s[2][p] * s[0][q] - s[0][p] * s[2][q];
+        c[2][j] = s[0][p] * s[1][q] - s[1][p] * s[0][q];
     }
 }
 
@@ -581,35 +617,21 @@ static __device__ __noinline__ float corot_pHp(CorotPIn ci)
     return q;
 }
 
-// First Piola-Kirchhoff stress of the FP32 form, evaluated from the metric change so that it stays accurate for
-// small strains under any rotation.  With C = F^T F and a density of I2 and I3 (Sec. 3.1: NH or SNH) written in C,
-//   P = F^-T (mu (C - I) + (mu + Psi_3 J) I),   C - I = Dm^-T (Ds^T Ds - Dm^T Dm) Dm^-1,
-// which equals mu F + Psi_3 cof(F) (the I2/I3 form) exactly; mu + Psi_3 J is lambda log J for NH.  The metric
-// change G = Ds^T Ds - Dm^T Dm is accumulated in float-float from the float-float current positions and the tet's
-// float-float rest metric, and G W is formed with compensated products, so that rounding never acts on the parts
-// that cancel.  J - 1 = (det Ds - det Dm) / det Dm comes from det Ds in float-float and the tet's
-// float-float det Dm: under large shear a nearly incompressible tet keeps J near 1 while the entries of C - I are
-// of order one, and det C - 1 expanded in those entries cancels (lambda log J then carried about 1e-5 of the
-// stress).  F^-T = cof(F) / J.  Returns false (and flags the error) when det F <= 0.  Also returns Psi_33 for the
-// diagonal.
-template <bool CO>
-__device__ inline bool tet_stress_metric(const Dev<float> &D, const TetIn<float> &in, TetF<float> &T, float P[3][3],
-                                         float &Psi33, int e, CorotOut *cr = nullptr)
+// What the FP32 form's stresses start from: the edge vectors in float-float, their metric change G = Ds^T Ds - Dm^T Dm
+// accumulated in float-float against the tet's rest metric, so that rounding never acts on the parts that cancel, and
+// J - 1 = (det Ds - det Dm) / det Dm from det Ds in float-float: under large shear a nearly incompressible tet keeps J
+// near 1 while the entries of C - I are of order one, and det C - 1 expanded in those entries cancels (lambda log J
+// then carried about 1e-5 of the stress).
+__device__ inline void tet_metric(const Dev<float> &D, const TetIn<float> &in, ffl ds[3][3], ffl G[3][3], float &Jm1)
 {
-    const int4 tv = in.tv;
-    const int vid[4] = {tv.x, tv.y, tv.z, tv.w};
+    const int vid[4] = {in.tv.x, in.tv.y, in.tv.z, in.tv.w};
     float4 xh[4], xl[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) { xh[k] = ldcg4(D.xh + vid[k]); xl[k] = ldcg4(D.xl + vid[k]); }
-    float g0h[6], g0l[6];
-#pragma unroll
-    for (int q = 0; q < 6; ++q) { g0h[q] = in.g0[q]; g0l[q] = in.g0[6 + q]; }
-    ffl ds[3][3];
 #pragma unroll
     for (int c = 0; c < 3; ++c)
 #pragma unroll
         for (int a = 0; a < 3; ++a) ds[a][c] = ff_sub(comp(xh[c + 1], a), comp(xl[c + 1], a), comp(xh[0], a), comp(xl[0], a));
-    ffl G[3][3];
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -618,25 +640,163 @@ __device__ inline bool tet_stress_metric(const Dev<float> &D, const TetIn<float>
             ffacc acc = ffacc::prod(ds[0][i], ds[0][j]);
 #pragma unroll
             for (int a = 1; a < 3; ++a) acc.add_prod(ds[a][i], ds[a][j], 1.0f);
-            acc.sub_ff(g0h[q], g0l[q]);
+            acc.sub_ff(in.g0[q], in.g0[6 + q]);
             G[i][j] = G[j][i] = acc.ff();
         }
+    ffn a[3][3];
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) a[r][c] = ffn(ds[r][c].h, ds[r][c].l);
+    const ffn det = a[0][0] * (a[1][1] * a[2][2] - a[1][2] * a[2][1]) -
+                    a[0][1] * (a[1][0] * a[2][2] - a[1][2] * a[2][0]) +
+                    a[0][2] * (a[1][0] * a[2][1] - a[1][1] * a[2][0]);
+    const ffn dd = det - ffn(in.g0[12], in.g0[13]);
+    Jm1 = __fdiv_rn(__fadd_rn(dd.h, dd.l), in.g0[12]);
+}
+
+// Element gradient and Jacobi diagonal of the densities of I2 and I3 (NH, SNH) on the tet's edge vectors Ds (columns
+// x_i - x_0) instead of F = Ds Dm^-1: the corner forces of x_1..x_3 are the columns of
+//   h^2 V P Dm^-T = Ds (2 Psi_2 h^2 V M) + h^2 V Psi_3 det(Dm^-1) cof(Ds),    M = Dm^-1 Dm^-T,
+// and diag = 2 Psi_2 h^2 V M_ii + h^2 V Psi_33 (det(Dm^-1) cof(Ds)_ai)^2, so that neither F, its cofactors, the stress nor
+// their products with Dm^-1 are formed.  The FP32 form takes the forces from the metric change,
+//   h^2 V Ds^-T (mu G M + (mu + Psi_3 J) I),    G = Ds^T Ds - Dm^T Dm,
+// which equals the line above exactly and stays accurate for small strains under any rotation (mu + Psi_3 J is lambda
+// log J for NH); G M is formed with compensated (Dot2) products from the float-float G, its terms being up to
+// cond(Dm)^2 times larger than the result.  Both leave the record that tet_pHp_vec reads (e >= 0).  Returns false (and
+// flags the error) when det F <= 0.
+// FP64: 170 FP64 operations a tet where the form on F took about 430, at 1.65 FP64 lanes per clock and SM.
+template <typename R>
+__device__ inline bool tet_grad_edges(const Dev<R> &D, const TetIn<R> &in, R gv[4][3], R dv[4][3], int e)
+{
+    const R mu = D.mu * in.es, lam = D.lam * in.es;
+    R c[3][3];       // FP64: cof(Ds); FP32: Z = Ds^-T
+    R k33;           // diag's second term: k33 c_ai^2
+    R H[3][3];       // forces of x_1..x_3 (columns)
+    if constexpr (sizeof(R) == 4) {
+        ffl ds[3][3], G[3][3];
+        float Jm1;
+        tet_metric(D, in, ds, G, Jm1);
+        float s[3][3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) s[a][i] = ff_val(ds[a][i]);
+        cof3<float>(s, c);
+        const float J = 1.0f + Jm1;
+        if (!(J > 0.0f) || !(s[0][0] * c[0][0] + s[1][0] * c[1][0] + s[2][0] * c[2][0] > 0.0f)) {
+            flag_error(D.ctrl, ERR_INVERTED);
+            return false;
+        }
+        // mJ = mu + Psi_3 J: lambda log J (NH), (J - 1)(lambda J - mu) (SNH); k1 = J (Psi_33 J + Psi_3) / 4, k2 =
+        // -Psi_3 J / 2: the coefficients of p^T H p (tet_pHp_vec); k33 = h^2 V Psi_33 J^2
+        float mJ, k1, k2;
+        if (D.model == MAT_SNH) {
+            mJ = Jm1 * (lam * J - mu);
+            k33 = lam * J * J;
+            k1 = 0.25f * J * (lam * (J + Jm1) - mu);
+            k2 = 0.5f * J * (mu - lam * Jm1);
+        } else {
+            const float L = log1pf(Jm1);
+            mJ = lam * L;
+            k33 = mu + lam * (1.0f - L);
+            k1 = 0.25f * lam;
+            k2 = 0.5f * (mu - lam * L);
+        }
+        k33 *= in.hv;
+        const float id = 1.0f / (J * in.g0[12]);   // 1 / det Ds
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) c[a][i] *= id;
+        const float M[3][3] = {{in.m[0], in.m[1], in.m[2]}, {in.m[1], in.m[3], in.m[4]}, {in.m[2], in.m[4], in.m[5]}};
+        const float hj = in.hv * mJ;
+        float K[3][3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                ffacc acc = ffacc::prod_f(G[i][0], M[0][b]);
+#pragma unroll
+                for (int j = 1; j < 3; ++j) acc.add_prod_f(G[i][j], M[j][b]);
+                K[i][b] = mu * acc.value() + (i == b ? hj : 0.0f);
+            }
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) H[a][i] = c[a][0] * K[0][i] + c[a][1] * K[1][i] + c[a][2] * K[2][i];
+        if (e >= 0) {
+            float S[3][3];
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+#pragma unroll
+                for (int j = i; j < 3; ++j) S[i][j] = c[0][i] * H[0][j] + c[1][i] * H[1][j] + c[2][i] * H[2][j];
+            const size_t n = (size_t)D.nt;
+            D.tS[e] = make_float4(c[0][0], c[0][1], c[0][2], c[1][0]);
+            D.tS[n + e] = make_float4(c[1][1], c[1][2], c[2][0], c[2][1]);
+            D.tS[2 * n + e] = make_float4(c[2][2], S[0][0], S[0][1], S[0][2]);
+            D.tS[3 * n + e] = make_float4(S[1][1], S[1][2], S[2][2], in.hv * k2);
+            D.tk[e] = in.hv * k1;
+        }
+    } else {
+        R s[3][3];
+        tet_ds<R>(D, in.tv, s);
+        cof3<R>(s, c);
+        const R J = in.dw * (s[0][0] * c[0][0] + s[1][0] * c[1][0] + s[2][0] * c[2][0]);
+        if (!(J > R(0))) { flag_error(D.ctrl, ERR_INVERTED); return false; }
+        const R hd = in.hv * in.dw;
+        R k3;
+        if (D.model == MAT_SNH) {
+            k3 = hd * (lam * (J - R(1)) - mu);
+            k33 = hd * in.dw * lam;
+        } else {
+            const R L = log(J), ij = R(1) / J, q = hd * ij;
+            k3 = q * (lam * L - mu);
+            k33 = q * (in.dw * ij) * (mu + lam * (R(1) - L));
+        }
+        if (e >= 0) {
+            D.tk[e] = k33;
+            D.tk[(size_t)D.nt + e] = k3;
+        }
+        const R M[3][3] = {{mu * in.m[0], mu * in.m[1], mu * in.m[2]}, {mu * in.m[1], mu * in.m[3], mu * in.m[4]},
+                           {mu * in.m[2], mu * in.m[4], mu * in.m[5]}};
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) H[a][i] = s[a][0] * M[0][i] + s[a][1] * M[1][i] + s[a][2] * M[2][i] + k3 * c[a][i];
+    }
+    const R m0 = mu * in.m[0], m1 = mu * in.m[3], m2 = mu * in.m[5];
+    const R ms = m0 + m1 + m2 + R(2) * mu * (in.m[1] + in.m[2] + in.m[4]);   // x_0's weights are minus the others' sum
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        gv[1][a] = H[a][0]; gv[2][a] = H[a][1]; gv[3][a] = H[a][2];
+        gv[0][a] = -(H[a][0] + H[a][1] + H[a][2]);
+        const R cs = c[a][0] + c[a][1] + c[a][2];
+        dv[0][a] = ms + k33 * (cs * cs);
+        dv[1][a] = m0 + k33 * (c[a][0] * c[a][0]);
+        dv[2][a] = m1 + k33 * (c[a][1] * c[a][1]);
+        dv[3][a] = m2 + k33 * (c[a][2] * c[a][2]);
+    }
+    return true;
+}
+
+// The corotated densities' stress in the FP32 form: from the metric change A = C - I = W^T G W, W = Dm^-1 (G W with
+// compensated products from the float-float G, rounded once, then W^T (G W) in float), and F; corot_terms has the
+// rest.  Writes their p^T H p record (e >= 0).  Returns false (and flags the error) when det F <= 0.
+__device__ inline bool tet_stress_corot(const Dev<float> &D, const TetIn<float> &in, TetF<float> &T, CorotOut &co, int e)
+{
+    ffl ds[3][3], G[3][3];
+    float Jm1;
+    tet_metric(D, in, ds, G, Jm1);
     float dsf[3][3];
 #pragma unroll
     for (int a = 0; a < 3; ++a)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) dsf[a][c] = ff_val(ds[a][c]);
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) T.w[r][c] = in.w[r][c];
+        for (int c = 0; c < 3; ++c) { dsf[a][c] = ff_val(ds[a][c]); T.w[a][c] = in.w[a][c]; }
     tet_F_from<float>(dsf, T);
-    if (!(T.J > 0.0f)) { flag_error(D.ctrl, ERR_INVERTED); return false; }
-    // A = C - I = W^T G W with W = Dm^-1 (T.w[r][c] = W_rc): G W with compensated (Dot2) products from the
-    // float-float G, rounded once, then W^T (G W) in float.  The terms are up to cond(Dm)^2 times larger than A and
-    // cancel; in plain float from a rounded G that cost about 1e-6 of the stress on strongly sheared tets
-    // (compensating the second product as well gained nothing measurable)
-    float GW[3][3], A[3][3];
+    const float J = 1.0f + Jm1;
+    if (!(T.J > 0.0f) || !(J > 0.0f)) { flag_error(D.ctrl, ERR_INVERTED); return false; }
+    float GW[3][3];
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -646,134 +806,51 @@ __device__ inline bool tet_stress_metric(const Dev<float> &D, const TetIn<float>
             for (int j = 1; j < 3; ++j) acc.add_prod_f(G[i][j], T.w[j][b]);
             GW[i][b] = acc.value();
         }
+    CorotIn ci;
 #pragma unroll
     for (int a = 0; a < 3; ++a)
 #pragma unroll
-        for (int b = a; b < 3; ++b) A[a][b] = A[b][a] = T.w[0][a] * GW[0][b] + T.w[1][a] * GW[1][b] + T.w[2][a] * GW[2][b];
-    // J - 1 from det Ds (float-float; the edge vectors ds[a][c] = component a of edge c) and det Dm
-    float Jm1;
-    {
-        ffn a[3][3];
-#pragma unroll
-        for (int r = 0; r < 3; ++r)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) a[r][c] = ffn(ds[r][c].h, ds[r][c].l);
-        const ffn det = a[0][0] * (a[1][1] * a[2][2] - a[1][2] * a[2][1]) -
-                        a[0][1] * (a[1][0] * a[2][2] - a[1][2] * a[2][0]) +
-                        a[0][2] * (a[1][0] * a[2][1] - a[1][1] * a[2][0]);
-        const ffn dd = det - ffn(in.g0[12], in.g0[13]);
-        Jm1 = __fdiv_rn(__fadd_rn(dd.h, dd.l), in.g0[12]);
-    }
-    const float J = 1.0f + Jm1;
-    if (!(J > 0.0f)) { flag_error(D.ctrl, ERR_INVERTED); return false; }
-    const float detC = J * J;
-    const float mu = D.mu * in.es, lam = D.lam * in.es;
-    if (CO && (D.model == MAT_FCR || D.model == MAT_ARAP)) {
-        CorotIn ci;
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b) { ci.A[a][b] = A[a][b]; ci.F[a][b] = T.F[a][b]; ci.cf[a][b] = T.cf[a][b]; ci.w[a][b] = T.w[a][b]; }
-        ci.J = J; ci.Jm1 = Jm1; ci.mu = mu; ci.lam = lam; ci.hv = in.hv; ci.fcr = D.model == MAT_FCR;
-        const CorotOut co = corot_terms(ci);
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b) P[a][b] = co.P[a][b];
-        Psi33 = co.Psi33;
-        if (cr) *cr = co;
-        if (e >= 0) {   // R, Dq and J - 1 for the p^T H p pass
-            const size_t n = (size_t)D.nt;
-            D.tS[e] = make_float4(co.rec[0], co.rec[1], co.rec[2], co.rec[3]);
-            D.tS[n + e] = make_float4(co.rec[4], co.rec[5], co.rec[6], co.rec[7]);
-            D.tS[2 * n + e] = make_float4(co.rec[8], co.rec[9], co.rec[10], co.rec[11]);
-            D.tS[3 * n + e] = make_float4(co.rec[12], co.rec[13], co.rec[14], co.rec[15]);
-        }
-        return true;
-    }
-    // mJ = mu + Psi_3 J: lambda log J (NH), (J - 1)(lambda J - mu) (SNH)
-    // k1 = J (Psi_33 J + Psi_3) / 4, k2 = -Psi_3 J / 2: the coefficients of p^T H p in C (tet_pHp_vec)
-    float mJ, k1, k2;
-    if (D.model == MAT_SNH) {
-        mJ = Jm1 * (lam * J - mu);
-        Psi33 = lam;
-        k1 = 0.25f * J * (lam * (J + Jm1) - mu);
-        k2 = 0.5f * J * (mu - lam * Jm1);
-    } else {
-        const float L = log1pf(Jm1);                                                // log J
-        mJ = lam * L;
-        Psi33 = (mu + lam * (1.0f - L)) / detC;
-        k1 = 0.25f * lam;
-        k2 = 0.5f * (mu - lam * L);
-    }
-    // C^-1 = cof(C) / det C (C symmetric)
-    const float c00 = 1.0f + A[0][0], c11 = 1.0f + A[1][1], c22 = 1.0f + A[2][2];
-    const float ic = 1.0f / detC;
-    float Ci[3][3];
-    Ci[0][0] = (c11 * c22 - A[1][2] * A[1][2]) * ic;
-    Ci[1][1] = (c00 * c22 - A[0][2] * A[0][2]) * ic;
-    Ci[2][2] = (c00 * c11 - A[0][1] * A[0][1]) * ic;
-    Ci[0][1] = Ci[1][0] = (A[0][2] * A[1][2] - A[0][1] * c22) * ic;
-    Ci[0][2] = Ci[2][0] = (A[0][1] * A[1][2] - A[0][2] * c11) * ic;
-    Ci[1][2] = Ci[2][1] = (A[0][1] * A[0][2] - A[1][2] * c00) * ic;
-    float M[3][3];
+        for (int b = a; b < 3; ++b) ci.A[a][b] = ci.A[b][a] = T.w[0][a] * GW[0][b] + T.w[1][a] * GW[1][b] + T.w[2][a] * GW[2][b];
 #pragma unroll
     for (int a = 0; a < 3; ++a)
 #pragma unroll
-        for (int b = 0; b < 3; ++b) M[a][b] = mu * A[a][b] + (a == b ? mJ : 0.0f);
-    float S[3][3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b) S[a][b] = Ci[a][0] * M[0][b] + Ci[a][1] * M[1][b] + Ci[a][2] * M[2][b];
-    // P = F^-T M with F^-T = cof(F) / J (T.cf[a][c] is the cofactor of F_ac)
-    const float sc = in.hv, sj = sc / J;
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b) P[a][b] = sj * (T.cf[a][0] * M[0][b] + T.cf[a][1] * M[1][b] + T.cf[a][2] * M[2][b]);
-    if (e >= 0) {   // S (symmetric: C^-1 commutes with C - I), C^-1, k1, k2 for the p^T H p pass
+        for (int b = 0; b < 3; ++b) { ci.F[a][b] = T.F[a][b]; ci.cf[a][b] = T.cf[a][b]; ci.w[a][b] = T.w[a][b]; }
+    ci.J = J; ci.Jm1 = Jm1; ci.mu = D.mu * in.es; ci.lam = D.lam * in.es; ci.hv = in.hv; ci.fcr = D.model == MAT_FCR;
+    co = corot_terms(ci);
+    if (e >= 0) {   // R, Dq and J - 1 for the p^T H p pass
         const size_t n = (size_t)D.nt;
-        D.tS[e] = make_float4(S[0][0], 0.5f * (S[0][1] + S[1][0]), 0.5f * (S[0][2] + S[2][0]), S[1][1]);
-        D.tS[n + e] = make_float4(0.5f * (S[1][2] + S[2][1]), S[2][2], Ci[0][0], Ci[0][1]);
-        D.tS[2 * n + e] = make_float4(Ci[0][2], Ci[1][1], Ci[1][2], Ci[2][2]);
-        D.tS[3 * n + e] = make_float4(k1, k2, 0.0f, 0.0f);
+        D.tS[e] = make_float4(co.rec[0], co.rec[1], co.rec[2], co.rec[3]);
+        D.tS[n + e] = make_float4(co.rec[4], co.rec[5], co.rec[6], co.rec[7]);
+        D.tS[2 * n + e] = make_float4(co.rec[8], co.rec[9], co.rec[10], co.rec[11]);
+        D.tS[3 * n + e] = make_float4(co.rec[12], co.rec[13], co.rec[14], co.rec[15]);
     }
     return true;
 }
 
-// Element gradient and Jacobi diagonal (Sec. 3.1 split; no density here has Psi_11 or Psi_22 terms and the H3
-// term has a zero diagonal, so diag_i[a] = h^2 V (2 Psi_2 |w_i|^2 + Psi_33 (cof(F) w_i)_a^2 + Psi_1 d2I1 entry)).  The contributions go to the
-// per-(tet, corner) buffer (segmented scatter), to the block's shared accumulators sacc ([6][SCATTER_MAXU],
-// indexed by the chunk-local vertex; block scatter) or straight to the global accumulators.
-template <typename R, bool CO = false>
-__device__ inline bool tet_grad_eval(const Dev<R> &D, const TetIn<R> &in, R gv[4][3], R dv[4][3], int e = -1)
+// The same for FCR and ARAP, on F, with the I1 terms in the stress and on the diagonal: diag_i[a] = h^2 V (2 Psi_2
+// |w_i|^2 + Psi_33 (cof(F) w_i)_a^2 + Psi_1 d2I1 entry), w_i the corner's weights.
+template <typename R>
+__device__ inline bool tet_grad_rotated(const Dev<R> &D, const TetIn<R> &in, R gv[4][3], R dv[4][3], int e)
 {
-    const int4 tv = in.tv;
     TetF<R> T;
     R P[3][3], Psi33;
     const R sc = in.hv;
-    const R mu = D.mu * in.es, lam = D.lam * in.es;
-    R c2 = mu;        // 2 Psi_2
-    R Psi1 = R(0);    // the I1 term (FCR, ARAP)
+    const R mu = D.mu * in.es, lam = D.lam * in.es, c2 = R(2) * mu;   // 2 Psi_2
     if constexpr (sizeof(R) == 4) {
-        if constexpr (CO) {
-            CorotOut cr;
-            if (!tet_stress_metric<true>(D, in, T, P, Psi33, e, &cr)) return false;
-            if (D.model == MAT_FCR || D.model == MAT_ARAP) {   // Psi_1 d2I1 on the diagonal
-                c2 = R(2) * mu;
-                Psi1 = R(-2) * mu;
+        CorotOut cr;
+        if (!tet_stress_corot(D, in, T, cr, e)) return false;
+        Psi33 = cr.Psi33;
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+        for (int a = 0; a < 3; ++a)
 #pragma unroll
-                    for (int a = 0; a < 3; ++a) dv[i][a] = cr.dv[i][a];
-            }
-        } else {
-            if (!tet_stress_metric<false>(D, in, T, P, Psi33, e)) return false;
-        }
+            for (int b = 0; b < 3; ++b) P[a][b] = cr.P[a][b];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) dv[i][a] = cr.dv[i][a];
     } else {
         R ds[3][3];
-        tet_ds<R>(D, tv, ds);
+        tet_ds<R>(D, in.tv, ds);
 #pragma unroll
         for (int r = 0; r < 3; ++r)
 #pragma unroll
@@ -782,57 +859,51 @@ __device__ inline bool tet_grad_eval(const Dev<R> &D, const TetIn<R> &in, R gv[4
         if (!(T.J > R(0))) { flag_error(D.ctrl, ERR_INVERTED); return false; }
         const MatTerms<R> mt = mat_terms<R>(D.model, mu, lam, T.J);
         Psi33 = mt.Psi33;
-        c2 = mt.c2;
-        Psi1 = mt.Psi1;
+        Polar pol;
+        polar_of(T.F, pol);
 #pragma unroll
         for (int a = 0; a < 3; ++a)
 #pragma unroll
-            for (int b = 0; b < 3; ++b) P[a][b] = sc * (c2 * T.F[a][b] + mt.Psi3 * T.cf[a][b]);
-        if (Psi1 != R(0)) {   // FCR, ARAP: Psi_1 R in the stress, Psi_1 d2I1 on the diagonal
-            Polar pol;
-            polar_of(T.F, pol);
+            for (int b = 0; b < 3; ++b) P[a][b] = sc * (c2 * T.F[a][b] + mt.Psi3 * T.cf[a][b]) + sc * mt.Psi1 * pol.R[a][b];
 #pragma unroll
-            for (int a = 0; a < 3; ++a)
+        for (int i = 0; i < 4; ++i) {
+            double w[3];
 #pragma unroll
-                for (int b = 0; b < 3; ++b) P[a][b] += sc * Psi1 * pol.R[a][b];
+            for (int b = 0; b < 3; ++b)
+                w[b] = i == 0 ? -(T.w[0][b] + T.w[1][b] + T.w[2][b]) : T.w[i - 1][b];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                double w[3];
-#pragma unroll
-                for (int b = 0; b < 3; ++b)
-                    w[b] = i == 0 ? -(T.w[0][b] + T.w[1][b] + T.w[2][b]) : T.w[i - 1][b];
-#pragma unroll
-                for (int a = 0; a < 3; ++a) dv[i][a] = sc * Psi1 * polar_h1_diag(pol, w, a);
-            }
+            for (int a = 0; a < 3; ++a) dv[i][a] = sc * mt.Psi1 * polar_h1_diag(pol, w, a);
         }
     }
-    const bool i1 = Psi1 != R(0);
 #pragma unroll
-    for (int i = 1; i < 4; ++i) {
-        const R *w = T.w[i - 1];
+    for (int i = 0; i < 4; ++i) {
+        R w[3];
+#pragma unroll
+        for (int b = 0; b < 3; ++b) w[b] = i == 0 ? -(T.w[0][b] + T.w[1][b] + T.w[2][b]) : T.w[i - 1][b];
         const R ww = w[0] * w[0] + w[1] * w[1] + w[2] * w[2];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             gv[i][a] = P[a][0] * w[0] + P[a][1] * w[1] + P[a][2] * w[2];
             const R cw = T.cf[a][0] * w[0] + T.cf[a][1] * w[1] + T.cf[a][2] * w[2];
-            dv[i][a] = (i1 ? dv[i][a] : R(0)) + sc * (c2 * ww + Psi33 * cw * cw);
+            dv[i][a] += sc * (c2 * ww + Psi33 * cw * cw);
         }
     }
-    {
-        R w0[3];
 #pragma unroll
-        for (int b = 0; b < 3; ++b) w0[b] = -(T.w[0][b] + T.w[1][b] + T.w[2][b]);
-        const R ww = w0[0] * w0[0] + w0[1] * w0[1] + w0[2] * w0[2];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            gv[0][a] = -(gv[1][a] + gv[2][a] + gv[3][a]);
-            const R cw = T.cf[a][0] * w0[0] + T.cf[a][1] * w0[1] + T.cf[a][2] * w0[2];
-            dv[0][a] = (i1 ? dv[0][a] : R(0)) + sc * (c2 * ww + Psi33 * cw * cw);
-        }
-    }
+    for (int a = 0; a < 3; ++a) gv[0][a] = -(gv[1][a] + gv[2][a] + gv[3][a]);
     return true;
 }
 
+// Element gradient and Jacobi diagonal (Sec. 3.1 split; no density here has Psi_11 or Psi_22 terms and the H3 term has a
+// zero diagonal) of one tet; e >= 0: leaves the record of the p^T H p pass.
+template <typename R, bool CO = false>
+__device__ inline bool tet_grad_eval(const Dev<R> &D, const TetIn<R> &in, R gv[4][3], R dv[4][3], int e = -1)
+{
+    if constexpr (CO) return tet_grad_rotated<R>(D, in, gv, dv, e);
+    else return tet_grad_edges<R>(D, in, gv, dv, e);
+}
+
+// The tet's contributions go to the per-(tet, corner) buffer (segmented scatter), to the block's shared accumulators
+// sacc ([6][SCATTER_MAXU], indexed by the chunk-local vertex; block scatter) or straight to the global accumulators.
 template <typename R, bool CO = false>
 __device__ inline void tet_grad(const Dev<R> &D, int e, int par, const TetIn<R> &in, R *sacc = nullptr)
 {
@@ -883,7 +954,7 @@ __device__ inline void tet_grad(const Dev<R> &D, int e, int par, const TetIn<R> 
 }
 
 // Colouring scatter: the tets of one colour (positions t0 .. t0 + n of the colour order), one thread each.  Dc is
-// D with the per-tet inputs (tet, Dm, hv, escale, G0) in colour order, so that the loads of a colour stay
+// D with the per-tet inputs (tet, Dm, hv, escale, G0, tc, td) in colour order, so that the loads of a colour stay
 // coalesced; the record of the p^T H p pass is written at the tet's own index color_tets[q].
 template <typename R, bool CO = false>
 __global__ void __launch_bounds__(EB) k_grad_color(Dev<R> D, Dev<R> Dc, int par, int t0, int n)
@@ -891,13 +962,13 @@ __global__ void __launch_bounds__(EB) k_grad_color(Dev<R> D, Dev<R> Dc, int par,
     const int q = t0 + (int)(blockIdx.x * blockDim.x + threadIdx.x);
     if (q >= t0 + n) return;
     TetIn<R> in;
-    load_tet_in<R>(Dc, q, in);
+    load_tet_in<R, CO>(Dc, q, in);
     tet_grad<R, CO>(D, D.color_tets[q], par, in);
 }
 
 // The colour-ordered copies of the per-tet inputs (once, at setup): position q holds tet color_tets[q].
 template <typename R>
-__global__ void k_color_gather(Dev<R> D, int4 *tet, R *Dm, R *hv, R *es, float *G0)
+__global__ void k_color_gather(Dev<R> D, int4 *tet, R *Dm, R *hv, R *es, float *G0, float4 *tc, double4_32a *td)
 {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= D.nt) return;
@@ -909,6 +980,10 @@ __global__ void k_color_gather(Dev<R> D, int4 *tet, R *Dm, R *hv, R *es, float *
     if (es) es[q] = D.escale[e];
     if (G0)
         for (int k = 0; k < 14; ++k) G0[k * n + q] = D.G0[k * n + e];
+    if (tc)
+        for (int k = 0; k < 5; ++k) tc[k * n + q] = D.tc[k * n + e];
+    if (td)
+        for (int k = 0; k < 2; ++k) td[k * n + q] = D.td[k * n + e];
 }
 
 // The tets of chunk ch (SCATTER_CHUNK consecutive tets, one per thread of the block): gradient and diagonal,
@@ -929,7 +1004,7 @@ __device__ inline void tet_grad_chunk(const Dev<R> &D, int ch, int par, R *sacc)
     }
     if (e < D.nt) {
         TetIn<R> in;
-        load_tet_in<R>(D, e, in);
+        load_tet_in<R, CO>(D, e, in);
         tet_grad<R, CO>(D, e, par, in, blk ? sacc : nullptr);
     }
     if (blk) {
@@ -1295,105 +1370,132 @@ __global__ void __launch_bounds__(VB) k_dir(Dev<R> D, int par)
 
 // ------------------------------------------------------------------------------------------ a6-a7: p^T H p, step
 
-// h^2 V [2 Psi_2 |dF|^2 + Psi_33 (cof(F) : dF)^2 + Psi_3 d2det(F)[dF, dF] + Psi_1 d2I1(F)[dF, dF]] (Sec. 3.1 with
-// H2 = 2I, H3 the det Hessian, H1 the Hessian of tr(S)) for the direction values P0..P3 of the tet's vertices.
+// p^T H p of one tet for the direction values P0..P3 of its vertices: h^2 V [2 Psi_2 |dF|^2 + Psi_33 (cof(F) : dF)^2 +
+// Psi_3 d2det(F)[dF, dF] + Psi_1 d2I1(F)[dF, dF]] (Sec. 3.1 with H2 = 2I, H3 the det Hessian, H1 the Hessian of
+// tr(S)), at the x of the last gradient pass, whose record it reads.  On the direction's edge vectors Dp (columns p_i -
+// p_0) for NH and SNH, so that neither D_m^-1 nor dF is needed:
+//   FP64: 2 Psi_2 h^2 V M : Dp^T Dp + h^2 V Psi_33 det(Dm^-1)^2 (cof(Ds) : Dp)^2 + h^2 V Psi_3 det(Dm^-1) 2 cof(Dp) : Ds
+// (about 115 FP64 operations; on F and with the scalars formed anew it took 330).
+//   FP32: the second derivative of Psi written in C = F^T F, S : dF^T dF + k1 (tr C^-1 E)^2 + k2 tr(C^-1 E C^-1 E), E =
+// dF^T F + F^T dF.  With L = dF F^-1 = Dp Ds^-1, tr C^-1 E = tr(L + L^T) and tr(C^-1 E C^-1 E) = |L + L^T|^2, and S : dF^T dF =
+// (Dm^-1 S Dm^-T) : Dp^T Dp.  A direction that rotates the tet cancels inside L + L^T, so the large terms mu |dF|^2 and
+// Psi_3 d2det(F)[dF, dF] of the I2/I3 form, which cancel for it, never meet in float.  The record (68 bytes: Ds^-T, the
+// weighted stress, k1, k2) stands in for the positions' eight gathers and D_m^-1.
+template <typename R>
+__device__ inline R tet_pHp_edges(const Dev<R> &D, int e, const int4 &tv, const R dp[3][3])
+{
+    const size_t n = (size_t)D.nt;
+    if constexpr (sizeof(R) == 4) {
+        const float4 q0 = __ldcg(D.tS + e), q1 = __ldcg(D.tS + n + e), q2 = __ldcg(D.tS + 2 * n + e);
+        const float4 q3 = __ldcg(D.tS + 3 * n + e);
+        const float k1 = __ldcg(D.tk + e);
+        const float Z[3][3] = {{q0.x, q0.y, q0.z}, {q0.w, q1.x, q1.y}, {q1.z, q1.w, q2.x}};
+        float L[3][3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) L[a][b] = dp[a][0] * Z[b][0] + dp[a][1] * Z[b][1] + dp[a][2] * Z[b][2];
+        const float e0 = 2.0f * L[0][0], e1 = 2.0f * L[1][1], e2 = 2.0f * L[2][2];
+        const float e01 = L[0][1] + L[1][0], e02 = L[0][2] + L[2][0], e12 = L[1][2] + L[2][1];
+        const float tr = e0 + e1 + e2;
+        const float t2 = e0 * e0 + e1 * e1 + e2 * e2 + 2.0f * (e01 * e01 + e02 * e02 + e12 * e12);
+        float g[3][3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = i; j < 3; ++j) g[i][j] = dp[0][i] * dp[0][j] + dp[1][i] * dp[1][j] + dp[2][i] * dp[2][j];
+        const float SD = q2.y * g[0][0] + q3.x * g[1][1] + q3.z * g[2][2] +
+                         2.0f * (q2.z * g[0][1] + q2.w * g[0][2] + q3.y * g[1][2]);
+        return SD + k1 * tr * tr + q3.w * t2;
+    } else {
+        R mu, lam;
+        tet_material<R>(D, e, mu, lam);
+        const double4_32a a = D.td[e], b = D.td[n + e];
+        const R k33 = __ldcg(D.tk + e), k3 = __ldcg(D.tk + n + e);
+        R s[3][3], c[3][3];
+        tet_ds<R>(D, tv, s);
+        cof3<R>(s, c);
+        R g3 = R(0);
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) g3 += c[r][i] * dp[r][i];
+        cof3<R>(dp, c);
+        R h3 = R(0);
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) h3 += c[r][i] * s[r][i];
+        R g[3][3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = i; j < 3; ++j) g[i][j] = dp[0][i] * dp[0][j] + dp[1][i] * dp[1][j] + dp[2][i] * dp[2][j];
+        const R md = a.x * g[0][0] + a.w * g[1][1] + b.y * g[2][2] + R(2) * (a.y * g[0][1] + a.z * g[0][2] + b.x * g[1][2]);
+        return mu * md + k33 * (g3 * g3) + (R(2) * k3) * h3;
+    }
+}
+
+// The same for FCR and ARAP, on F; the FP32 form's record holds the rotation (corot_pHp).
+template <typename R>
+__device__ inline R tet_pHp_rotated(const Dev<R> &D, int e, const int4 &tv, const R dp[3][3])
+{
+    R mu, lam;
+    tet_material<R>(D, e, mu, lam);
+    if constexpr (sizeof(R) == 4) {
+        const size_t n = (size_t)D.nt;
+        const float4 q0 = __ldcg(D.tS + e), q1 = __ldcg(D.tS + n + e), q2 = __ldcg(D.tS + 2 * n + e);
+        const float4 q3 = __ldcg(D.tS + 3 * n + e);
+        TetF<R> T;
+        tet_F<R>(D, e, tv, T);
+        CorotPIn ci;
+        const float rq[16] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w, q2.x, q2.y, q2.z, q2.w,
+                              q3.x, q3.y, q3.z, q3.w};
+#pragma unroll
+        for (int k = 0; k < 16; ++k) ci.rec[k] = rq[k];
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                ci.dF[a][b] = dp[a][0] * T.w[0][b] + dp[a][1] * T.w[1][b] + dp[a][2] * T.w[2][b];
+                ci.F[a][b] = T.F[a][b];
+                ci.cf[a][b] = T.cf[a][b];
+            }
+        ci.mu = mu; ci.lam = lam; ci.fcr = D.model == MAT_FCR;
+        return D.hv[e] * corot_pHp(ci);
+    } else {
+        TetF<R> T;
+        tet_F<R>(D, e, tv, T);
+        if (!(T.J > R(0))) { flag_error(D.ctrl, ERR_INVERTED); return R(0); }
+        R dF[3][3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) dF[a][b] = dp[a][0] * T.w[0][b] + dp[a][1] * T.w[1][b] + dp[a][2] * T.w[2][b];
+        const MatTerms<R> mt = mat_terms<R>(D.model, mu, lam, T.J);
+        R n2 = 0, g3 = 0, h3 = 0;
+        R cd[3][3];
+        cof3<R>(dF, cd);
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) { n2 += dF[a][b] * dF[a][b]; g3 += T.cf[a][b] * dF[a][b]; h3 += cd[a][b] * T.F[a][b]; }
+        Polar pol;
+        polar_of(T.F, pol);
+        return D.hv[e] * (mt.c2 * n2 + mt.Psi33 * g3 * g3 + mt.Psi3 * (R(2) * h3) + mt.Psi1 * polar_h1(pol, dF));
+    }
+}
+
 template <typename R, bool CO = false>
 __device__ inline R tet_pHp_vec(const Dev<R> &D, int e, const int4 &tv, const typename V4<R>::T &P0,
                                 const typename V4<R>::T &P1, const typename V4<R>::T &P2, const typename V4<R>::T &P3)
 {
-    TetF<R> T;
-    tet_F<R>(D, e, tv, T);
-    if (!(T.J > R(0))) { flag_error(D.ctrl, ERR_INVERTED); return R(0); }
     R dp[3][3];
     dp[0][0] = P1.x - P0.x; dp[1][0] = P1.y - P0.y; dp[2][0] = P1.z - P0.z;
     dp[0][1] = P2.x - P0.x; dp[1][1] = P2.y - P0.y; dp[2][1] = P2.z - P0.z;
     dp[0][2] = P3.x - P0.x; dp[1][2] = P3.y - P0.y; dp[2][2] = P3.z - P0.z;
-    R dF[3][3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b) dF[a][b] = dp[a][0] * T.w[0][b] + dp[a][1] * T.w[1][b] + dp[a][2] * T.w[2][b];
-    if constexpr (sizeof(R) == 4) {
-        // FP32 form: the second derivative along dF of Psi written in C = F^T F,
-        //   S : dF^T dF + k1 (tr C^-1 E)^2 + k2 tr(C^-1 E C^-1 E),   E = dF^T F + F^T dF,
-        // with S = 2 dPsi/dC, C^-1, k1 = J (Psi_33 J + Psi_3) / 4, k2 = -Psi_3 J / 2 from the gradient pass at
-        // the same x (formed there from the metric change, accurate for small strains).  A direction that rotates
-        // the tet cancels inside E, so the large terms mu |dF|^2 and Psi_3 d2det(F)[dF, dF] of the I2/I3 form,
-        // which cancel for it, never meet in float.
-        const size_t n = (size_t)D.nt;
-        const float4 q0 = __ldcg(D.tS + e), q1 = __ldcg(D.tS + n + e), q2 = __ldcg(D.tS + 2 * n + e);
-        const float4 q3 = __ldcg(D.tS + 3 * n + e);
-        if (CO && (D.model == MAT_FCR || D.model == MAT_ARAP)) {
-            CorotPIn ci;
-            const float rq[16] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w, q2.x, q2.y, q2.z, q2.w,
-                                  q3.x, q3.y, q3.z, q3.w};
-#pragma unroll
-            for (int k = 0; k < 16; ++k) ci.rec[k] = rq[k];
-#pragma unroll
-            for (int a = 0; a < 3; ++a)
-#pragma unroll
-                for (int b = 0; b < 3; ++b) { ci.dF[a][b] = dF[a][b]; ci.F[a][b] = T.F[a][b]; ci.cf[a][b] = T.cf[a][b]; }
-            R mu, lam;
-            tet_material<R>(D, e, mu, lam);
-            ci.mu = mu; ci.lam = lam; ci.fcr = D.model == MAT_FCR;
-            return D.hv[e] * corot_pHp(ci);
-        }
-        const float S00 = q0.x, S01 = q0.y, S02 = q0.z, S11 = q0.w, S12 = q1.x, S22 = q1.y;
-        const float C00 = q1.z, C01 = q1.w, C02 = q2.x, C11 = q2.y, C12 = q2.z, C22 = q2.w;
-        const float k1 = q3.x, k2 = q3.y;
-        float E[3][3], DD[3][3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = a; b < 3; ++b) {
-                float fe = 0.0f, dd = 0.0f;
-#pragma unroll
-                for (int r = 0; r < 3; ++r) {
-                    fe += dF[r][a] * T.F[r][b] + T.F[r][a] * dF[r][b];
-                    dd += dF[r][a] * dF[r][b];
-                }
-                E[a][b] = E[b][a] = fe;
-                DD[a][b] = DD[b][a] = dd;
-            }
-        const float Ci[3][3] = {{C00, C01, C02}, {C01, C11, C12}, {C02, C12, C22}};
-        float X[3][3];   // C^-1 E
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b) X[a][b] = Ci[a][0] * E[0][b] + Ci[a][1] * E[1][b] + Ci[a][2] * E[2][b];
-        const float trX = X[0][0] + X[1][1] + X[2][2];
-        float trX2 = 0.0f;
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b) trX2 += X[a][b] * X[b][a];
-        const float SD = S00 * DD[0][0] + S11 * DD[1][1] + S22 * DD[2][2] +
-                         2.0f * (S01 * DD[0][1] + S02 * DD[0][2] + S12 * DD[1][2]);
-        return D.hv[e] * (SD + k1 * trX * trX + k2 * trX2);
-    }
-    R mu, lam;
-    tet_material<R>(D, e, mu, lam);
-    const MatTerms<R> mt = mat_terms<R>(D.model, mu, lam, T.J);
-    R n2 = 0, g3 = 0;
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b) { n2 += dF[a][b] * dF[a][b]; g3 += T.cf[a][b] * dF[a][b]; }
-    // columns: f_b = F[.][b], df_b = dF[.][b]
-    v3<R> f0 = mkv(T.F[0][0], T.F[1][0], T.F[2][0]), f1 = mkv(T.F[0][1], T.F[1][1], T.F[2][1]),
-          f2 = mkv(T.F[0][2], T.F[1][2], T.F[2][2]);
-    v3<R> d0 = mkv(dF[0][0], dF[1][0], dF[2][0]), d1 = mkv(dF[0][1], dF[1][1], dF[2][1]),
-          d2 = mkv(dF[0][2], dF[1][2], dF[2][2]);
-    const R h3 = R(2) * (dot(d0, cross(d1, f2)) + dot(d0, cross(f1, d2)) + dot(f0, cross(d1, d2)));
-    R q = mt.c2 * n2 + mt.Psi33 * g3 * g3 + mt.Psi3 * h3;
-    if constexpr (sizeof(R) == 8) {
-        if (mt.Psi1 != R(0)) {
-            Polar pol;
-            polar_of(T.F, pol);
-            q += mt.Psi1 * polar_h1(pol, dF);
-        }
-    }
-    return D.hv[e] * q;
+    if constexpr (CO) return tet_pHp_rotated<R>(D, e, tv, dp);
+    else return tet_pHp_edges<R>(D, e, tv, dp);
 }
 
 template <typename R, bool CO = false>

@@ -2,5 +2,5 @@
 #include "persist_shapes.cuh"
 
 namespace pncg {
-PNCG_PERSIST_DEF(float, 4)
+PNCG_PERSIST_DEF(float, 4, false)
 }

@@ -2,5 +2,5 @@
 #include "persist_shapes.cuh"
 
 namespace pncg {
-PNCG_PERSIST_DEF(double, 2)
+PNCG_PERSIST_DEF(double, 2, false)
 }

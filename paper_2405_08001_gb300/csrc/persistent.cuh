@@ -630,7 +630,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
                 const int nts = ts.b1 - ts.b0;
                 for (int q = threadIdx.x; q < nts; q += PB) {
                     TetIn<R> in;
-                    load_tet_in<R>(D, ts.b0 + q, in);
+                    load_tet_in<R, CO>(D, ts.b0 + q, in);
                     tet_grad<R, CO>(D, ts.b0 + q, par, in);
                 }
                 if (lead) c->ticket[TK_PAIRS + ((k + 1) & 1)] = 0u;   // the next iteration's cursor

@@ -734,7 +734,8 @@ public:
             D1.mu = R(1.0 / (2.0 * (1.0 + M.nu)));
             D1.lam = R(M.nu / ((1.0 + M.nu) * (1.0 - 2.0 * M.nu)));
             D1.escale = nullptr;
-            k_adj_youngs<R><<<(M.nt + EB - 1) / EB, EB, 0, s>>>(D1, adj_x, adj_dE);
+            if (corot) k_adj_youngs<R, true><<<(M.nt + EB - 1) / EB, EB, 0, s>>>(D1, adj_x, adj_dE);
+            else k_adj_youngs<R><<<(M.nt + EB - 1) / EB, EB, 0, s>>>(D1, adj_x, adj_dE);
             CK(cudaMemcpyAsync(dE, adj_dE, sizeof(double) * M.nt, cudaMemcpyDefault, s));
         }
         CK(cudaStreamSynchronize(s));
@@ -767,10 +768,12 @@ private:
     int4 *c_tet = nullptr;
     R *c_Dm = nullptr, *c_hv = nullptr, *c_es = nullptr;
     float *c_G0 = nullptr;
+    float4 *c_tc = nullptr;
+    double4_32a *c_td = nullptr;
     std::vector<cudaEvent_t> prof_ev;
     // persistent form
     bool persist = false;
-    bool corot = false;                // FP32 form with a corotated density (FCR, ARAP): its own kernel instantiations
+    bool corot = false;                // a corotated density (FCR, ARAP): its own kernel instantiations
     int shape = 0;                     // block shape of the persistent form (persist_shapes.cuh)
     int shape_grid[N_PSHAPES] = {};    // its grid (blocks), 0 = the shape cannot be launched
     std::vector<int> tune_cfg;         // autotuning candidates: shape index, or -1 = per-phase kernels
@@ -830,7 +833,6 @@ private:
     sim_status setup_persistent()
     {
         persist = false;
-        corot = sizeof(R) == 4 && (M.model == MAT_FCR || M.model == MAT_ARAP);
         if (!M.opt.persistent) return SIM_OK;
         if (M.opt.scatter == SIM_SCATTER_COLOR) return SIM_OK;         // one kernel per colour: per-phase form
         if (((3 * B.H) >> B.cshift_p) > BP_MAX_CHUNKS) return SIM_OK;   // chunk offsets live in shared memory
@@ -841,13 +843,9 @@ private:
         int gmax = 0;
         for (int sh = 0; sh < N_PSHAPES; ++sh) {
             int per_sm = 0;
-            if (corot && sh > 0) { shape_grid[sh] = 0; continue; }   // the corotated FP32 kernel: shape 0 only
-            if constexpr (sizeof(R) == 4) {
-                if (corot) CK(persist_occupancy_corot(&per_sm));
-                else CK(persist_occupancy_shape<R>(sh, &per_sm));
-            } else {
-                CK(persist_occupancy_shape<R>(sh, &per_sm));
-            }
+            if (sizeof(R) == 4 && corot && sh > 0) { shape_grid[sh] = 0; continue; }   // the corotated FP32 kernel: shape 0 only
+            if (corot) CK((persist_occupancy_shape<R, true>(sh, &per_sm)));
+            else CK((persist_occupancy_shape<R, false>(sh, &per_sm)));
             per_sm = std::min(per_sm, PSHAPE_MINB[sh]);
             shape_grid[sh] = per_sm > 0 ? std::min(per_sm * nsm, MAXG) : 0;
             gmax = std::max(gmax, shape_grid[sh]);
@@ -909,15 +907,29 @@ private:
         D.xh = D.xl = nullptr;
         D.xth = D.xtl = nullptr;
         D.G0 = nullptr;
+        D.tc = nullptr;
+        D.td = nullptr;
         D.tS = nullptr;
+        corot = M.model == MAT_FCR || M.model == MAT_ARAP;
         D.xbh = nullptr;
         D.pg = D.pnext = nullptr;
         if (sizeof(R) == 4) {
             AL(D.xh, nv); AL(D.xl, nv); AL(D.xbh, nv); AL(D.xth, nv); AL(D.xtl, nv);
-            float *g0;
-            AL(g0, 14 * (size_t)nt);
-            D.G0 = g0;
+            if (corot) {
+                float *g0;
+                AL(g0, 14 * (size_t)nt);
+                D.G0 = g0;
+            }
+            float4 *tc;
+            AL(tc, 5 * (size_t)nt);
+            D.tc = tc;
             AL(D.tS, 4 * (size_t)nt);
+            AL(D.tk, (size_t)nt);
+        } else {
+            double4_32a *td;
+            AL(td, 2 * (size_t)nt);
+            D.td = td;
+            AL(D.tk, 2 * (size_t)nt);
         }
         double *mass; AL(mass, nv); D.mass = mass;
         int *fs; AL(fs, nv); D.fix_slot = fs;
@@ -951,7 +963,9 @@ private:
             int *ct; AL(ct, (size_t)nt); D.color_tets = ct;
             AL(c_tet, nt); AL(c_Dm, 9 * (size_t)nt); AL(c_hv, nt);
             if (!M.escale.empty()) AL(c_es, nt);
-            if (sizeof(R) == 4) AL(c_G0, 14 * (size_t)nt);
+            if (D.G0) AL(c_G0, 14 * (size_t)nt);
+            if (sizeof(R) == 4) AL(c_tc, 5 * (size_t)nt);
+            else AL(c_td, 2 * (size_t)nt);
         }
         D.nseg = M.nseg;
         D.vscene = nullptr; D.seg = nullptr; D.sacc = nullptr; D.smax = nullptr; D.cmark = nullptr;
@@ -1089,9 +1103,31 @@ private:
         if ((st = up(B.edge, ed.data(), sizeof(int4) * M.ne))) return st;
         if ((st = up(B.obj, M.obj.data(), sizeof(int) * nv))) return st;
         if (B.excl && (st = up(B.excl, M.excl.data(), sizeof(unsigned long long) * M.excl.size()))) return st;
-        if (D.G0) {
+        // h^2 V M with M = Dm^-1 Dm^-T (00 01 02 11 12 22) and det Dm^-1, in double
+        auto weighted = [&](int e, double m[6], double &dw) {
+            double w[3][3];
+            for (int r = 0; r < 3; ++r)
+                for (int c = 0; c < 3; ++c) w[r][c] = M.Dm[(size_t)(3 * r + c) * nt + e];
+            int q = 0;
+            for (int i = 0; i < 3; ++i)
+                for (int j = i; j < 3; ++j, ++q) m[q] = M.hv[e] * (w[i][0] * w[j][0] + w[i][1] * w[j][1] + w[i][2] * w[j][2]);
+            dw = w[0][0] * (w[1][1] * w[2][2] - w[1][2] * w[2][1]) - w[0][1] * (w[1][0] * w[2][2] - w[1][2] * w[2][0]) +
+                 w[0][2] * (w[1][0] * w[2][1] - w[1][1] * w[2][0]);
+        };
+        if (D.td) {
+            std::vector<double4_32a> td(2 * (size_t)nt);
+            for (int e = 0; e < nt; ++e) {
+                double m[6], dw;
+                weighted(e, m, dw);
+                td[e] = make_double4_32a(m[0], m[1], m[2], m[3]);
+                td[(size_t)nt + e] = make_double4_32a(m[4], m[5], dw, M.hv[e]);
+            }
+            if ((st = up(D.td, td.data(), sizeof(double4_32a) * 2 * (size_t)nt))) return st;
+        }
+        if (D.tc) {
             // rest metric Dm^T Dm and det Dm (six times the rest volume) per tet in double, stored as float-float
             std::vector<float> g0(14 * (size_t)nt);
+            std::vector<float4> tc(5 * (size_t)nt);
             for (int e = 0; e < nt; ++e) {
                 double dm[3][3];
                 for (int c = 0; c < 3; ++c)
@@ -1110,11 +1146,17 @@ private:
                 const float dh = (float)det;
                 g0[(size_t)12 * nt + e] = dh;
                 g0[(size_t)13 * nt + e] = (float)(det - (double)dh);
+                double m[6], dw;
+                weighted(e, m, dw);
+                auto g = [&](int k) { return k < 14 ? g0[(size_t)k * nt + e] : (float)m[k - 14]; };
+                for (int k = 0; k < 5; ++k)
+                    tc[(size_t)k * nt + e] = make_float4(g(4 * k), g(4 * k + 1), g(4 * k + 2), g(4 * k + 3));
             }
-            if ((st = up(D.G0, g0.data(), sizeof(float) * 14 * (size_t)nt))) return st;
+            if (D.G0 && (st = up(D.G0, g0.data(), sizeof(float) * 14 * (size_t)nt))) return st;
+            if ((st = up(D.tc, tc.data(), sizeof(float4) * 5 * (size_t)nt))) return st;
         }
         if (D.colored) {
-            k_color_gather<R><<<(nt + 255) / 256, 256, 0, s>>>(D, c_tet, c_Dm, c_hv, c_es, c_G0);
+            k_color_gather<R><<<(nt + 255) / 256, 256, 0, s>>>(D, c_tet, c_Dm, c_hv, c_es, c_G0, c_tc, c_td);
             CK(cudaGetLastError());
         }
         refresh_ff();
@@ -1238,7 +1280,7 @@ private:
         k_update<R><<<nvb, VB, 0, s>>>(D, par);
     }
     void launch_finish() { k_finish<R><<<nvb, VB, 0, s>>>(D); }
-    // the element kernels: the FP32 corotated densities run their own instantiations
+    // the element kernels: the corotated densities run their own instantiations
     void launch_grad_kernel(int par)
     {
         // colouring scatter: the candidates alone (no tet blocks), then one kernel per colour
@@ -1247,7 +1289,7 @@ private:
         else k_grad<R><<<nt_blocks + ncb, EB, 0, s>>>(D, par, nt_blocks);
         if (D.colored) {
             Dev<R> Dc = D;
-            Dc.tet = c_tet; Dc.Dm = c_Dm; Dc.hv = c_hv; Dc.escale = c_es; Dc.G0 = c_G0;
+            Dc.tet = c_tet; Dc.Dm = c_Dm; Dc.hv = c_hv; Dc.escale = c_es; Dc.G0 = c_G0; Dc.tc = c_tc; Dc.td = c_td;
             for (size_t c = 0; c + 1 < M.color_off.size(); ++c) {
                 const int t0 = M.color_off[c], n = M.color_off[c + 1] - t0;
                 if (corot) k_grad_color<R, true><<<(n + EB - 1) / EB, EB, 0, s>>>(D, Dc, par, t0, n);
@@ -1277,10 +1319,7 @@ private:
         A.part = ppart;
         A.stamps = stamps; A.stamp_kind = kinds; A.max_stamps = max_stamps;
         A.arrive = arrive; A.depart = depart; A.bar_kind = bar_kind; A.max_bar = max_bar;
-        if constexpr (sizeof(R) == 4) {
-            if (corot) return persist_launch_corot(D, B, A, pgrid, s);
-        }
-        return persist_launch_shape<R>(shape, D, B, A, pgrid, s);
+        return corot ? persist_launch_shape<R, true>(shape, D, B, A, pgrid, s) : persist_launch_shape<R, false>(shape, D, B, A, pgrid, s);
     }
     sim_status launch_step()
     {
