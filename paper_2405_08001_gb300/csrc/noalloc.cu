@@ -29,8 +29,46 @@ std::mutex g_setup_mutex;
 NoAllocScratch *g_scratch_ptr[NA_MAX_DEVICES] = {};
 thread_local std::string g_noalloc_err;
 
+struct Mat3 { double m[3][3]; };   // columns are edge vectors
+__device__ inline Mat3 edges(const double *x, const int v[4])
+{
+    Mat3 d;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const double x0 = x[3 * v[0] + a];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) d.m[a][c] = x[3 * v[c + 1] + a] - x0;
+    }
+    return d;
+}
+// columns d1 x d2, d2 x d0, d0 x d1
+__device__ inline Mat3 cofactors(const Mat3 &d)
+{
+    Mat3 c;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        const int p = (b + 1) % 3, q = (b + 2) % 3;
+        c.m[0][b] = d.m[1][p] * d.m[2][q] - d.m[2][p] * d.m[1][q];
+        c.m[1][b] = d.m[2][p] * d.m[0][q] - d.m[0][p] * d.m[2][q];
+        c.m[2][b] = d.m[0][p] * d.m[1][q] - d.m[1][p] * d.m[0][q];
+    }
+    return c;
+}
+__device__ inline double inner(const Mat3 &a, const Mat3 &b)
+{
+    double s = 0.0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) s += a.m[i][j] * b.m[i][j];
+    return s;
+}
+
 // p^T M p + h^2 sum_e V_e [mu |dF|^2 + Psi_33 (cof F : dF)^2 + Psi_3 d2det(F)[dF, dF]] in double precision, one
-// thread per tet (and per vertex for the inertia term); D_m^-1 and V_e are formed from the rest positions.
+// thread per tet (and per vertex for the inertia term).  With the edge vectors of the rest, current and direction
+// values Dm, Ds, Dp (columns): J = det Ds / det Dm, cof F : dF = cof(Ds) : Dp / det Dm, d2det(F)[dF, dF] = 2 cof(Dp) : Ds /
+// det Dm and dF = Dp cof(Dm)^T / det Dm, so that neither D_m^-1 nor F is formed.  Bound by FP64 issue (1.65 lanes per
+// clock and SM): about 205 operations a tet with two divisions, where the form on F took about 400 with nine.
 __global__ void __launch_bounds__(NA_THREADS) k_pHp_noalloc(NoAllocScratch *scr, int nv, int nt, const double *x,
                                                              const double *p, const double *X, const int *tets,
                                                              const double *mass, double mu, double lam, double h2,
@@ -45,55 +83,25 @@ __global__ void __launch_bounds__(NA_THREADS) k_pHp_noalloc(NoAllocScratch *scr,
     }
     if (i < nt) {
         const int v[4] = {tets[4 * i], tets[4 * i + 1], tets[4 * i + 2], tets[4 * i + 3]};
-        double A[3][3], Ds[3][3], Dp[3][3];
-        for (int c = 0; c < 3; ++c)
-            for (int a = 0; a < 3; ++a) {
-                A[a][c] = X[3 * v[c + 1] + a] - X[3 * v[0] + a];
-                Ds[a][c] = x[3 * v[c + 1] + a] - x[3 * v[0] + a];
-                Dp[a][c] = p[3 * v[c + 1] + a] - p[3 * v[0] + a];
-            }
-        const double det = A[0][0] * (A[1][1] * A[2][2] - A[1][2] * A[2][1]) - A[0][1] * (A[1][0] * A[2][2] - A[1][2] * A[2][0]) +
-                           A[0][2] * (A[1][0] * A[2][1] - A[1][1] * A[2][0]);
-        double W[3][3];
-        W[0][0] = (A[1][1] * A[2][2] - A[1][2] * A[2][1]) / det;
-        W[0][1] = (A[0][2] * A[2][1] - A[0][1] * A[2][2]) / det;
-        W[0][2] = (A[0][1] * A[1][2] - A[0][2] * A[1][1]) / det;
-        W[1][0] = (A[1][2] * A[2][0] - A[1][0] * A[2][2]) / det;
-        W[1][1] = (A[0][0] * A[2][2] - A[0][2] * A[2][0]) / det;
-        W[1][2] = (A[0][2] * A[1][0] - A[0][0] * A[1][2]) / det;
-        W[2][0] = (A[1][0] * A[2][1] - A[1][1] * A[2][0]) / det;
-        W[2][1] = (A[0][1] * A[2][0] - A[0][0] * A[2][1]) / det;
-        W[2][2] = (A[0][0] * A[1][1] - A[0][1] * A[1][0]) / det;
-        double F[3][3], dF[3][3];
-        for (int a = 0; a < 3; ++a)
-            for (int b = 0; b < 3; ++b) {
-                F[a][b] = Ds[a][0] * W[0][b] + Ds[a][1] * W[1][b] + Ds[a][2] * W[2][b];
-                dF[a][b] = Dp[a][0] * W[0][b] + Dp[a][1] * W[1][b] + Dp[a][2] * W[2][b];
-            }
-        // cofactor columns f1 x f2, f2 x f0, f0 x f1 of F and of the mixed terms
-        double cf[3][3];
-        for (int b = 0; b < 3; ++b) {
-            const int b1 = (b + 1) % 3, b2 = (b + 2) % 3;
-            cf[0][b] = F[1][b1] * F[2][b2] - F[2][b1] * F[1][b2];
-            cf[1][b] = F[2][b1] * F[0][b2] - F[0][b1] * F[2][b2];
-            cf[2][b] = F[0][b1] * F[1][b2] - F[1][b1] * F[0][b2];
-        }
-        const double J = F[0][0] * cf[0][0] + F[1][0] * cf[1][0] + F[2][0] * cf[2][0];
-        if (J > 0.0 && det > 0.0) {
+        const Mat3 A = edges(X, v), Ds = edges(x, v), Dp = edges(p, v);
+        const Mat3 ca = cofactors(A), cs = cofactors(Ds);
+        const double det = A.m[0][0] * ca.m[0][0] + A.m[1][0] * ca.m[1][0] + A.m[2][0] * ca.m[2][0];
+        const double ds = Ds.m[0][0] * cs.m[0][0] + Ds.m[1][0] * cs.m[1][0] + Ds.m[2][0] * cs.m[2][0];
+        if (ds > 0.0 && det > 0.0) {
+            const double idet = 1.0 / det, J = ds * idet, iJ = det / ds;
             const double L = log(J);
-            const double Psi3 = (lam * L - mu) / J, Psi33 = (mu + lam * (1.0 - L)) / (J * J);
-            double n2 = 0.0, g3 = 0.0;
+            const double Psi3 = (lam * L - mu) * iJ, Psi33 = (mu + lam * (1.0 - L)) * iJ * iJ;
+            double n2 = 0.0;
+#pragma unroll
             for (int a = 0; a < 3; ++a)
-                for (int b = 0; b < 3; ++b) { n2 += dF[a][b] * dF[a][b]; g3 += cf[a][b] * dF[a][b]; }
-            // d2det(F)[dF, dF] = 2 (df0 . (df1 x f2) + df0 . (f1 x df2) + f0 . (df1 x df2)), columns
-            auto col = [](const double M[3][3], int b, double o[3]) { o[0] = M[0][b]; o[1] = M[1][b]; o[2] = M[2][b]; };
-            auto tri = [](const double a[3], const double b[3], const double c[3]) {
-                return a[0] * (b[1] * c[2] - b[2] * c[1]) + a[1] * (b[2] * c[0] - b[0] * c[2]) + a[2] * (b[0] * c[1] - b[1] * c[0]);
-            };
-            double f0[3], f1[3], f2[3], d0[3], d1[3], d2[3];
-            col(F, 0, f0); col(F, 1, f1); col(F, 2, f2); col(dF, 0, d0); col(dF, 1, d1); col(dF, 2, d2);
-            const double h3 = 2.0 * (tri(d0, d1, f2) + tri(d0, f1, d2) + tri(f0, d1, d2));
-            s[0] += h2 * (det / 6.0) * (mu * n2 + Psi33 * g3 * g3 + Psi3 * h3);
+#pragma unroll
+                for (int b = 0; b < 3; ++b) {
+                    const double f = Dp.m[a][0] * ca.m[b][0] + Dp.m[a][1] * ca.m[b][1] + Dp.m[a][2] * ca.m[b][2];
+                    n2 += f * f;
+                }
+            const double g3 = inner(cs, Dp) * idet;
+            const double h3 = 2.0 * inner(cofactors(Dp), Ds) * idet;
+            s[0] += h2 * (det * (1.0 / 6.0)) * (mu * (n2 * idet * idet) + Psi33 * (g3 * g3) + Psi3 * h3);
         } else {
             s[0] = nan("");     // an inverted current tet, or a rest tet of non-positive volume
         }
