@@ -135,7 +135,9 @@ typedef struct {
                              above (a tet or pair spanning groups adds to each group's p^T H p with the other groups'
                              entries of p zero).  Group g = 2 object + (1 for the collision part); a group without
                              vertices takes no step.  Works without scene_of_vert (one object, two groups). */
-    int32_t block_shape;  /* block shape of the persistent form: 0 (default) = 256 threads x 2 blocks per SM,
+    int32_t block_shape;  /* block shape of the persistent form: 0 (default) = 256 threads x 2 blocks per SM, or for a
+                             small mesh (8,192 tets in the FP32 form, 4,096 in FP64; not with SIM_SCATTER_BLOCK) one
+                             thread-block cluster of 16 blocks of 256 threads;
                              1 = 512 x 1, 2 = 256 x 3, 3 = 256 x 1, 4 = 384 x 1 (the compiler fits the registers
                              per thread to the shape: 128, 128, 85, 255, 168); -1 = autotuned: from the second time
                              step on, each shape runs two time steps (interleaved), timed on the GPU (those steps
@@ -161,7 +163,7 @@ typedef struct {
     int32_t n_near_fp64;   /* FP32 form: pair evaluations of the last step (or of the last sim_eval_* call) whose
                               distance fell below 1e-3 dhat, where the barrier terms are evaluated in double */
     int32_t block_threads; /* persistent form: threads per block and blocks per SM of the shape in use (0 in the */
-    int32_t blocks_per_sm; /*   per-phase form) */
+    int32_t blocks_per_sm; /*   per-phase form; 256 and 1 as one cluster) */
     int32_t n_colors;      /* scatter SIM_SCATTER_COLOR: colours of the tet colouring (gradient kernels per
                               iteration); 0 with the other scatters */
 } sim_stats;

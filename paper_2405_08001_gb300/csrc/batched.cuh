@@ -119,8 +119,8 @@ template <typename R> __device__ inline void seg_reset(const Dev<R> &D)
 // Beta, direction + p^T H p, and update phases of iteration k for nseg > 1 scenes (three grid barriers, as in the
 // single-scene form).  sbuf holds the scenes' beta and alpha (2 x MAX_SCENES doubles).  Returns 1 when some vertex
 // has moved far enough since the candidate build to need a new one.
-template <typename R, int PB, bool CO>
-__device__ inline int batched_tail(const Dev<R> &D, Ctrl *c, PShared<R, PB> &sh, unsigned char *sbuf, Bar &br,
+template <typename R, int PB, bool CO, bool CL>
+__device__ inline int batched_tail(const Dev<R> &D, Ctrl *c, PShared<R, PB, CL> &sh, unsigned char *sbuf, Bar &br,
                                    Stamper &st, RedBufs &rb, int k, int par, int &sred, double disp_lim)
 {
     typedef typename V4<R>::T R4;
@@ -141,7 +141,7 @@ __device__ inline int batched_tail(const Dev<R> &D, Ctrl *c, PShared<R, PB> &sh,
             const int4 v = __ldcg(&D.act[kk].v);
             D.cmark[v.x] = 1; D.cmark[v.y] = 1; D.cmark[v.z] = 1; D.cmark[v.w] = 1;
         }
-        grid_barrier(br, c);
+        grid_barrier<CL>(br, c);
     }
 
     // ------------------------------------------------------------ beta (per scene) and P g
@@ -172,7 +172,7 @@ __device__ inline int batched_tail(const Dev<R> &D, Ctrl *c, PShared<R, PB> &sh,
             }
             seg_warp_sum<R, 5>(a5, key, acc, 0);
         }
-        grid_barrier(br, c);
+        grid_barrier<CL>(br, c);
         if (threadIdx.x == 0) sh.fi = (volatile const int &)c->n_active;
         for (int s = threadIdx.x; s < ns; s += blockDim.x) {
             double t[5];
@@ -291,7 +291,7 @@ __device__ inline int batched_tail(const Dev<R> &D, Ctrl *c, PShared<R, PB> &sh,
                                               ks[2] == u[j] ? pv[2] : z, ks[3] == u[j] ? pv[3] : z));
             }
         }
-        grid_barrier(br, c);
+        grid_barrier<CL>(br, c);
         if (threadIdx.x == 0) sh.fe = (volatile const uint32_t &)c->err;
         __syncthreads();
         const uint32_t err = sh.fe;
@@ -360,7 +360,7 @@ __device__ inline int batched_tail(const Dev<R> &D, Ctrl *c, PShared<R, PB> &sh,
         D.p[i] = P;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) c->n_active = 0;
-    const R m = grid_max<R, PB>(md, rb.max_region<PT, R>(), sh, br, c);
+    const R m = grid_max<R, PB, CL>(md, rb.max_region<PT, R>(), sh, br, c);
     st.mark(11);  // K_UPDATE
     return (double)m >= disp_lim * disp_lim ? 1 : 0;
 }

@@ -1,0 +1,6 @@
+// The cluster form of the persistent time step of the corotated densities (persist_shapes.cuh), in a translation unit of its own.
+#include "persist_shapes.cuh"
+
+namespace pncg {
+PNCG_CLUSTER_DEF(double, true)
+}

@@ -14,12 +14,19 @@ constexpr int N_PSHAPES = 5;
 constexpr int PSHAPE_PB[N_PSHAPES] = {256, 512, 256, 256, 384};
 constexpr int PSHAPE_MINB[N_PSHAPES] = {2, 1, 3, 1, 1};
 
+// The cluster form of small meshes: CLUSTER_PB threads per block, all blocks of the launch in one cluster.
+constexpr int CLUSTER_PB = 256;
+
 // Launch of shape S (cooperative, grid blocks, PSHAPE_PB[S] threads) and its occupancy (blocks per SM).  The corotated
 // densities (FCR, ARAP; CO) run instantiations of their own, so that the kernels of the others carry none of their
 // code and registers; the FP32 form has them in the default shape only.
 template <typename R, int S, bool CO> cudaError_t persist_launch(const Dev<R> &D, const BPDev &B, const PersistArgs &A,
                                                                  int grid, cudaStream_t s);
 template <typename R, int S, bool CO> cudaError_t persist_occupancy(int *per_sm);
+// The same of the cluster form; *blocks receives the blocks of the largest cluster (16 or 8) the device can hold, 0 = none.
+template <typename R, bool CO> cudaError_t cluster_launch(const Dev<R> &D, const BPDev &B, const PersistArgs &A, int grid,
+                                                          cudaStream_t s);
+template <typename R, bool CO> cudaError_t cluster_blocks(int *blocks);
 
 #define PNCG_PERSIST_DECL(R, S, CO)                                                                             \
     template <> cudaError_t persist_launch<R, S, CO>(const Dev<R> &, const BPDev &, const PersistArgs &, int,   \
@@ -32,6 +39,12 @@ PNCG_PERSIST_DECL(double, 3, false) PNCG_PERSIST_DECL(double, 4, false)
 PNCG_PERSIST_DECL(double, 0, true) PNCG_PERSIST_DECL(double, 1, true) PNCG_PERSIST_DECL(double, 2, true)
 PNCG_PERSIST_DECL(double, 3, true) PNCG_PERSIST_DECL(double, 4, true)
 #undef PNCG_PERSIST_DECL
+#define PNCG_CLUSTER_DECL(R, CO)                                                                                \
+    template <> cudaError_t cluster_launch<R, CO>(const Dev<R> &, const BPDev &, const PersistArgs &, int,      \
+                                                  cudaStream_t);                                               \
+    template <> cudaError_t cluster_blocks<R, CO>(int *);
+PNCG_CLUSTER_DECL(float, false) PNCG_CLUSTER_DECL(float, true) PNCG_CLUSTER_DECL(double, false) PNCG_CLUSTER_DECL(double, true)
+#undef PNCG_CLUSTER_DECL
 
 // the definitions, one shape per translation unit
 #define PNCG_PERSIST_DEF(R, S, CO)                                                                              \
@@ -50,6 +63,49 @@ PNCG_PERSIST_DECL(double, 3, true) PNCG_PERSIST_DECL(double, 4, true)
         return cudaOccupancyMaxActiveBlocksPerMultiprocessor(                                                  \
             per_sm, k_persistent<R, PSHAPE_PB[S], PSHAPE_MINB[S], CO>, PSHAPE_PB[S], 0);                        \
     }
+#define PNCG_CLUSTER_DEF(R, CO)                                                                                 \
+    template <> cudaError_t cluster_launch<R, CO>(const Dev<R> &D, const BPDev &B, const PersistArgs &A,        \
+                                                  int grid, cudaStream_t s)                                    \
+    {                                                                                                          \
+        cudaLaunchAttribute at;                                                                                \
+        const cudaLaunchConfig_t cfg = cluster_config(grid, at, s);                                            \
+        return cudaLaunchKernelEx(&cfg, k_persistent<R, CLUSTER_PB, 1, CO, true>, D, B, A);                     \
+    }                                                                                                          \
+    template <> cudaError_t cluster_blocks<R, CO>(int *blocks)                                                 \
+    {                                                                                                          \
+        return largest_cluster((const void *)k_persistent<R, CLUSTER_PB, 1, CO, true>, blocks);                 \
+    }
+
+// one cluster of `blocks` blocks (the attribute must outlive the configuration)
+inline cudaLaunchConfig_t cluster_config(int blocks, cudaLaunchAttribute &at, cudaStream_t s)
+{
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = blocks;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(CLUSTER_PB);
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+inline cudaError_t largest_cluster(const void *kernel, int *blocks)
+{
+    *blocks = 0;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        cudaGetLastError();
+        return cudaSuccess;
+    }
+    for (int c = CLUSTER_MAX; c >= 8 && *blocks == 0; c /= 2) {
+        cudaLaunchAttribute at;
+        const cudaLaunchConfig_t cfg = cluster_config(c, at, nullptr);
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) cudaGetLastError();
+        else if (n > 0) *blocks = c;
+    }
+    return cudaSuccess;
+}
 
 // run-time dispatch over the shapes
 template <typename R, bool CO>

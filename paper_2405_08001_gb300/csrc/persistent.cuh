@@ -15,6 +15,10 @@
 //
 // Barrier waits are bounded: a block that waits longer than the limit sets ERR_TIMEOUT and carries on; later
 // barriers do not wait once the bit is set, so the launch always terminates and the host reports SIM_ERR_TIMEOUT.
+//
+// Small meshes run it as one thread-block cluster (the template parameter CL, at most CLUSTER_MAX blocks): the
+// barrier is the hardware's cluster barrier (0.23 us for 16 blocks of 512 threads where the counter barrier takes
+// 2.1 us on 304 blocks and 1.5 us on 16) and the reductions' partials go straight into the other blocks' shared memory.
 #pragma once
 
 #include "broadphase.cuh"
@@ -26,6 +30,7 @@ namespace pncg {
 // the library instantiates a few shapes (persist_shapes) and can pick one per workload by timing (the block-shape
 // autotuner, sim_options.block_shape = -1).
 constexpr int MAXG = 1024;   // most blocks a persistent launch may have (the host caps its grid at this)
+constexpr int CLUSTER_MAX = 16;   // blocks of the cluster form (the largest non-portable cluster)
 constexpr unsigned long long BARRIER_LIMIT_NS = 4000000000ull;   // a barrier wait gives up after 4 s
 
 // Arrival counter of the grid barriers, zeroed before each launch.  Every block passes the same sequence of
@@ -50,6 +55,19 @@ __device__ inline void fence_acq_rel() { asm volatile("fence.acq_rel.gpu;" ::: "
 __device__ inline void red_release_add(unsigned int *p, unsigned int v)
 {
     asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+// every thread of the cluster; its writes before are seen by the others' reads after
+__device__ inline void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+// writes v to p's place in the shared memory of the cluster's block `rank` (p points to this block's own)
+__device__ inline void st_peer(void *p, int rank, unsigned long long v)
+{
+    unsigned int a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((unsigned int)__cvta_generic_to_shared(p)), "r"(rank));
+    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
 }
 __device__ inline unsigned long long global_ns()
 {
@@ -81,8 +99,22 @@ __device__ inline bool wait_count(const unsigned int *count, unsigned int target
 // cumulative fence followed by the add, so no separate fence is needed; the add needs no round trip).  The lead
 // thread polls the counter with relaxed loads and, once it has seen every arrival, orders the block's later reads
 // after the other blocks' writes with one acquire fence, before the CTA barrier hands on to the block.
-__device__ inline void grid_barrier(Bar &br, Ctrl *c)
+// CL: the grid is one cluster, and the barrier the hardware's.
+template <bool CL> __device__ inline void grid_barrier(Bar &br, Ctrl *c)
 {
+    if constexpr (CL) {
+        br.n += 1;
+        const bool rec = br.arrive && threadIdx.x == 0 && (int)br.n <= br.max;
+        const size_t at = (size_t)(br.n - 1) * gridDim.x + blockIdx.x;
+        if (br.arrive) __syncthreads();   // the block arrives with its last thread
+        if (rec) br.arrive[at] = global_ns();
+        cluster_sync();
+        if (rec) {
+            br.depart[at] = global_ns();
+            if (blockIdx.x == 0) br.kind[br.n - 1] = br.phase;
+        }
+        return;
+    }
     __syncthreads();
     br.n += 1;
     if (threadIdx.x == 0) {
@@ -196,9 +228,11 @@ __device__ inline Share share_of(int n)
     return {b0, min(n, b0 + per)};
 }
 
-template <typename R, int PB> struct PShared {
+template <typename R, int PB, bool CL> struct PShared {
     Acc<R> t[NQ][PB];
     R mx[PB];
+    // cluster form: every block's partials; consecutive reductions alternate between the halves (RedBufs)
+    unsigned long long cp[2][NQ + 1][CL ? CLUSTER_MAX : 1];
     double res[NQ + 1];   // reduced results: sums, then the max
     double o[4];          // scalars computed by thread 0 and broadcast to the block
     int oi[2];
@@ -208,9 +242,36 @@ template <typename R, int PB> struct PShared {
 
 // Block part of a grid reduction: N sums (and, with MX, a max of non-negative values) of the block's threads,
 // written as the block's partials (quantity q at part[q * gridDim.x + block], the max in slot N).
-template <typename R, int PB, int N, bool MX>
-__device__ inline void block_publish(Acc<R> (&a)[N], R mx, typename PartT<R>::T *part, PShared<R, PB> &sh)
+__device__ inline unsigned long long acc_bits(const Acc<float> &a)
 {
+    return (unsigned long long)__float_as_uint(a.l) << 32 | __float_as_uint(a.h);
+}
+__device__ inline unsigned long long acc_bits(const Acc<double> &a) { return (unsigned long long)__double_as_longlong(a.v); }
+__device__ inline void acc_from(unsigned long long b, Acc<float> &a)
+{
+    a.h = __uint_as_float((unsigned int)b);
+    a.l = __uint_as_float((unsigned int)(b >> 32));
+}
+__device__ inline void acc_from(unsigned long long b, Acc<double> &a) { a.v = __longlong_as_double((long long)b); }
+
+// a partial of the block (valid in lane 0 of the calling warp) to its slot q of every block of the cluster
+template <typename R, int PB, bool CL> __device__ inline void peer_publish(const Acc<R> &a, int q, int half, PShared<R, PB, CL> &sh)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned long long v = __shfl_sync(0xffffffffu, acc_bits(a), 0);
+    if (lane < (int)gridDim.x) st_peer(&sh.cp[half][q][blockIdx.x], lane, v);
+}
+
+// Destination of a reduction's partials: in global memory, or (cluster form) a half of every block's sh.cp.
+template <typename P> struct PartDst {
+    P *g;
+    int half;
+};
+
+template <typename R, int PB, bool CL, int N, bool MX>
+__device__ inline void block_publish(Acc<R> (&a)[N], R mx, const PartDst<typename PartT<R>::T> &dst, PShared<R, PB, CL> &sh)
+{
+    typename PartT<R>::T *part = dst.g;
     static_assert(N <= NQ && N + (MX ? 1 : 0) <= PB / 32, "one warp per quantity");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -222,13 +283,17 @@ __device__ inline void block_publish(Acc<R> (&a)[N], R mx, typename PartT<R>::T 
 #pragma unroll
         for (int j = 1; j < PB / 32; ++j) s.add(sh.t[warp][lane + 32 * j]);
         for (int o = 16; o > 0; o >>= 1) s.add(s.shfl_down(o));
-        if (lane == 0) put_part(part + warp * gridDim.x + blockIdx.x, s);
+        if constexpr (CL) peer_publish<R, PB, CL>(s, warp, dst.half, sh);
+        else if (lane == 0) put_part(part + warp * gridDim.x + blockIdx.x, s);
     } else if (MX && warp == N) {
         R m = sh.mx[lane];
 #pragma unroll
         for (int j = 1; j < PB / 32; ++j) m = fmax(m, sh.mx[lane + 32 * j]);
         for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
-        if (lane == 0) { Acc<R> b; b.add(m); put_part(part + N * gridDim.x + blockIdx.x, b); }
+        Acc<R> b;
+        b.add(m);
+        if constexpr (CL) peer_publish<R, PB, CL>(b, N, dst.half, sh);
+        else if (lane == 0) put_part(part + N * gridDim.x + blockIdx.x, b);
     }
 }
 
@@ -236,11 +301,33 @@ __device__ inline void block_publish(Acc<R> (&a)[N], R mx, typename PartT<R>::T 
 // L2), then the block reduces them transposed like block_publish (warp q sums quantity q, warp N takes the max, in
 // block order within each lane's stride); the results land in sh.res (sums in double), and thread 0 reads the
 // fetched scalars.  Every block computes bitwise the same results.  Ends with a CTA barrier.
-template <typename R, int PB, int N, bool MX>
-__device__ inline void grid_collect(const typename PartT<R>::T *part, PShared<R, PB> &sh, const Fetch *f)
+template <typename R, int PB, bool CL, int N, bool MX>
+__device__ inline void grid_collect(const PartDst<typename PartT<R>::T> &dst, PShared<R, PB, CL> &sh, const Fetch *f)
 {
+    const typename PartT<R>::T *part = dst.g;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int G = gridDim.x;
+    if constexpr (CL) {
+        // the blocks' partials are in this block's shared memory: warp q takes quantity q, one block per lane
+        if (f && threadIdx.x == 0) {
+            if (f->pi) sh.fi = (volatile const int &)*f->pi;
+            if (f->pe) sh.fe = (volatile const uint32_t &)*f->pe;
+        }
+        if (warp < N + (MX ? 1 : 0)) {
+            Acc<R> s;
+            if (lane < G) acc_from(sh.cp[dst.half][warp][lane], s);
+            if (warp < N) {
+                for (int o = CLUSTER_MAX / 2; o > 0; o >>= 1) s.add(s.shfl_down(o));
+                if (lane == 0) sh.res[warp] = s.value();
+            } else {
+                R m = s.head();
+                for (int o = CLUSTER_MAX / 2; o > 0; o >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
+                if (lane == 0) sh.res[N] = (double)m;
+            }
+        }
+        __syncthreads();
+        return;
+    }
     if (f && threadIdx.x == 0) {
         if (f->pi) sh.fi = (volatile const int &)*f->pi;
         if (f->pe) sh.fe = (volatile const uint32_t &)*f->pe;
@@ -282,20 +369,21 @@ __device__ inline void grid_collect(const typename PartT<R>::T *part, PShared<R,
 }
 
 // Grid-wide sums of N accumulators (and a max): block part, barrier, collection into sh.res.
-template <typename R, int PB, int N, bool MX>
-__device__ inline void grid_reduce(Acc<R> (&a)[N], R mx, typename PartT<R>::T *part, PShared<R, PB> &sh, Bar &br,
-                                   Ctrl *c, const Fetch *f = nullptr)
+template <typename R, int PB, bool CL, int N, bool MX>
+__device__ inline void grid_reduce(Acc<R> (&a)[N], R mx, const PartDst<typename PartT<R>::T> &part, PShared<R, PB, CL> &sh,
+                                   Bar &br, Ctrl *c, const Fetch *f = nullptr)
 {
-    block_publish<R, PB, N, MX>(a, mx, part, sh);
-    grid_barrier(br, c);
-    grid_collect<R, PB, N, MX>(part, sh, f);
+    block_publish<R, PB, CL, N, MX>(a, mx, part, sh);
+    grid_barrier<CL>(br, c);
+    grid_collect<R, PB, CL, N, MX>(part, sh, f);
 }
 
 // Grid-wide max of non-negative values of the element type (exact); one grid barrier.  `part` holds gridDim.x
 // values of type R.  Returned in every thread.
-template <typename R, int PB>
-__device__ inline R grid_max(R v, R *part, PShared<R, PB> &sh, Bar &br, Ctrl *c)
+template <typename R, int PB, bool CL>
+__device__ inline R grid_max(R v, const PartDst<R> &dst, PShared<R, PB, CL> &sh, Bar &br, Ctrl *c)
 {
+    R *part = dst.g;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     sh.mx[threadIdx.x] = v;
     __syncthreads();
@@ -304,9 +392,23 @@ __device__ inline R grid_max(R v, R *part, PShared<R, PB> &sh, Bar &br, Ctrl *c)
 #pragma unroll
         for (int j = 1; j < PB / 32; ++j) m = fmax(m, sh.mx[lane + 32 * j]);
         for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
-        if (lane == 0) part[blockIdx.x] = m;
+        if constexpr (CL) {
+            Acc<R> b;
+            b.add(m);
+            peer_publish<R, PB, CL>(b, NQ, dst.half, sh);
+        } else if (lane == 0) {
+            part[blockIdx.x] = m;
+        }
     }
-    grid_barrier(br, c);
+    grid_barrier<CL>(br, c);
+    if constexpr (CL) {
+        Acc<R> b;
+        if (lane < (int)gridDim.x) acc_from(sh.cp[dst.half][NQ][lane], b);
+        R m = b.head();
+#pragma unroll
+        for (int o = CLUSTER_MAX / 2; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+        return __shfl_sync(0xffffffffu, m, 0);
+    }
     R m = R(0);
 #pragma unroll
     for (int j = 0; j < (MAXG + PB - 1) / PB; ++j) {
@@ -368,8 +470,16 @@ struct RedBufs {
     void *base;
     int n;
     int sum_i = 0, max_i = 0;
-    template <typename PT> __device__ inline PT *sum_region() { return (PT *)base + (size_t)(sum_i++ & 1) * 8 * n; }
-    template <typename PT, typename R> __device__ inline R *max_region() { return (R *)((PT *)base + (size_t)16 * n) + (size_t)(max_i++ & 1) * n; }
+    template <typename PT> __device__ inline PartDst<PT> sum_region()
+    {
+        const int h = sum_i++ & 1;
+        return {(PT *)base + (size_t)h * 8 * n, h};
+    }
+    template <typename PT, typename R> __device__ inline PartDst<R> max_region()
+    {
+        const int h = max_i++ & 1;
+        return {(R *)((PT *)base + (size_t)16 * n) + (size_t)h * n, h};
+    }
 };
 
 // the displacement reference of a vertex (its position at the last candidate build): the float copy in the FP32
@@ -398,14 +508,14 @@ namespace pncg {
 
 // ------------------------------------------------------------------------------------------------ the kernel
 
-template <typename R, int PB, int MINB, bool CO = false>
+template <typename R, int PB, int MINB, bool CO = false, bool CL = false>
 __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, PersistArgs A)
 {
     typedef typename V4<R>::T R4;
     typedef typename PartT<R>::T PT;
     static_assert(PB % 32 == 0 && PB / 32 >= NQ + 1, "one warp per reduced quantity");
-    __shared__ __align__(16) unsigned char sh_raw[sizeof(PShared<R, PB>)];   // raw storage: Acc has initialisers
-    PShared<R, PB> &sh = *reinterpret_cast<PShared<R, PB> *>(sh_raw);
+    __shared__ __align__(16) unsigned char sh_raw[sizeof(PShared<R, PB, CL>)];   // raw storage: Acc has initialisers
+    PShared<R, PB, CL> &sh = *reinterpret_cast<PShared<R, PB, CL> *>(sh_raw);
     __shared__ int sh_i;
     // one buffer for several phases: the gradient's block-scatter accumulators, the candidate build's chunk
     // offsets, then the warps' query batches
@@ -437,7 +547,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
     const double disp_lim = 0.5 * D.pad_r * (1.0 - 1e-4);
     Stamper st{A.stamps, A.stamp_kind, A.max_stamps};
     if (lead) { c->ticket[TK_PAIRS] = 0u; c->ticket[TK_PAIRS1] = 0u; }
-    grid_barrier(br, c);
+    grid_barrier<CL>(br, c);
     st.mark(-1);
 
     // ---------------------------------------------------------------- a0: prediction and iteration-0 init
@@ -467,7 +577,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
                 md = fmax(md, (R)disp2<R>(D, i, X));
             }
         }
-        const R m = grid_max<R, PB>(md, rb.max_region<PT, R>(), sh, br, c);
+        const R m = grid_max<R, PB, CL>(md, rb.max_region<PT, R>(), sh, br, c);
         if (!skip_step && (double)m >= disp_lim * disp_lim) rebuild = 1;
         gPg_prev = 0.0;
         dE0 = 0.0;
@@ -477,7 +587,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
             c->n_active = 0; c->dE0 = 0.0; c->gPg_prev = 0.0;
         }
         if (D.nseg > 1) seg_reset<R>(D);
-        grid_barrier(br, c);
+        grid_barrier<CL>(br, c);
         st.mark(0);   // K_PREDICT
     }
 
@@ -505,7 +615,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
                 B.bhi[j] = hi;
                 ext_max = fmaxf(ext_max, fmaxf(__fsub_ru(hi.x, lo.x), fmaxf(__fsub_ru(hi.y, lo.y), __fsub_ru(hi.z, lo.z))));
             }
-            const float ext = (float)grid_max<R, PB>(R(ext_max), rb.max_region<PT, R>(), sh, br, c);
+            const float ext = (float)grid_max<R, PB, CL>(R(ext_max), rb.max_region<PT, R>(), sh, br, c);
             if (lead) c->cell_bits = __float_as_uint(ext);
             st.mark(1);   // K_BP_BOXES
             const CellGrid cg = grid_of(ext * 1.0001f);   // as cell_size() forms it from cell_bits
@@ -519,7 +629,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
                 if (point_cell(B, j, cg, v, X, cc)) atomicAdd(&B.cnt[point_bucket(B, cc[0], cc[1], cc[2])], 1u);
                 else atomicOr(&c->err, ERR_RANGE);
             }
-            grid_barrier(br, c);
+            grid_barrier<CL>(br, c);
             st.mark(2);   // K_BP_COUNT
             // exclusive scans of the chunks of 2^cshift buckets, one warp per chunk, four buckets per lane; the work
             // units of the triangle and edge buckets are listed on the way
@@ -551,7 +661,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
                     if (lane == 0) B.ctot[ch] = run;
                 }
             }
-            grid_barrier(br, c);
+            grid_barrier<CL>(br, c);
             st.mark(3);   // K_BP_SCAN
             // every block scans the chunk totals into shared memory; the buckets' global offsets go to goff for
             // the queries, and the entries to their slots
@@ -591,7 +701,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
                 for (int j = ps.b0 + (int)threadIdx.x; j < ps.b1; j += PB) fill_prim(B, j, cg, slot_of);
                 for (int j = ss.b0 + (int)threadIdx.x; j < ss.b1; j += PB) fill_point(B, j, cg, slot_of);
             }
-            grid_barrier(br, c);
+            grid_barrier<CL>(br, c);
             st.mark(4);   // K_BP_FILL
             // queries: the listed work units, the warp's staging area in sbuf; a warp takes its own unit, then
             // whichever units are left
@@ -605,7 +715,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
                     return __shfl_sync(0xffffffffu, nx, 0);
                 });
             }
-            grid_barrier(br, c);
+            grid_barrier<CL>(br, c);
             st.mark(5);   // K_BP_QUERY
             ncand = block_read(&c->n_cand, &sh_i);
             rebuild = 0;
@@ -674,7 +784,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
                 }
             }
         }
-        grid_barrier(br, c);
+        grid_barrier<CL>(br, c);
         st.mark(6);   // K_GRAD
         if (D.segmented) {
             br.phase = 7;   // K_GATHER
@@ -692,11 +802,11 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
                 D.g[par][i] = G;
                 D.dg[par][i] = Dg;
             }
-            grid_barrier(br, c);
+            grid_barrier<CL>(br, c);
             st.mark(7);   // K_GATHER
         }
         if (D.nseg > 1) {   // batched scenes: per-scene beta, alpha (batched.cuh)
-            if (batched_tail<R, PB, CO>(D, c, sh, sbuf, br, st, rb, k, par, sred, disp_lim)) rebuild = 1;
+            if (batched_tail<R, PB, CO, CL>(D, c, sh, sbuf, br, st, rb, k, par, sred, disp_lim)) rebuild = 1;
             continue;
         }
         // ------------------------------------------------------------ a4: beta (and P g for the direction)
@@ -707,6 +817,9 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
         br.phase = 8;   // K_DOTS
         {
             Acc<R> s5[5];
+            // complete since the gradient pass's barrier, as are its error bits: read here, where the vertices' loads
+            // hide the round trip
+            if (threadIdx.x == 0) { sh.fi = (volatile const int &)c->n_active; sh.fe = (volatile const uint32_t &)c->err; }
             for (int i = ov; i < vs.b1; i += PB) {
                 const R4 G = ldcg4(D.g[par] + i), Dg = ldcg4(D.dg[par] + i), G0 = ldcg4(D.g[par ^ 1] + i);
                 R4 P0 = ldcg4(D.p + i);
@@ -725,9 +838,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
                 D.pg[i] = PG;
                 if (i == ov) { oG = G; oDg = Dg; oPG = PG; oP0 = P0; }
             }
-            Fetch f;
-            f.pi = &c->n_active;
-            grid_reduce<R, PB, 5, false>(s5, R(0), rb.sum_region<PT>(), sh, br, c, &f);
+            grid_reduce<R, PB, CL, 5, false>(s5, R(0), rb.sum_region<PT>(), sh, br, c);
             st.mark(8);   // K_DOTS
             // beta and the restart test: scalar FP64 work, done by one thread and broadcast
             if (threadIdx.x == 0) {
@@ -806,10 +917,10 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
                 }
             }
             Fetch f;
-            f.pe = &c->err;
-            PT *part = rb.sum_region<PT>();
-            block_publish<R, PB, 3, true>(s3, pm, part, sh);
-            grid_barrier(br, c);
+            f.pe = CL ? nullptr : &c->err;   // with bounded waits: a time-out since then counts too
+            const PartDst<PT> part = rb.sum_region<PT>();
+            block_publish<R, PB, CL, 3, true>(s3, pm, part, sh);
+            grid_barrier<CL>(br, c);
             // the update's loads of this thread's own vertex go out before the partial collection and the step rule
             if (ov < vs.b1) {
                 uX = ldcg4(D.x + ov);
@@ -817,7 +928,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
                 if constexpr (sizeof(R) == 8) uXT = ldcg4(D.xtil + ov);
                 uXB = disp_ref<R>(D, ov);
             }
-            grid_collect<R, PB, 3, true>(part, sh, &f);
+            grid_collect<R, PB, CL, 3, true>(part, sh, &f);
             st.mark(10);  // K_PHP (direction included)
             // the step rule (Sec. 4.3) and the predicted decrease: scalar FP64 work, done by one thread
             if (threadIdx.x == 0) {
@@ -895,7 +1006,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
                 }
             }
             if (lead) c->n_active = 0;
-            const R m = grid_max<R, PB>(md, rb.max_region<PT, R>(), sh, br, c);
+            const R m = grid_max<R, PB, CL>(md, rb.max_region<PT, R>(), sh, br, c);
             st.mark(11);  // K_UPDATE
             if ((double)m >= disp_lim * disp_lim) rebuild = 1;
         }
@@ -905,7 +1016,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
     // ---------------------------------------------------------------- velocity update
     if (A.do_finish) {
         br.phase = 12;   // K_FINISH
-        grid_barrier(br, c);
+        grid_barrier<CL>(br, c);
         const bool bad = (volatile uint32_t &)c->err != 0u;
         for (int i = ov; i < vs.b1; i += PB) {
             const double4_32a X = ldcg4(D.x + i), XT = ldcg4(D.xt + i);
@@ -922,7 +1033,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
             if (bad) { if (c->err_step < 0) c->err_step = (int)c->step; }
             else c->step += 1;
         }
-        grid_barrier(br, c);
+        grid_barrier<CL>(br, c);
         st.mark(12);  // K_FINISH
     }
 }
