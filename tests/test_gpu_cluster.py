@@ -1,0 +1,43 @@
+"""The cluster form of the persistent step (small meshes, default block shape): lock-step against the oracle on both
+sides of the size rule, with ragged cell counts, down to one cell, in both precisions; and against the whole-grid form
+over the options that it takes (beta rule, densities, p-norm, split objects, batches)."""
+import numpy as np
+import pytest
+
+from paper_2405_08001_gb300 import scenes as S
+from test_gpu_parity import B, CHECKED, O, TOL, lockstep  # noqa: F401  (B and O are fixtures)
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("prec,cells,blocks", [(1, (1, 1, 1), 1), (1, (9, 11, 13), 1), (1, (11, 11, 12), 2),
+                                               (0, (1, 2, 1), 1), (0, (8, 8, 10), 1), (0, (8, 9, 10), 2)])
+def test_both_sides_of_the_size_rule(B, O, prec, cells, blocks):  # noqa: F811
+    sc = S.cube_drop(n=max(cells), cells=cells, drop=0.0)
+    sc.x0 = sc.x0 + np.array([0.0, 0.0, 0.6 * sc.dhat])
+    sim = B.Sim(sc, precision=prec)
+    st = sim.state()[2]
+    assert (st["block_threads"], st["blocks_per_sm"]) == (256, blocks), st
+    worst = lockstep(B, O, O.Oracle.from_scene(sc), sim, sc, 3, prec)
+    for k in CHECKED:
+        assert worst[k] < TOL[prec], (k, worst[k])
+    sim.close()
+
+
+@pytest.mark.parametrize("make,kw", [(lambda: S.two_blocks(1), dict(beta=1)), (lambda: S.two_blocks(1), dict(pnorm=1)),
+                                     (lambda: S.two_blocks(2), dict(model=1)), (lambda: S.two_blocks(2), dict(model=2)),
+                                     (lambda: S.two_blocks(2), dict(use_graph=0)),
+                                     (lambda: S.two_blocks(2), dict(scatter=1)),
+                                     (lambda: S.objects(0), dict(split_objects=1)),
+                                     (lambda: S.batched(3, n_min=2, n_max=4), {})])
+def test_same_step_as_the_whole_grid(B, make, kw):  # noqa: F811
+    """One FP64 step in the cluster form and in 256 x 1 blocks on the whole grid (the same arithmetic, another order of
+    the sums): equal within the growth of rounding over the step's iterations, about 1e3 to 1e5 on these scenes."""
+    sc = make()
+    out = []
+    for shape in (0, 3):
+        sim = B.Sim(sc, precision=0, block_shape=shape, iters=8, **kw)
+        sim.step(1, sc.targets(0))
+        out.append(sim.state()[0])
+        sim.close()
+    assert np.abs(out[0] - out[1]).max() <= 1e-9 * np.abs(out[1] - sc.x0).max()
