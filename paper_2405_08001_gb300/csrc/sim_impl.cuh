@@ -654,19 +654,51 @@ public:
     // ------------------------------------------------------------------------------------------ differentiation
     sim_status adj_alloc()
     {
-        if (adj_b) return SIM_OK;
+        if (adj_p) return SIM_OK;
         const size_t n3 = 3 * (size_t)M.nv;
-        AL3(adj_b, n3); AL3(adj_x, n3); AL3(adj_r, n3); AL3(adj_z, n3); AL3(adj_p, n3); AL3(adj_q, n3);
+        AL3(adj_x, M.nv); AL3(adj_r, M.nv); AL3(adj_P, M.nv); AL3(adj_q, M.nv);
         AL3(adj_av, n3); AL3(adj_ax, n3); AL3(adj_cg, (size_t)CG_N);
         AL3(adj_dE, (size_t)M.nt);
+        // the solver's launch: one cluster on a small mesh, else as many resident blocks as the device takes together
+        int coop = 0, per_sm = 0;
+        CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+        cg_cluster = 0;
+        if (small_mesh()) CK(largest_cluster(cg_kernel(true), &cg_cluster));
+        cg_coop = cg_cluster == 0 && coop;
+        if (cg_coop) CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cg_kernel(false), CG_PB, 0));
+        cg_grid = cg_cluster > 0 ? cg_cluster : std::max(1, std::min(std::min(per_sm, 2) * nsm, MAXG));
+        AL3(cg_part, 16 * (size_t)cg_grid);
+        AL3(cg_count, 32);
+        AL3(adj_p, M.nv);
         return SIM_OK;
     }
-    // q = H p at the positions of the last eval_setup
-    void launch_hvp(const double *v, double *out)
+    const void *cg_kernel(bool cl) const
     {
-        const int nb = (M.nv + 127) / 128;
-        k_hvp_vert<R><<<nb, 128, 0, s>>>(D, 0, v, out);
-        k_hvp_tet<R><<<(M.nt + EB - 1) / EB, EB, 0, s>>>(D, v, out);
+        if (corot) return cl ? (const void *)k_cg<R, true, true> : (const void *)k_cg<R, true, false>;
+        return cl ? (const void *)k_cg<R, false, true> : (const void *)k_cg<R, false, false>;
+    }
+    // CG iterations it0 .. it1 - 1 at the positions of the last eval_setup
+    cudaError_t launch_cg(int it0, int it1, double tol)
+    {
+        CgArgs A{adj_x, adj_r, adj_p, adj_q, adj_P, adj_cg, cg_part, cg_count, it0, it1, tol * tol};
+        Dev<R> d = D;
+        void *args[] = {(void *)&d, (void *)&A};
+        if (cg_cluster > 0) {
+            cudaLaunchAttribute at;
+            const cudaLaunchConfig_t cfg = cluster_config(cg_grid, at, s);
+            return cudaLaunchKernelExC(&cfg, cg_kernel(true), args);
+        }
+        cudaError_t e = cudaMemsetAsync(cg_count, 0, sizeof(unsigned int), s);
+        if (e != cudaSuccess) return e;
+        if (!cg_coop) return cudaLaunchKernel(cg_kernel(false), dim3(1), dim3(CG_PB), args, 0, s);   // one block waits for none
+        return cudaLaunchCooperativeKernel(cg_kernel(false), dim3(cg_grid), dim3(CG_PB), args, 0, s);
+    }
+    // out = H v at the positions of the last eval_setup
+    void launch_hvp(const double4_32a *v, double4_32a *out)
+    {
+        k_hvp_vert<R><<<(M.nv + 127) / 128, 128, 0, s>>>(D, 0, v, out);
+        if (corot) k_hvp_tet<R, true><<<(M.nt + EB - 1) / EB, EB, 0, s>>>(D, v, out);
+        else k_hvp_tet<R, false><<<(M.nt + EB - 1) / EB, EB, 0, s>>>(D, v, out);
         k_hvp_pair<R><<<ncb, EB, 0, s>>>(D, v, out);
     }
     sim_status eval_hvp(const double *x, const double *v, double *out) override
@@ -677,10 +709,11 @@ public:
         if (r) return r;
         r = eval_setup(x, nullptr);
         if (r) return r;
-        const size_t bytes = sizeof(double) * 3 * (size_t)M.nv;
-        CK(cudaMemcpyAsync(adj_p, v, bytes, cudaMemcpyDefault, s));
+        CK(cudaMemcpyAsync(stage, v, 24 * (size_t)M.nv, cudaMemcpyDefault, s));
+        k_pack4<<<(M.nv + 255) / 256, 256, 0, s>>>(stage, adj_p, M.nv, 0);
         launch_hvp(adj_p, adj_q);
-        CK(cudaMemcpyAsync(out, adj_q, bytes, cudaMemcpyDefault, s));
+        r = out3(adj_q, out);
+        if (r) return r;
         CK(cudaStreamSynchronize(s));
         eval_restore();
         return sync_and_check();
@@ -695,37 +728,28 @@ public:
         if (r) return r;
         r = eval_setup(x1, nullptr);   // H at x_{t+1}: candidates, active pairs and the gradient pass there
         if (r) return r;
-        const size_t n3 = 3 * (size_t)M.nv, bytes = sizeof(double) * n3;
+        const size_t bytes = sizeof(double) * 3 * (size_t)M.nv;
         const int nb = (M.nv + VB - 1) / VB;
         CK(cudaMemcpyAsync(adj_ax, ax1, bytes, cudaMemcpyDefault, s));
         CK(cudaMemcpyAsync(adj_av, av1, bytes, cudaMemcpyDefault, s));
-        k_adj_rhs<R><<<nb, VB, 0, s>>>(D, adj_ax, adj_av, adj_b);
-        unsigned int *tk = &dctrl->ticket[TK_MISC];
-        k_cg_init<R><<<nb, VB, 0, s>>>(D, 0, adj_b, adj_x, adj_r, adj_z, adj_p, adj_cg, tk);
+        k_adj_rhs<R><<<nb, VB, 0, s>>>(D, adj_ax, adj_av, adj_r);
+        // launches of at most CG_LAUNCH iterations, so that none runs for long
         double hcg[CG_N] = {0};
-        CK(cudaMemcpyAsync(hcg, adj_cg, sizeof hcg, cudaMemcpyDeviceToHost, s));
-        CK(cudaStreamSynchronize(s));
-        const double bb = hcg[CG_BB];
         int it = 0;
-        double rr = hcg[CG_RR];
-        while (it < max_iters && bb > 0.0 && rr > tol * tol * bb) {
-            const int batch = std::min(8, max_iters - it);
-            for (int j = 0; j < batch; ++j) {
-                launch_hvp(adj_p, adj_q);
-                k_cg_pq<<<nb, VB, 0, s>>>((int)n3, adj_p, adj_q, D.part, adj_cg, tk);
-                k_cg_update<R><<<nb, VB, 0, s>>>(D, 0, adj_x, adj_r, adj_z, adj_p, adj_q, adj_cg, tk);
-                k_cg_dir<<<nb, VB, 0, s>>>((int)n3, adj_z, adj_p, adj_cg);
-            }
-            it += batch;
+        for (;;) {
+            const int it1 = max_iters - it > CG_LAUNCH ? it + CG_LAUNCH : max_iters;
+            CK(launch_cg(it, it1, tol));
             CK(cudaMemcpyAsync(hcg, adj_cg, sizeof hcg, cudaMemcpyDeviceToHost, s));
             CK(cudaStreamSynchronize(s));
-            rr = hcg[CG_RR];
+            it = (int)hcg[CG_IT];
+            if (it < it1 || it >= max_iters) break;
         }
+        const double bb = hcg[CG_BB], rr = hcg[CG_RR];
         if (iters) *iters = it;
         if (residual) *residual = bb > 0.0 ? std::sqrt(rr / bb) : 0.0;
-        k_adj_out<R><<<nb, VB, 0, s>>>(D, adj_x, adj_av, adj_ax, adj_b);
+        k_adj_out<R><<<nb, VB, 0, s>>>(D, adj_x, adj_av, adj_ax, stage);
         CK(cudaMemcpyAsync(ax0, adj_ax, bytes, cudaMemcpyDefault, s));
-        CK(cudaMemcpyAsync(av0, adj_b, bytes, cudaMemcpyDefault, s));
+        CK(cudaMemcpyAsync(av0, stage, bytes, cudaMemcpyDefault, s));
         if (dE) {
             CK(cudaMemcpyAsync(adj_dE, dE, sizeof(double) * M.nt, cudaMemcpyDefault, s));
             // the elastic gradient is linear in E_e: its derivative is the gradient with E_e = 1
@@ -787,8 +811,13 @@ private:
     unsigned int *bar_count = nullptr;
     void *ppart = nullptr;
     unsigned long long *stamp_buf = nullptr;
-    double *adj_b = nullptr, *adj_x = nullptr, *adj_r = nullptr, *adj_z = nullptr, *adj_p = nullptr, *adj_q = nullptr;
-    double *adj_av = nullptr, *adj_ax = nullptr, *adj_cg = nullptr, *adj_dE = nullptr;
+    // differentiation: the solver's vectors, its launch and its scalars
+    static constexpr int CG_LAUNCH = 1024;   // iterations per launch, a multiple of CG_STRIDE
+    double4_32a *adj_x = nullptr, *adj_r = nullptr, *adj_p = nullptr, *adj_q = nullptr, *adj_P = nullptr;
+    double *adj_av = nullptr, *adj_ax = nullptr, *adj_cg = nullptr, *adj_dE = nullptr, *cg_part = nullptr;
+    unsigned int *cg_count = nullptr;
+    int cg_cluster = 0, cg_grid = 1;
+    bool cg_coop = false;
     int *stamp_kind = nullptr;
 
     sim_status fail(sim_status st, const std::string &m) { err = m; return st; }
