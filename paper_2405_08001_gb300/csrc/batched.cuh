@@ -117,11 +117,11 @@ template <typename R> __device__ inline void seg_reset(const Dev<R> &D)
 }
 
 // Beta, direction + p^T H p, and update phases of iteration k for nseg > 1 scenes (three grid barriers, as in the
-// single-scene form).  sbuf holds the scenes' beta and alpha (2 x MAX_SCENES doubles).  Returns 1 when some vertex
-// has moved far enough since the candidate build to need a new one.
+// single-scene form).  sbuf holds the scenes' beta and alpha (2 x MAX_SCENES doubles).  Returns the largest squared
+// displacement of a vertex since the candidate build.
 template <typename R, int PB, bool CO, bool CL>
-__device__ inline int batched_tail(const Dev<R> &D, Ctrl *c, PShared<R, PB, CL> &sh, unsigned char *sbuf, Bar &br,
-                                   Stamper &st, RedBufs &rb, int k, int par, int &sred, double disp_lim)
+__device__ inline R batched_tail(const Dev<R> &D, Ctrl *c, PShared<R, PB, CL> &sh, unsigned char *sbuf, Bar &br,
+                                   Stamper &st, RedBufs &rb, int k, int par, int &sred)
 {
     typedef typename V4<R>::T R4;
     typedef typename PartT<R>::T PT;
@@ -362,7 +362,7 @@ __device__ inline int batched_tail(const Dev<R> &D, Ctrl *c, PShared<R, PB, CL> 
     if (blockIdx.x == 0 && threadIdx.x == 0) c->n_active = 0;
     const R m = grid_max<R, PB, CL>(md, rb.max_region<PT, R>(), sh, br, c);
     st.mark(11);  // K_UPDATE
-    return (double)m >= disp_lim * disp_lim ? 1 : 0;
+    return m;
 }
 
 } // namespace pncg

@@ -66,7 +66,8 @@ struct BPDev {
     uint2 *units;           // work units, listed by the scan: (bucket, row chunk | column chunk << 16) for edges,
                             // (bucket, row chunk | 0xffff << 16) for triangles
     int ucap;
-    int4 *cand;
+    int4 *cand;             // point-triangle pairs from the front, edge pairs from the end
+    float *cand_d;          // a lower bound of each candidate's distance at the build
     int cap;
     const unsigned long long *excl;
     int nexcl;
@@ -320,7 +321,7 @@ static __global__ void __launch_bounds__(BP_B) bp_boxes(BPDev B)
     const int n = max(max(B.nf + B.ne, B.nv), 3 * B.H);
     const int stride = gridDim.x * blockDim.x;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        B.ctrl->n_cand = 0; B.ctrl->n_units = 0; B.ctrl->n_units_h = 0; B.ctrl->n_rebuilds += 1;
+        B.ctrl->n_cand[0] = B.ctrl->n_cand[1] = 0; B.ctrl->n_units = 0; B.ctrl->n_units_h = 0; B.ctrl->n_rebuilds += 1;
     }
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += stride) {
         if (j < 3 * B.H) B.cnt[j] = 0u;
@@ -465,6 +466,7 @@ struct BPQWarp {
     uint4 ca[32], cb[32];           // the staged columns' records
     uint2 pend[BPQ_PEND];           // (row entry, column entry | BPQ_PT for a point column)
     int4 out[BPQ_OUT];
+    float outd[BPQ_OUT];
 };
 
 __device__ inline unsigned int lanemask_lt() { return (1u << (threadIdx.x & 31)) - 1u; }
@@ -475,21 +477,35 @@ __device__ inline void bpq_flush(const BPDev &B, BPQWarp &W, int &n)
     const int lane = threadIdx.x & 31;
     __syncwarp();
     if (n == 0) return;
-    int base = 0;
-    if (lane == 0) base = atomicAdd(&B.ctrl->n_cand, n);
-    base = __shfl_sync(0xffffffffu, base, 0);
-    for (int i = lane; i < n; i += 32)
-        if (base + i < B.cap) B.cand[base + i] = W.out[i];
+    // by type, so that the passes over the candidates run one kind of geometry per warp
+    for (int i0 = 0; i0 < n; i0 += 32) {
+        const int i = i0 + lane;
+        const int4 cnd = i < n ? W.out[i] : make_int4(0, 0, 0, 0);
+        const unsigned int ee = __ballot_sync(0xffffffffu, i < n && cnd.x < 0), pt = __ballot_sync(0xffffffffu, i < n && cnd.x >= 0);
+        int b = 0;
+        if (lane < 2 && (lane ? ee : pt)) b = atomicAdd(&B.ctrl->n_cand[lane], __popc(lane ? ee : pt));
+        const bool e = cnd.x < 0;
+        const int at = __shfl_sync(0xffffffffu, b, e ? 1 : 0) + __popc((e ? ee : pt) & lanemask_lt());
+        if (i < n && at < B.cap) {
+            const int slot = e ? B.cap - 1 - at : at;
+            B.cand[slot] = cnd;
+            B.cand_d[slot] = W.outd[i];
+        }
+    }
     __syncwarp();
     n = 0;
 }
 
 // holds the lanes' found pairs (all lanes call)
-__device__ inline void bpq_emit(const BPDev &B, BPQWarp &W, int &n, bool found, const int4 &cnd)
+__device__ inline void bpq_emit(const BPDev &B, BPQWarp &W, int &n, bool found, const int4 &cnd, float dlow)
 {
     const unsigned int m = __ballot_sync(0xffffffffu, found);
     if (!m) return;
-    if (found) W.out[n + __popc(m & lanemask_lt())] = cnd;
+    if (found) {
+        const int at = n + __popc(m & lanemask_lt());
+        W.out[at] = cnd;
+        W.outd[at] = dlow;
+    }
     n += __popc(m);
     if (n > BPQ_OUT - 32) bpq_flush(B, W, n);
 }
@@ -499,10 +515,12 @@ __device__ inline unsigned long long key_of(const uint4 &A) { return (unsigned l
 
 // exact tests of the first n queued pairs (all lanes call); both entries of a pair are in the same cell, so their
 // positions are relative to the same corner
-__device__ inline void bpq_exact(const BPDev &B, BPQWarp &W, int n, float thr, int &nout)
+__device__ inline void bpq_exact(const BPDev &B, BPQWarp &W, int n, const CellGrid &g, int &nout)
 {
     const int lane = threadIdx.x & 31;
+    const float thr = B.thr + 4e-6f * g.s;
     bool found = false;
+    float d = 0.0f;
     int4 cnd = make_int4(0, 0, 0, 0);
     if (lane < n) do {
         const uint2 pd = W.pend[lane];
@@ -520,7 +538,7 @@ __device__ inline void bpq_exact(const BPDev &B, BPQWarp &W, int n, float thr, i
                 const int f = __ldcg(B.eprim + qr), jp = __ldcg(B.eprim + qc);
                 if (B.tri[f].w == B.obj[v] && is_excluded(B, ((unsigned long long)jp << 31) | (unsigned long long)f)) break;
             }
-            const float d = pt_coeffs<float>(f3sub(c0, r0), f3sub(r1, r0), f3sub(r2, r0), cc, tv);
+            d = pt_coeffs<float>(f3sub(c0, r0), f3sub(r1, r0), f3sub(r2, r0), cc, tv);
             if (!(d < thr)) break;
             found = true;
             cnd = make_int4(v, (int)Ar.z, (int)Ar.w, t2);
@@ -535,17 +553,20 @@ __device__ inline void bpq_exact(const BPDev &B, BPQWarp &W, int n, float thr, i
                     is_excluded(B, (1ull << 62) | ((unsigned long long)a << 31) | (unsigned long long)b))
                     break;
             }
-            const float d = ee_coeffs<float>(f3sub(r0, c0), f3sub(r1, c0), f3sub(c1, c0), cc, tv);
+            d = ee_coeffs<float>(f3sub(r0, c0), f3sub(r1, c0), f3sub(c1, c0), cc, tv);
             if (!(d < thr)) break;
             found = true;
             cnd = make_int4(-1 - (int)Ar.z, (int)Ar.w, (int)Ac.z, (int)Ac.w);
         }
     } while (false);
-    bpq_emit(B, W, nout, found, cnd);
+    // the bound: less the rounding of the positions (as thr), and less what the clamped cases overestimate for nearly
+    // parallel edges or a sliver triangle (sin^2 of the angle under GeomEps<float>::par = 1e-5: at most L^2 par / (2 d), the
+    // edges no longer than a cell's diagonal)
+    bpq_emit(B, W, nout, found, cnd, d - 4e-6f * g.s - 1.5e-5f * g.s * g.s / fmaxf(d, 1e-30f));
 }
 
 // queues the lanes' passing pairs (all lanes call); runs the exact tests once 32 are queued
-__device__ inline void bpq_push(const BPDev &B, BPQWarp &W, int &np, int &nout, float thr, bool pass, unsigned int qr,
+__device__ inline void bpq_push(const BPDev &B, BPQWarp &W, int &np, int &nout, const CellGrid &g, bool pass, unsigned int qr,
                                 unsigned int qc)
 {
     const unsigned int m = __ballot_sync(0xffffffffu, pass);
@@ -554,7 +575,7 @@ __device__ inline void bpq_push(const BPDev &B, BPQWarp &W, int &np, int &nout, 
     np += __popc(m);
     if (np >= 32) {
         __syncwarp();
-        bpq_exact(B, W, 32, thr, nout);
+        bpq_exact(B, W, 32, g, nout);
         // drop the 32 done
         const int lane = threadIdx.x & 31;
         uint2 v = make_uint2(0u, 0u);
@@ -568,7 +589,7 @@ __device__ inline void bpq_push(const BPDev &B, BPQWarp &W, int &np, int &nout, 
 
 // Work unit (b, r | c << 16) (all lanes call): rows 32 r .. 32 r + 31 of bucket b; columns 32 c .. 32 c + 31 of the
 // same bucket (edges, the pairs with the row before the column), or all entries of point bucket b + 2H (c = 0xffff).
-__device__ inline void bpq_unit(const BPDev &B, uint2 unit, float thr, BPQWarp &W, int &np, int &nout)
+__device__ inline void bpq_unit(const BPDev &B, uint2 unit, const CellGrid &g, BPQWarp &W, int &np, int &nout)
 {
     const int lane = threadIdx.x & 31;
     const unsigned int b = unit.x, r = unit.y & 0xffffu, cc = unit.y >> 16;
@@ -608,17 +629,16 @@ __device__ inline void bpq_unit(const BPDev &B, uint2 unit, float thr, BPQWarp &
             } else {
                 pass &= (Ac.z != Ar.z) & (Ac.z != Ar.w) & (Ac.z != Br.w);
             }
-            bpq_push(B, W, np, nout, thr, pass, qr, (cst + j0 + k) | tag);
+            bpq_push(B, W, np, nout, g, pass, qr, (cst + j0 + k) | tag);
         }
     }
 }
 
 // Work units u = first, first + stride, ... (all lanes of the warp call; its batch area in W).  The candidate
-// threshold adds 4e-6 s to the exact-distance one: positions within a cell or two of a corner keep ~1e-7 s each
+// threshold (bpq_exact) adds 4e-6 s to the exact-distance one: positions within a cell or two of a corner keep ~1e-7 s each
 // in float, and the differences and the distance formed from them stay well inside that.
 template <typename Next> __device__ inline void bpq_units(const BPDev &B, const CellGrid &g, BPQWarp &W, int first, Next next)
 {
-    const float thr = B.thr + 4e-6f * g.s;
     const int nh = ((volatile Ctrl *)B.ctrl)->n_units_h, nl = ((volatile Ctrl *)B.ctrl)->n_units;
     const int nu = nh + nl;
     if (nu > B.ucap) {   // the two ends of the list met: the build cannot be trusted
@@ -627,9 +647,9 @@ template <typename Next> __device__ inline void bpq_units(const BPDev &B, const 
     }
     int np = 0, nout = 0;
     for (int u = first; u < nu; u = next())
-        bpq_unit(B, __ldcg(B.units + (u < nh ? u : B.ucap - 1 - (u - nh))), thr, W, np, nout);
+        bpq_unit(B, __ldcg(B.units + (u < nh ? u : B.ucap - 1 - (u - nh))), g, W, np, nout);
     __syncwarp();
-    if (np) bpq_exact(B, W, np, thr, nout);
+    if (np) bpq_exact(B, W, np, g, nout);
     bpq_flush(B, W, nout);
 }
 

@@ -37,7 +37,8 @@ struct Ctrl {
     unsigned int ticket[TK_COUNT];
     uint32_t err;          // sticky error bits
     int32_t err_step;      // time step index of the first error (-1 = none)
-    int32_t n_cand;        // candidates emitted by the last build (may exceed capacity)
+    int32_t n_cand[2];     // candidates emitted by the last build: point-triangle pairs, listed from the front of the
+                           // buffer, and edge pairs, from its end (together they may exceed the capacity)
     int32_t n_units;       // work units listed by the last build's scan, from the end of the list (may exceed
                            // capacity)
     int32_t n_units_h;     // the heavy ones (tiles of buckets of 64+ entries), from the front

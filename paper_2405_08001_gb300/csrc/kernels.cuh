@@ -50,7 +50,8 @@ template <typename R> struct Dev {
     R mu, lam;
     int model;                         // energy density: MAT_NH, MAT_SNH, MAT_FCR, MAT_ARAP (material.cuh)
     // contacts
-    const int4 *cand;                  // candidates: PT (v, t0, t1, t2), EE (-1 - a0, a1, b0, b1)
+    const int4 *cand;                  // candidates: PT (v, t0, t1, t2) from the front, EE (-1 - a0, a1, b0, b1) from the end
+    const float *cand_d;               // a lower bound of each one's distance at the build
     int cand_cap;
     Active<R> *act;
     // constants
@@ -1060,39 +1061,33 @@ __device__ inline ffn pair_geom_ffn(const Dev<float> &D, bool ee, const int4 &v,
     return ee_coeffs<ffn>(rel_ffn(D, v.x, v.z), rel_ffn(D, v.y, v.z), rel_ffn(D, v.w, v.z), c, t);
 }
 
-// The FP32 form's float filter of a candidate (the first test of pair_grad): whether its float distance is below
-// dhat (1 + 1e-4), i.e. whether pair_grad goes on to the float-float geometry.
-__device__ inline bool pair_passes_filter(const Dev<float> &D, int ci)
+// place of candidate ci in the buffer: the npt point-triangle pairs first, then the edge pairs
+__device__ inline int cand_slot(int ci, int npt, int cap) { return ci < npt ? ci : cap - 1 - (ci - npt); }
+
+// The FP32 form's float filter of a candidate: 0 = its float distance is not below dhat (1 + 1e-4), 1 = pair_grad goes on
+// to the float-float geometry, 2 = to the double one (d < 1e-3 dhat).
+__device__ inline int pair_filter(const Dev<float> &D, const int4 &q)
 {
-    const int4 q = ldcg4(D.cand + ci);
     const bool ee = q.x < 0;
     const int4 v = make_int4(ee ? -1 - q.x : q.x, q.y, q.z, q.w);
     float c[4];
     v3<float> t;
-    return pair_geom_ff(D, ee, v, c, t) < float(D.dhat) * 1.0001f;
+    const float d = pair_geom_ff(D, ee, v, c, t);
+    return !(d < float(D.dhat) * 1.0001f) ? 0 : d < 1e-3f * float(D.dhat) ? 2 : 1;
 }
 
-// Barrier gradient and diagonal of one candidate (Eqs. 8-11) when d < dhat; records the pair for p^T H p.
+// Barrier gradient and diagonal of one candidate (Eqs. 8-11) when d < dhat; records the pair for p^T H p.  `near`: the FP32
+// form's filter said 2.
 template <typename R>
-__device__ inline void pair_grad(const Dev<R> &D, int ci, int par)
+__device__ inline void pair_grad(const Dev<R> &D, const int4 &q, int par, bool near = false)
 {
-    const int4 q = ldcg4(D.cand + ci);
     const bool ee = q.x < 0;
     int4 v = make_int4(ee ? -1 - q.x : q.x, q.y, q.z, q.w);
     R c[4];
     v3<R> t;
-    R d;
+    R d = R(0), r = R(0);   // r = d - dhat: from the float-float distance in the FP32 form
     if constexpr (sizeof(R) == 4) {
-        d = pair_geom_ff(D, ee, v, c, t);
-        if (!(d < R(D.dhat) * R(1.0001))) return;   // float filter; the exact cut-off test follows
-    } else {
-        d = pair_geom<R>(ee, ldcg4(D.x + v.x), ldcg4(D.x + v.y), ldcg4(D.x + v.z), ldcg4(D.x + v.w), c, t);
-        if (!(d < R(D.dhat))) return;
-    }
-    R A, B;
-    R r = d - R(D.dhat);   // d - dhat: from the float-float distance in the FP32 form
-    if constexpr (sizeof(R) == 4) {
-        if (!(d < R(1e-3) * R(D.dhat))) {
+        if (!near) {
             ffn cf[4];
             v3<ffn> tf;
             const ffn df = pair_geom_ffn(D, ee, v, cf, tf);
@@ -1104,8 +1099,13 @@ __device__ inline void pair_grad(const Dev<R> &D, int ci, int par)
             d = __fadd_rn(df.h, df.l);
             r = __fadd_rn(rf.h, rf.l);
         }
+    } else {
+        d = pair_geom<R>(ee, ldcg4(D.x + v.x), ldcg4(D.x + v.y), ldcg4(D.x + v.z), ldcg4(D.x + v.w), c, t);
+        if (!(d < R(D.dhat))) return;
+        r = d - R(D.dhat);
     }
-    if (sizeof(R) == 4 && d < R(1e-3) * R(D.dhat)) {
+    R A, B;
+    if (near) {
         // near-zero distance: evaluate in double and round the results
         double cd[4];
         v3<double> td;
@@ -1147,6 +1147,17 @@ __device__ inline void pair_grad(const Dev<R> &D, int ci, int par)
     }
 }
 
+// pair_grad behind the FP32 form's filter
+template <typename R> __device__ inline void pair_test(const Dev<R> &D, const int4 &q, int par)
+{
+    if constexpr (sizeof(R) == 4) {
+        const int f = pair_filter(D, q);
+        if (f) pair_grad<R>(D, q, par, f == 2);
+    } else {
+        pair_grad<R>(D, q, par);
+    }
+}
+
 // Gradient pass: blocks [0, ntb) own tets, the rest loop over the candidates.
 template <typename R, bool CO = false>
 __global__ void __launch_bounds__(EB) k_grad(Dev<R> D, int par, int ntb)
@@ -1154,15 +1165,16 @@ __global__ void __launch_bounds__(EB) k_grad(Dev<R> D, int par, int ntb)
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         Ctrl *c = D.ctrl;
         c->rebuild = 0;
-        if (c->n_cand > D.cand_cap) flag_error(c, ERR_CAPACITY);
+        if (c->n_cand[0] + c->n_cand[1] > D.cand_cap) flag_error(c, ERR_CAPACITY);
     }
     if ((int)blockIdx.x < ntb) {
         __shared__ R sacc[6 * SCATTER_MAXU];
         tet_grad_chunk<R, CO>(D, blockIdx.x, par, sacc);
     } else {
-        const int nc = min(D.ctrl->n_cand, D.cand_cap);
+        const int npt = D.ctrl->n_cand[0], nc = min(npt + D.ctrl->n_cand[1], D.cand_cap);
         const int stride = (gridDim.x - ntb) * blockDim.x;
-        for (int ci = (blockIdx.x - ntb) * blockDim.x + threadIdx.x; ci < nc; ci += stride) pair_grad<R>(D, ci, par);
+        for (int ci = (blockIdx.x - ntb) * blockDim.x + threadIdx.x; ci < nc; ci += stride)
+            pair_test<R>(D, ldcg4(D.cand + cand_slot(ci, npt, D.cand_cap)), par);
     }
 }
 
@@ -1709,10 +1721,10 @@ __global__ void __launch_bounds__(EB) k_energy(Dev<R> D, int ntb, int nvb)
             }
         }
     } else {
-        const int nc = min(D.ctrl->n_cand, D.cand_cap);
+        const int npt = D.ctrl->n_cand[0], nc = min(npt + D.ctrl->n_cand[1], D.cand_cap);
         const int stride = (gridDim.x - ntb - nvb) * blockDim.x;
         for (int ci = (b - ntb - nvb) * blockDim.x + threadIdx.x; ci < nc; ci += stride) {
-            const int4 q = D.cand[ci];
+            const int4 q = D.cand[cand_slot(ci, npt, D.cand_cap)];
             const bool ee = q.x < 0;
             const double4_32a X0 = D.x[ee ? -1 - q.x : q.x], X1 = D.x[q.y], X2 = D.x[q.z], X3 = D.x[q.w];
             double c[4];

@@ -523,7 +523,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
                                  sizeof(BPQWarp) * (PB / 32));
     __shared__ __align__(16) unsigned char sbuf[SBUF];
     static_assert(SBUF >= 2 * MAX_SCENES * sizeof(double), "the batched form keeps per-scene beta and alpha here");
-    static_assert(SBUF >= (PB / 32) * 64 * sizeof(int), "the gradient pass queues candidates here, 64 per warp");
+    static_assert(SBUF >= (PB / 32) * 128 * sizeof(int), "the gradient pass queues candidates here, 2 x 64 per warp");
     // the block-aggregated scatter (options.scatter = block) covers one chunk of SCATTER_CHUNK tets per block: only
     // the shape with PB == SCATTER_CHUNK runs it (the host keeps that shape for it)
     Ctrl *c = D.ctrl;
@@ -543,7 +543,8 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
     double gPg_prev = (volatile double &)c->gPg_prev;
     double dE0 = (volatile double &)c->dE0;
     int converged = (volatile int &)c->converged;
-    int ncand = (volatile int &)c->n_cand;
+    int npt = (volatile int &)c->n_cand[0], ncand = npt + (volatile int &)c->n_cand[1];
+    R disp_max = R(-1);   // largest squared displacement of a vertex since the last candidate build; < 0: not known
     const double disp_lim = 0.5 * D.pad_r * (1.0 - 1e-4);
     Stamper st{A.stamps, A.stamp_kind, A.max_stamps};
     if (lead) { c->ticket[TK_PAIRS] = 0u; c->ticket[TK_PAIRS1] = 0u; }
@@ -578,6 +579,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
             }
         }
         const R m = grid_max<R, PB, CL>(md, rb.max_region<PT, R>(), sh, br, c);
+        disp_max = m;
         if (!skip_step && (double)m >= disp_lim * disp_lim) rebuild = 1;
         gPg_prev = 0.0;
         dE0 = 0.0;
@@ -598,7 +600,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
         if (rebuild) {
             br.phase = 1;   // K_BP_BOXES
             // boxes, bucket counts to zero, build positions; the cell size is the grid max of the box extents
-            if (lead) { c->n_cand = 0; c->n_units = 0; c->n_units_h = 0; c->n_rebuilds += 1; c->ticket[TK_QUERY] = 0u; }
+            if (lead) { c->n_cand[0] = c->n_cand[1] = 0; c->n_units = 0; c->n_units_h = 0; c->n_rebuilds += 1; c->ticket[TK_QUERY] = 0u; }
             const int nprim = B.nf + B.ne;
             float ext_max = 0.0f;
             for (int j = tid; j < 3 * B.H; j += nthr) B.cnt[j] = 0u;
@@ -717,7 +719,9 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
             }
             grid_barrier<CL>(br, c);
             st.mark(5);   // K_BP_QUERY
-            ncand = block_read(&c->n_cand, &sh_i);
+            npt = block_read(&c->n_cand[0], &sh_i);
+            ncand = npt + block_read(&c->n_cand[1], &sh_i);
+            disp_max = R(0);
             rebuild = 0;
         }
         // ------------------------------------------------------------ a2-a3: gradient + diagonal
@@ -727,12 +731,13 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
             if (ncand > D.cand_cap) flag_error(c, ERR_CAPACITY);
         }
         {
-            const Share cs = share_of(min(ncand, D.cand_cap));
             if (PB == SCATTER_CHUNK && D.scatter_block) {
                 const int nch = (D.nt + SCATTER_CHUNK - 1) / SCATTER_CHUNK;
                 for (int ch = blockIdx.x; ch < nch; ch += gridDim.x)
                     tet_grad_chunk<R, CO>(D, ch, par, reinterpret_cast<R *>(sbuf));
-                for (int ci = cs.b0 + (int)threadIdx.x; ci < cs.b1; ci += PB) pair_grad<R>(D, ci, par);
+                const Share cs = share_of(min(ncand, D.cand_cap));
+                for (int ci = cs.b0 + (int)threadIdx.x; ci < cs.b1; ci += PB)
+                    pair_test<R>(D, ldcg4(D.cand + cand_slot(ci, npt, D.cand_cap)), par);
             } else {
                 // the block's share of the tets, then candidates 32 at a time per warp from a grid-wide cursor: the
                 // active ones (float-float geometry) cluster in the candidate order, and a fixed share per block
@@ -746,40 +751,54 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
                 if (lead) c->ticket[TK_PAIRS + ((k + 1) & 1)] = 0u;   // the next iteration's cursor
                 unsigned int *cur = &c->ticket[TK_PAIRS + (k & 1)];
                 const int nc = min(ncand, D.cand_cap), lane = threadIdx.x & 31;
-                if constexpr (sizeof(R) == 4) {
-                    // the float filter first; the candidates that pass it queue in shared memory (per warp) and
-                    // take the float-float geometry 32 at a time, so that the long path runs with full warps (the
-                    // passing ones are a fraction of each batch: a warp otherwise ran it once per batch)
-                    int *wq = reinterpret_cast<int *>(sbuf) + (threadIdx.x >> 5) * 64;
-                    int qn = 0;
-                    const unsigned int below = (1u << lane) - 1u;
-                    for (;;) {
+                // d changes by at most twice the largest displacement, so a candidate whose distance at the build was
+                // above `reach` cannot be active: it is passed over on that number alone, without its positions
+                // (1e-3 of the displacement and of dhat + r cover the floats' rounding)
+                const float reach = disp_max < R(0) ? 3.0e38f
+                                                    : (float)D.dhat + 2.002f * sqrtf((float)disp_max) + (B.thr - (float)B.infl);
+                // the candidates within reach queue in shared memory, per warp, and are worked on 32 at a time, so that
+                // the geometry runs with full warps; in the FP32 form they take the float filter first, and those that
+                // pass it queue once more for the float-float geometry
+                int *q0 = reinterpret_cast<int *>(sbuf) + (threadIdx.x >> 5) * 128, *q1 = q0 + 64;
+                int n0 = 0, n1 = 0;
+                const unsigned int below = (1u << lane) - 1u;
+                for (bool more = true; more || n0 > 0 || n1 > 0;) {
+                    if (more && n0 < 32) {
                         int b0 = 0;
                         if (lane == 0) b0 = (int)atomicAdd(cur, 32u);
                         b0 = __shfl_sync(0xffffffffu, b0, 0);
-                        if (b0 >= nc) break;
-                        const int ci = b0 + lane;
-                        const bool pass = ci < nc && pair_passes_filter(D, ci);
-                        const unsigned int bal = __ballot_sync(0xffffffffu, pass);
-                        if (pass) wq[qn + __popc(bal & below)] = ci;
-                        qn += __popc(bal);
+                        more = b0 < nc;
+                        const int ci = b0 + lane, sl = cand_slot(ci, npt, D.cand_cap);
+                        const bool in = ci < nc && __ldcg(D.cand_d + sl) < reach;
+                        const unsigned int bal = __ballot_sync(0xffffffffu, in);
+                        if (in) q0[n0 + __popc(bal & below)] = sl;
+                        n0 += __popc(bal);
                         __syncwarp();
-                        if (qn >= 32) {
-                            const int cj = wq[qn - 32 + lane];
+                        if (more && n0 < 32) continue;
+                    }
+                    if (n0 > 0) {   // 32, or the last ones
+                        const int n = min(n0, 32), sl = lane < n ? q0[n0 - n + lane] : 0;
+                        __syncwarp();
+                        n0 -= n;
+                        if constexpr (sizeof(R) == 4) {
+                            const int f = lane < n ? pair_filter(D, ldcg4(D.cand + sl)) : 0;
+                            const unsigned int bal = __ballot_sync(0xffffffffu, f != 0);
+                            if (f) q1[n1 + __popc(bal & below)] = f == 2 ? sl | (int)0x80000000 : sl;
+                            n1 += __popc(bal);
                             __syncwarp();
-                            qn -= 32;
-                            pair_grad<R>(D, cj, par);
+                        } else {
+                            if (lane < n) pair_grad<R>(D, ldcg4(D.cand + sl), par);
+                            __syncwarp();
                         }
                     }
-                    if (lane < qn) pair_grad<R>(D, wq[lane], par);
-                    __syncwarp();
-                } else {
-                    for (;;) {
-                        int b0 = 0;
-                        if (lane == 0) b0 = (int)atomicAdd(cur, 32u);
-                        b0 = __shfl_sync(0xffffffffu, b0, 0);
-                        if (b0 >= nc) break;
-                        if (b0 + lane < nc) pair_grad<R>(D, b0 + lane, par);
+                    if constexpr (sizeof(R) == 4) {
+                        if (n1 >= 32 || (!more && n0 == 0 && n1 > 0)) {
+                            const int n = min(n1, 32), sl = lane < n ? q1[n1 - n + lane] : 0;
+                            __syncwarp();
+                            n1 -= n;
+                            if (lane < n) pair_grad<R>(D, ldcg4(D.cand + (sl & 0x7fffffff)), par, sl < 0);
+                            __syncwarp();
+                        }
                     }
                 }
             }
@@ -806,7 +825,8 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
             st.mark(7);   // K_GATHER
         }
         if (D.nseg > 1) {   // batched scenes: per-scene beta, alpha (batched.cuh)
-            if (batched_tail<R, PB, CO, CL>(D, c, sh, sbuf, br, st, rb, k, par, sred, disp_lim)) rebuild = 1;
+            disp_max = batched_tail<R, PB, CO, CL>(D, c, sh, sbuf, br, st, rb, k, par, sred);
+            if ((double)disp_max >= disp_lim * disp_lim) rebuild = 1;
             continue;
         }
         // ------------------------------------------------------------ a4: beta (and P g for the direction)
@@ -1008,6 +1028,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
             if (lead) c->n_active = 0;
             const R m = grid_max<R, PB, CL>(md, rb.max_region<PT, R>(), sh, br, c);
             st.mark(11);  // K_UPDATE
+            disp_max = m;
             if ((double)m >= disp_lim * disp_lim) rebuild = 1;
         }
     }

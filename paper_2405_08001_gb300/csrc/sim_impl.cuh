@@ -281,7 +281,7 @@ public:
             std::memset(st, 0, sizeof *st);
             st->step = hctrl->step;
             st->iters_done = hctrl->iters_done;
-            st->n_candidates = hctrl->n_cand;
+            st->n_candidates = hctrl->n_cand[0] + hctrl->n_cand[1];
             st->n_active = hctrl->n_active_last;
             st->n_rebuilds = hctrl->n_rebuilds;
             st->n_capped = hctrl->n_capped;
@@ -457,12 +457,15 @@ public:
     {
         CK(cudaSetDevice(dev));
         sim_status r = sync_and_check();
-        const int n = std::min(hctrl->n_cand, cap);
-        if (count) *count = hctrl->n_cand;
+        const int npt = std::min(hctrl->n_cand[0], cap), n = std::min(hctrl->n_cand[0] + hctrl->n_cand[1], cap);
+        if (count) *count = hctrl->n_cand[0] + hctrl->n_cand[1];
         const int m = std::min(n, std::max(max, 0));
         if (m > 0 && idx) {
+            // point-triangle pairs from the front of the buffer, edge pairs from its end
             std::vector<int4> h(m);
-            CK(cudaMemcpy(h.data(), D.cand, sizeof(int4) * (size_t)m, cudaMemcpyDeviceToHost));
+            const int m0 = std::min(m, npt), m1 = m - m0;
+            CK(cudaMemcpy(h.data(), D.cand, sizeof(int4) * (size_t)m0, cudaMemcpyDeviceToHost));
+            if (m1 > 0) CK(cudaMemcpy(h.data() + m0, D.cand + cap - m1, sizeof(int4) * (size_t)m1, cudaMemcpyDeviceToHost));
             for (int i = 0; i < m; ++i) {
                 const bool ee = h[i].x < 0;
                 idx[5 * i] = ee ? 1 : 0;
@@ -931,9 +934,13 @@ private:
     sim_status alloc_candidates()
     {
         int4 *cd;
+        float *dist;
         AL(cd, (size_t)cap);
+        AL(dist, (size_t)cap);
         AL(D.act, (size_t)cap);
         D.cand = cd;
+        D.cand_d = dist;
+        B.cand_d = dist;
         D.cand_cap = cap;
         B.cand = cd;
         B.cap = cap;
@@ -1283,7 +1290,7 @@ private:
         else if (e & ERR_RANGE) { st = SIM_ERR_NONFINITE; what = "positions outside the hash grid range"; }
         else if (e & ERR_TIMEOUT) { st = SIM_ERR_TIMEOUT; what = "device wait timed out"; }
         err = what + " in time step " + std::to_string(hctrl->err_step);
-        const int need = hctrl->n_cand;
+        const int need = hctrl->n_cand[0] + hctrl->n_cand[1];
         hctrl->err = 0u;
         hctrl->err_step = -1;
         CK(cudaMemcpy(&dctrl->err, &hctrl->err, sizeof(uint32_t), cudaMemcpyHostToDevice));
