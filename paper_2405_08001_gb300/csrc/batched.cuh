@@ -11,8 +11,9 @@
 // in several groups adds to each of them with the other groups' entries of p zero.
 //
 // Per-scene sums: the lanes of a warp take consecutive vertices (tets), so their scene ids are non-decreasing (with
-// parts, runs of equal ids); a segmented warp scan adds up each run of equal ids and the run's last lane adds it to
-// the scene's accumulator with a double atomic.  Accumulators are used round robin over three buffers: reduction r accumulates into buffer
+// parts, runs of equal ids).  A block takes a contiguous share, so that its warps stay in one scene for many items, whose
+// sums stay in registers (SegRun); where the ids within the 32 items differ a segmented warp scan adds up each run of
+// equal ids and the run's last lane adds it to the scene's accumulator with a double atomic.  Accumulators are used round robin over three buffers: reduction r accumulates into buffer
 // r % 3 and zeroes buffer (r + 1) % 3 for the next one, which every block last read before the barrier of
 // reduction r - 1.  After the barrier every block computes all scenes' scalars itself (identical values) into
 // shared memory; block 0 also writes them to the per-scene state.
@@ -95,6 +96,50 @@ __device__ inline void seg_warp_max(R m, int key, unsigned long long *mx)
     if (key >= 0 && (lane == 31 || kn != key)) atomicMax(mx + key, max_bits<R>(m));
 }
 
+// Running sums of a warp whose items mostly stay in one group: while all its lanes' items have the group of the sums so
+// far, each lane adds its own; a change of group sends the sums to the accumulator.  The scan of seg_warp_sum, about
+// 100 instructions a quantity, thus runs once per group that a warp meets instead of once per 32 items.
+template <typename R, int N> struct SegRun {
+    Acc<R> a[N];
+    R m = R(0);     // a maximum of non-negative values beside the sums (where mx is given)
+    int key = -1;   // warp-uniform; -1: empty
+    // all lanes call; k < 0: the lane has no item (its v and w are zero)
+    __device__ inline void add(Acc<R> (&v)[N], int k, double *acc, int q0, unsigned long long *mx = nullptr, R w = R(0))
+    {
+        if (!__all_sync(0xffffffffu, k == key || k < 0)) {
+            flush(acc, q0, mx);
+            const unsigned int has = __ballot_sync(0xffffffffu, k >= 0);
+            const int k0 = __shfl_sync(0xffffffffu, k, __ffs(has) - 1);   // some lane has an item: the sums were not its group's
+            if (!__all_sync(0xffffffffu, k == k0 || k < 0)) {
+                seg_warp_sum<R, N>(v, k, acc, q0);
+                if (mx) seg_warp_max<R>(w, k, mx);
+                return;
+            }
+            key = k0;
+        }
+#pragma unroll
+        for (int q = 0; q < N; ++q) a[q].add(v[q]);
+        m = fmax(m, w);
+    }
+    __device__ inline void flush(double *acc, int q0, unsigned long long *mx = nullptr)
+    {
+        if (key >= 0) {
+#pragma unroll
+            for (int q = 0; q < N; ++q) {
+                for (int o = 16; o > 0; o >>= 1) a[q].add(a[q].shfl_down(o));
+                if ((threadIdx.x & 31) == 0) atomicAdd(acc + (size_t)key * 8 + q0 + q, a[q].value());
+                a[q] = Acc<R>();
+            }
+            if (mx) {
+                for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
+                if ((threadIdx.x & 31) == 0) atomicMax(mx + key, max_bits<R>(m));
+            }
+        }
+        m = R(0);
+        key = -1;
+    }
+};
+
 // zeroes the accumulators reduction r + 1 will use
 __device__ inline void seg_zero_next(double *sacc, unsigned long long *smax, int nseg, int r, int tid, int nthr)
 {
@@ -127,6 +172,7 @@ __device__ inline R batched_tail(const Dev<R> &D, Ctrl *c, PShared<R, PB, CL> &s
     typedef typename PartT<R>::T PT;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x, nthr = gridDim.x * blockDim.x;
     const int lane = threadIdx.x & 31;
+    const Share vs = share_of(D.nv), ts = share_of(D.nt);
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
     const int ns = D.nseg;
     const int rp = (k - 1) & 1, wp = k & 1;
@@ -149,11 +195,12 @@ __device__ inline R batched_tail(const Dev<R> &D, Ctrl *c, PShared<R, PB, CL> &s
     {
         double *acc = D.sacc + (size_t)(sred % 3) * ns * 8;
         seg_zero_next(D.sacc, D.smax, ns, sred, tid, nthr);
-        for (int base = tid - lane; base < D.nv; base += nthr) {
+        SegRun<R, 5> run;
+        for (int base = vs.b0 + (int)threadIdx.x - lane; base < vs.b1; base += PB) {
             const int i = base + lane;
             Acc<R> a5[5];
             int key = -1;
-            if (i < D.nv) {
+            if (i < vs.b1) {
                 key = group_of(D, i);
                 const R4 G = ldcg4(D.g[par] + i), Dg = ldcg4(D.dg[par] + i), G0 = ldcg4(D.g[par ^ 1] + i);
                 const R4 P0 = ldcg4(D.p + i);
@@ -170,8 +217,9 @@ __device__ inline R batched_tail(const Dev<R> &D, Ctrl *c, PShared<R, PB, CL> &s
                 }
                 D.pg[i] = PG;
             }
-            seg_warp_sum<R, 5>(a5, key, acc, 0);
+            run.add(a5, key, acc, 0);
         }
+        run.flush(acc, 0);
         grid_barrier<CL>(br, c);
         if (threadIdx.x == 0) sh.fi = (volatile const int &)c->n_active;
         for (int s = threadIdx.x; s < ns; s += blockDim.x) {
@@ -206,12 +254,13 @@ __device__ inline R batched_tail(const Dev<R> &D, Ctrl *c, PShared<R, PB, CL> &s
         double *acc = D.sacc + (size_t)(sred % 3) * ns * 8;
         unsigned long long *mx = D.smax + (size_t)(sred % 3) * ns;
         seg_zero_next(D.sacc, D.smax, ns, sred, tid, nthr);
-        for (int base = tid - lane; base < D.nv; base += nthr) {
+        SegRun<R, 3> runv;
+        for (int base = vs.b0 + (int)threadIdx.x - lane; base < vs.b1; base += PB) {
             const int i = base + lane;
             Acc<R> a2[3];   // g^T p, p^T M p, vertices (a group without vertices takes no step)
             R pmv = R(0);
             int key = -1;
-            if (i < D.nv) {
+            if (i < vs.b1) {
                 key = group_of(D, i);
                 a2[2].add(R(1));
                 const double bd = sbeta[key];
@@ -232,21 +281,23 @@ __device__ inline R batched_tail(const Dev<R> &D, Ctrl *c, PShared<R, PB, CL> &s
                 }
                 D.pnext[i] = Pn;
             }
-            seg_warp_sum<R, 3>(a2, key, acc, 0);
-            seg_warp_max<R>(pmv, key, mx);
+            runv.add(a2, key, acc, 0, mx, pmv);
         }
-        for (int base = tid - lane; base < D.nt; base += nthr) {
+        runv.flush(acc, 0, mx);
+        SegRun<R, 1> runt;
+        for (int base = ts.b0 + (int)threadIdx.x - lane; base < ts.b1; base += PB) {
             const int e = base + lane;
             Acc<R> a1[1];
             int key = -1;
-            if (e < D.nt) {
+            if (e < ts.b1) {
                 const int4 tv = D.tet[e];
                 const int vv[4] = {tv.x, tv.y, tv.z, tv.w};
                 int ks[4];
                 R4 pv[4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {   // each vertex takes the direction of its own group
-                    ks[q] = group_of(D, vv[q]);
+                for (int q = 0; q < 4; ++q) {   // each vertex takes the direction of its own group (without parts a
+                                                // tet lies in one)
+                    ks[q] = q == 0 || D.cmark ? group_of(D, vv[q]) : ks[0];
                     const double bd = sbeta[ks[q]];
                     pv[q] = dir_of<R>(D, vv[q], R(bd), bd != 0.0);
                 }
@@ -263,8 +314,9 @@ __device__ inline R batched_tail(const Dev<R> &D, Ctrl *c, PShared<R, PB, CL> &s
                                                              ks[2] == u[j] ? pv[2] : z, ks[3] == u[j] ? pv[3] : z));
                 }
             }
-            seg_warp_sum<R, 1>(a1, key, acc, 4);
+            runt.add(a1, key, acc, 4);
         }
+        runt.flush(acc, 4);
         for (int kk = tid; kk < na; kk += nthr) {   // active pairs come in no order: one atomic each
             Active<R> ap;
             load_active<R>(D, kk, ap);
@@ -343,7 +395,7 @@ __device__ inline R batched_tail(const Dev<R> &D, Ctrl *c, PShared<R, PB, CL> &s
     // ------------------------------------------------------------ update (per-scene alpha)
     br.phase = 11;   // K_UPDATE
     R md = R(0);
-    for (int i = tid; i < D.nv; i += nthr) {
+    for (int i = vs.b0 + (int)threadIdx.x; i < vs.b1; i += PB) {
         double4_32a X = ldcg4(D.x + i);
         const R4 P = ldcg4(D.pnext + i);
         const double a = salpha[group_of(D, i)];
