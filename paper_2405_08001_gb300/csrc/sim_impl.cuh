@@ -56,6 +56,57 @@ template <typename R4, typename R> __global__ void k_precond_out(const R4 *dg, d
     out[3 * i + 1] = double(precond<R>(d.y, d.w));
     out[3 * i + 2] = double(precond<R>(d.z, d.w));
 }
+// set_state: x and v ([n][3], null = keep) into the state and its float-float copy; the next pass builds candidates
+template <typename R> __global__ void k_set_state(Dev<R> D, const double *x, const double *v)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) { D.ctrl->rebuild = 1; D.ctrl->cell_bits = 0u; }
+    if (i >= D.nv) return;
+    if (x) put_x<R>(D, i, make_double4_32a(x[3 * i], x[3 * i + 1], x[3 * i + 2], 0.0));
+    if (v) D.v[i] = make_double4_32a(v[3 * i], v[3 * i + 1], v[3 * i + 2], 0.0);
+}
+// two [n][3] outputs at once (null = none)
+template <typename R4> __global__ void k_out2(const R4 *a, const R4 *b, double *oa, double *ob, int n)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    if (oa) { const R4 v = a[i]; oa[3 * i] = double(v.x); oa[3 * i + 1] = double(v.y); oa[3 * i + 2] = double(v.z); }
+    if (ob) { const R4 v = b[i]; ob[3 * i] = double(v.x); ob[3 * i + 1] = double(v.y); ob[3 * i + 2] = double(v.z); }
+}
+// Before an evaluation at x (and x~ = xt; null keeps it): the state's x and x~ set aside, every vertex free, iteration 0's
+// accumulators initialised, a candidate build requested and the counters cleared.
+template <typename R> __global__ void k_eval_in(Dev<R> D, const double *x, const double *xt, double4_32a *xsave, double4_32a *xtsave)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) {
+        Ctrl *c = D.ctrl;
+        c->rebuild = 1; c->cell_bits = 0u; c->n_active = 0; c->n_near64 = 0;
+    }
+    if (i >= D.nv) return;
+    const double4_32a T = D.xtil[i];
+    xsave[i] = D.x[i];
+    xtsave[i] = T;
+    const double4_32a X = make_double4_32a(x[3 * i], x[3 * i + 1], x[3 * i + 2], 0.0);
+    const double4_32a XT = xt ? make_double4_32a(xt[3 * i], xt[3 * i + 1], xt[3 * i + 2], D.mass[i]) : make_double4_32a(T.x, T.y, T.z, D.mass[i]);
+    D.xtil[i] = XT;
+    put_x<R>(D, i, X);
+    put_xt<R>(D, i, XT);
+    init_vertex<R>(D, i, X, XT, 0);
+}
+// After it: the state as it was, the evaluation's active pairs as the last ones
+template <typename R> __global__ void k_eval_out(Dev<R> D, const double4_32a *xsave, const double4_32a *xtsave)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) {
+        Ctrl *c = D.ctrl;
+        c->rebuild = 1; c->cell_bits = 0u; c->n_active_last = c->n_active; c->n_active = 0;
+    }
+    if (i >= D.nv) return;
+    const double4_32a T = xtsave[i];
+    D.xtil[i] = T;
+    put_x<R>(D, i, xsave[i]);
+    put_xt<R>(D, i, T);
+}
 // inertia / plane initialisation of parity par at the current x (after the caller changed x or xtil)
 template <typename R> __global__ void k_reinit(Dev<R> D, int par)
 {
@@ -71,12 +122,6 @@ template <typename R> __global__ void k_refresh_ff(Dev<R> D)
         put_x<R>(D, i, D.x[i]);
         put_xt<R>(D, i, D.xtil[i]);
     }
-}
-// xtil.w = mass for every vertex (unmasked evaluation)
-static __global__ void k_set_mass_w(double4_32a *xt, const double *mass, int n)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) xt[i].w = mass[i];
 }
 // p^T M p + plane part for sim_eval_pHp: written to ctrl->pHp_vert
 template <typename R> __global__ void __launch_bounds__(VB) k_eval_vert_pHp(Dev<R> D, int par)
@@ -122,8 +167,6 @@ template <typename R, bool CO = false> __global__ void __launch_bounds__(EB) k_e
         if (threadIdx.x == 0) D.ctrl->pHp = t[0] + D.ctrl->pHp_vert;
     }
 }
-static __global__ void k_copy_count(Ctrl *c) { c->n_active_last = c->n_active; }
-
 #define AL3(p, n) do { sim_status st_ = dalloc(p, n); if (st_ != SIM_OK) return st_; } while (0)
 #define CK(call)                                                                      \
     do {                                                                              \
@@ -274,8 +317,7 @@ public:
     sim_status get_state(double *x, double *v, sim_stats *st) override
     {
         CK(cudaSetDevice(dev));
-        if (x) { sim_status r = out3(D.x, x); if (r) return r; }
-        if (v) { sim_status r = out3(D.v, v); if (r) return r; }
+        if (x || v) { sim_status r = out2(D.x, D.v, x, v); if (r) return r; }
         sim_status r = sync_and_check();
         if (st) {
             std::memset(st, 0, sizeof *st);
@@ -301,9 +343,11 @@ public:
     sim_status set_state(const double *x, const double *v) override
     {
         CK(cudaSetDevice(dev));
-        if (x) { sim_status r = in3(x, D.x); if (r) return r; }
-        if (v) { sim_status r = in3(v, D.v); if (r) return r; }
-        force_rebuild();
+        const double *dx = nullptr, *dv = nullptr;
+        if (x) { sim_status r = on_device(x, stage, dx); if (r) return r; }
+        if (v) { sim_status r = on_device(v, stage + 3 * (size_t)M.nv, dv); if (r) return r; }
+        k_set_state<R><<<(M.nv + 255) / 256, 256, 0, s>>>(D, dx, dv);
+        CK(cudaGetLastError());
         CK(cudaStreamSynchronize(s));
         return SIM_OK;
     }
@@ -357,31 +401,20 @@ public:
     // Runs the candidate build and the gradient pass at the given x (and xtilde) with all vertices free.
     sim_status eval_setup(const double *x, const double *xt)
     {
-        CK(cudaMemcpyAsync(xsave, D.x, sizeof(double4_32a) * (size_t)M.nv, cudaMemcpyDeviceToDevice, s));
-        CK(cudaMemcpyAsync(xtsave, D.xtil, sizeof(double4_32a) * (size_t)M.nv, cudaMemcpyDeviceToDevice, s));
-        sim_status r = in3(x, D.x);
+        const double *dx = nullptr, *dt = nullptr;
+        sim_status r = on_device(x, stage, dx);
         if (r) return r;
-        if (xt) { r = in3(xt, D.xtil); if (r) return r; }
-        const int nb = (M.nv + 255) / 256;
-        k_set_mass_w<<<nb, 256, 0, s>>>(D.xtil, D.mass, M.nv);
-        refresh_ff();
-        k_reinit<R><<<nb, 256, 0, s>>>(D, 0);
-        force_rebuild();
-        zero_active();
-        zero_near64();
+        if (xt) { r = on_device(xt, stage + 3 * (size_t)M.nv, dt); if (r) return r; }
+        k_eval_in<R><<<(M.nv + 255) / 256, 256, 0, s>>>(D, dx, dt, xsave, xtsave);
         launch_bp();
         launch_grad(0);
-        k_copy_count<<<1, 1, 0, s>>>(dctrl);
         CK(cudaGetLastError());
         return SIM_OK;
     }
     sim_status eval_restore()
     {
-        CK(cudaMemcpyAsync(D.x, xsave, sizeof(double4_32a) * (size_t)M.nv, cudaMemcpyDeviceToDevice, s));
-        CK(cudaMemcpyAsync(D.xtil, xtsave, sizeof(double4_32a) * (size_t)M.nv, cudaMemcpyDeviceToDevice, s));
-        refresh_ff();
-        force_rebuild();
-        zero_active();
+        k_eval_out<R><<<(M.nv + 255) / 256, 256, 0, s>>>(D, xsave, xtsave);
+        CK(cudaGetLastError());
         return SIM_OK;
     }
 
@@ -391,9 +424,7 @@ public:
         if (!x || !xt) return fail(SIM_ERR_INVALID_ARG, "x and xtilde are required");
         sim_status r = eval_setup(x, xt);
         if (r) return r;
-        const int nb = (M.nv + 255) / 256;
-        if (g) { k_unpackR<R4><<<nb, 256, 0, s>>>(D.g[0], stage, M.nv); CK(cudaMemcpyAsync(g, stage, 24 * (size_t)M.nv, cudaMemcpyDefault, s)); CK(cudaStreamSynchronize(s)); }
-        if (d) { k_unpackR<R4><<<nb, 256, 0, s>>>(D.dg[0], stage, M.nv); CK(cudaMemcpyAsync(d, stage, 24 * (size_t)M.nv, cudaMemcpyDefault, s)); CK(cudaStreamSynchronize(s)); }
+        if (g || d) { r = out2(D.g[0], D.dg[0], g, d); if (r) return r; }
         eval_restore();
         return sync_and_check();
     }
@@ -712,12 +743,13 @@ public:
         if (r) return r;
         r = eval_setup(x, nullptr);
         if (r) return r;
-        CK(cudaMemcpyAsync(stage, v, 24 * (size_t)M.nv, cudaMemcpyDefault, s));
-        k_pack4<<<(M.nv + 255) / 256, 256, 0, s>>>(stage, adj_p, M.nv, 0);
-        launch_hvp(adj_p, adj_q);
-        r = out3(adj_q, out);
+        const double *dv = nullptr;
+        r = on_device(v, stage, dv);
         if (r) return r;
-        CK(cudaStreamSynchronize(s));
+        k_pack4<<<(M.nv + 255) / 256, 256, 0, s>>>(dv, adj_p, M.nv, 0);
+        launch_hvp(adj_p, adj_q);
+        r = out2(adj_q, adj_q, out, (double *)nullptr);
+        if (r) return r;
         eval_restore();
         return sync_and_check();
     }
@@ -1053,7 +1085,7 @@ private:
         const size_t npart = (size_t)std::max(std::max(5 * nvb, 4 * (ntb + nvb + npb_max + 4)), ntb + npb_max + 8);
         AL(D.part, npart);
         AL(D.trace, (size_t)TRACE_COLS * std::max(M.opt.iters, 1));
-        AL(stage, 3 * (size_t)nv);
+        AL(stage, 6 * (size_t)nv);
         AL(xsave, nv); AL(xtsave, nv); AL(psave, nv);
         // broad phase
         B.nv = nv; B.ns = M.ns; B.nf = M.nf; B.ne = M.ne;
@@ -1241,18 +1273,34 @@ private:
         cudaMemcpyAsync(&dctrl->rebuild, &one, sizeof one, cudaMemcpyHostToDevice, s);
         cudaMemcpyAsync(&dctrl->cell_bits, &zero, sizeof zero, cudaMemcpyHostToDevice, s);
     }
-    void zero_active()
-    {
-        static const int32_t zero = 0;
-        cudaMemcpyAsync(&dctrl->n_active, &zero, sizeof zero, cudaMemcpyHostToDevice, s);
-    }
-    void zero_near64()
-    {
-        static const int32_t zero = 0;
-        cudaMemcpyAsync(&dctrl->n_near64, &zero, sizeof zero, cudaMemcpyHostToDevice, s);
-    }
-
     void refresh_ff() { k_refresh_ff<R><<<(M.nv + 255) / 256, 256, 0, s>>>(D); }
+
+    // an input array where the device can read it: the caller's own buffer, or its copy in `buf`
+    sim_status on_device(const double *src, double *buf, const double *&out)
+    {
+        if (device_ptr(src)) { out = src; return SIM_OK; }
+        CK(cudaMemcpyAsync(buf, src, 24 * (size_t)M.nv, cudaMemcpyDefault, s));
+        out = buf;
+        return SIM_OK;
+    }
+    bool device_ptr(const void *p) const
+    {
+        cudaPointerAttributes at;
+        if (cudaPointerGetAttributes(&at, p) != cudaSuccess) { cudaGetLastError(); return false; }
+        return at.type == cudaMemoryTypeDevice && at.device == dev;
+    }
+    // two [n_verts][3] outputs (null = skip), written into the caller's device buffers or through the staging buffer;
+    // the caller synchronises
+    template <typename T> sim_status out2(const T *a, const T *b, double *oa, double *ob)
+    {
+        const size_t n3 = 3 * (size_t)M.nv;
+        double *da = !oa ? nullptr : device_ptr(oa) ? oa : stage, *db = !ob ? nullptr : device_ptr(ob) ? ob : stage + n3;
+        k_out2<T><<<(M.nv + 255) / 256, 256, 0, s>>>(a, b, da, db, M.nv);
+        CK(cudaGetLastError());
+        if (da && da != oa) CK(cudaMemcpyAsync(oa, da, 8 * n3, cudaMemcpyDefault, s));
+        if (db && db != ob) CK(cudaMemcpyAsync(ob, db, 8 * n3, cudaMemcpyDefault, s));
+        return SIM_OK;
+    }
 
     sim_status in3(const double *src, double4_32a *dst)
     {
