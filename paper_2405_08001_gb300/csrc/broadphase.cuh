@@ -5,8 +5,9 @@
 // dropped.  Since d changes by at most twice the largest vertex displacement, every pair with d < dhat is a
 // candidate until some vertex has moved r/2.
 //
-// Three hash tables of H buckets each: triangles [0, H) and edges [H, 2H), each registered in every cell its box
-// inflated by dhat + r covers, and surface points [2H, 3H), each in its own cell.  The five kernels run only when
+// Three hash tables of H buckets each: triangles [0, H), registered in every cell their box inflated by dhat + r covers,
+// and surface points [2H, 3H), each in its own cell, on one grid; and edges [H, 2H) on a finer one, registered by their box
+// inflated by half of dhat + r, so that the boxes of two edges within dhat + r of each other meet.  The five kernels run only when
 // Ctrl::rebuild is set (they return at once otherwise):
 //   bp_boxes  : inflated float boxes (rounded outwards), largest extent -> cell size, zero bucket counts, x_b = x
 //   bp_count  : entries per bucket (a box covers at most 2 cells per axis)
@@ -100,6 +101,15 @@ __device__ inline unsigned long long cell_key(int ix, int iy, int iz)
 struct CellGrid { float s, inv; };
 __device__ inline CellGrid grid_of(float s) { return {s, 1.0f / s}; }
 
+// The build's two grids from the largest extent of a box inflated by dhat + r (bp_box): the cells are that large for the
+// triangles and points, and smaller by dhat + r for the edges, whose boxes are inflated by half as much (with one grid and
+// one inflation for both, a cell held about 1.8 times the edges).  The margins keep the rounding of q / s from making a box
+// span three cells along an axis, as far from the origin on the finer grid (at least half as large) as on the other.
+struct Grids {
+    CellGrid t, e;
+    __device__ inline const CellGrid &of(bool edge) const { return edge ? e : t; }
+};
+
 __device__ inline __half2 u2h(unsigned int u) { __half2 h; memcpy(&h, &u, 4); return h; }
 __device__ inline unsigned int h2u(__half2 h) { unsigned int u; memcpy(&u, &h, 4); return u; }
 
@@ -128,9 +138,11 @@ __device__ inline bool cell_of(float q, const CellGrid &g, int &i)
     return true;
 }
 
-// hash cell size: the largest inflated box extent of the build, with a margin so that rounding in q / s can never
-// make a box span three cells along an axis
-__device__ inline float cell_size(const BPDev &B) { return __uint_as_float(B.ctrl->cell_bits) * 1.0001f; }
+__device__ inline Grids grids_of(const BPDev &B, float ext)
+{
+    return {grid_of(ext * 1.0001f), grid_of(__fsub_ru(ext, __double2float_rd(B.infl)) * 1.0002f)};
+}
+__device__ inline Grids grids_of(const BPDev &B) { return grids_of(B, __uint_as_float(B.ctrl->cell_bits)); }
 
 __device__ inline void box_of(const double4_32a *x, const int *v, int n, double infl, float4 &lo, float4 &hi)
 {
@@ -150,6 +162,21 @@ __device__ inline float4 rel_corner(const double4_32a &X, int ix, int iy, int iz
 {
     const double sd = s;
     return make_float4((float)(X.x - ix * sd), (float)(X.y - iy * sd), (float)(X.z - iz * sd), __int_as_float(w));
+}
+
+// Registration box of primitive j (triangles first, then edges), and its extent as the grids count it.
+__device__ inline float bp_box(const BPDev &B, int j)
+{
+    int v[3];
+    int nvp;
+    if (j < B.nf) { const int4 t = B.tri[j]; v[0] = t.x; v[1] = t.y; v[2] = t.z; nvp = 3; }
+    else { const int4 e = B.edge[j - B.nf]; v[0] = e.x; v[1] = e.y; nvp = 2; }
+    float4 lo, hi;
+    box_of(B.x, v, nvp, j < B.nf ? B.infl : 0.5 * B.infl, lo, hi);
+    B.blo[j] = lo;
+    B.bhi[j] = hi;
+    const float ext = fmaxf(__fsub_ru(hi.x, lo.x), fmaxf(__fsub_ru(hi.y, lo.y), __fsub_ru(hi.z, lo.z)));
+    return j < B.nf ? ext : __fadd_ru(ext, __double2float_ru(B.infl));
 }
 
 __device__ inline void prim_verts(const BPDev &B, int j, int v[3], int &nvp)
@@ -190,8 +217,9 @@ __device__ inline bool point_cell(const BPDev &B, int j, const CellGrid &g, int 
 // Writes primitive j's entries, one per cell of its registration box: the records of the cheap tests and the
 // vertices relative to the entry's cell corner (formed once in double against the box's lowest cell, then shifted
 // by whole cells in float).  slot_of(b) reserves a slot of bucket b; all slots are reserved before any is written.
-template <typename F> __device__ inline void fill_prim(const BPDev &B, int j, const CellGrid &g, F slot_of)
+template <typename F> __device__ inline void fill_prim(const BPDev &B, int j, const Grids &gs, F slot_of)
 {
+    const CellGrid g = gs.of(j >= B.nf);
     const float s = g.s;
     const float4 lo = __ldcg(B.blo + j), hi = __ldcg(B.bhi + j);
     int l[3], h[3];
@@ -330,16 +358,7 @@ static __global__ void __launch_bounds__(BP_B) bp_boxes(BPDev B)
             if (B.xbh) B.xbh[j] = B.xh[j];
         }
         if (j < B.nf + B.ne) {
-            int v[3];
-            int nvp;
-            if (j < B.nf) { const int4 t = B.tri[j]; v[0] = t.x; v[1] = t.y; v[2] = t.z; nvp = 3; }
-            else { const int4 e = B.edge[j - B.nf]; v[0] = e.x; v[1] = e.y; nvp = 2; }
-            float4 lo, hi;
-            box_of(B.x, v, nvp, B.infl, lo, hi);
-            B.blo[j] = lo;
-            B.bhi[j] = hi;
-            float ext = fmaxf(__fsub_ru(hi.x, lo.x), fmaxf(__fsub_ru(hi.y, lo.y), __fsub_ru(hi.z, lo.z)));
-            atomicMax(&B.ctrl->cell_bits, __float_as_uint(ext));
+            atomicMax(&B.ctrl->cell_bits, __float_as_uint(bp_box(B, j)));
         }
     }
 }
@@ -348,10 +367,11 @@ static __global__ void __launch_bounds__(BP_B) bp_boxes(BPDev B)
 static __global__ void __launch_bounds__(BP_B) bp_count(BPDev B)
 {
     if (!B.ctrl->rebuild) return;
-    const CellGrid g = grid_of(cell_size(B));
+    const Grids gs = grids_of(B);
+    const CellGrid &g = gs.t;
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < B.nf + B.ne)
-        for_cells(B, B.blo[j], B.bhi[j], g, [&](int i, int jj, int k) { atomicAdd(&B.cnt[prim_bucket(B, j, i, jj, k)], 1u); });
+        for_cells(B, B.blo[j], B.bhi[j], gs.of(j >= B.nf), [&](int i, int jj, int k) { atomicAdd(&B.cnt[prim_bucket(B, j, i, jj, k)], 1u); });
     if (j < B.ns) {
         int v, c[3];
         double4_32a X;
@@ -425,13 +445,13 @@ static __global__ void __launch_bounds__(BP_SCAN_T) bp_scan(BPDev B)
 static __global__ void __launch_bounds__(BP_B) bp_fill(BPDev B)
 {
     if (!B.ctrl->rebuild) return;
-    const CellGrid g = grid_of(cell_size(B));
+    const Grids g = grids_of(B);
     for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < 3 * B.H; b += gridDim.x * blockDim.x)
         B.goff[b] = B.boff[b / BP_SCAN_N] + B.off[b];
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     auto slot_of = [&](unsigned int b) { return B.boff[b / BP_SCAN_N] + B.off[b] + atomicAdd(&B.cnt[b], 1u); };
     if (j < B.nf + B.ne) fill_prim(B, j, g, slot_of);
-    if (j < B.ns) fill_point(B, j, g, slot_of);
+    if (j < B.ns) fill_point(B, j, g.t, slot_of);
 }
 
 __device__ inline bool is_excluded(const BPDev &B, unsigned long long key)
@@ -515,12 +535,11 @@ __device__ inline unsigned long long key_of(const uint4 &A) { return (unsigned l
 
 // exact tests of the first n queued pairs (all lanes call); both entries of a pair are in the same cell, so their
 // positions are relative to the same corner
-__device__ inline void bpq_exact(const BPDev &B, BPQWarp &W, int n, const CellGrid &g, int &nout)
+__device__ inline void bpq_exact(const BPDev &B, BPQWarp &W, int n, const Grids &gs, int &nout)
 {
     const int lane = threadIdx.x & 31;
-    const float thr = B.thr + 4e-6f * g.s;
     bool found = false;
-    float d = 0.0f;
+    float d = 0.0f, s = gs.e.s;   // the pair's cell size
     int4 cnd = make_int4(0, 0, 0, 0);
     if (lane < n) do {
         const uint2 pd = W.pend[lane];
@@ -530,6 +549,7 @@ __device__ inline void bpq_exact(const BPDev &B, BPQWarp &W, int n, const CellGr
         float cc[4];
         v3<float> tv;
         if (pd.y & BPQ_PT) {
+            s = gs.t.s;
             // row: triangle (Ar.z, Ar.w, v2), column: point Ac.z
             const float4 r2 = __ldcg(B.ev + 2 * (size_t)B.ecap + qr);
             const int t2 = (int)__ldcg(&B.erB[qr].w), v = (int)Ac.z;
@@ -539,7 +559,7 @@ __device__ inline void bpq_exact(const BPDev &B, BPQWarp &W, int n, const CellGr
                 if (B.tri[f].w == B.obj[v] && is_excluded(B, ((unsigned long long)jp << 31) | (unsigned long long)f)) break;
             }
             d = pt_coeffs<float>(f3sub(c0, r0), f3sub(r1, r0), f3sub(r2, r0), cc, tv);
-            if (!(d < thr)) break;
+            if (!(d < B.thr + 4e-6f * s)) break;
             found = true;
             cnd = make_int4(v, (int)Ar.z, (int)Ar.w, t2);
         } else {
@@ -554,7 +574,7 @@ __device__ inline void bpq_exact(const BPDev &B, BPQWarp &W, int n, const CellGr
                     break;
             }
             d = ee_coeffs<float>(f3sub(r0, c0), f3sub(r1, c0), f3sub(c1, c0), cc, tv);
-            if (!(d < thr)) break;
+            if (!(d < B.thr + 4e-6f * s)) break;
             found = true;
             cnd = make_int4(-1 - (int)Ar.z, (int)Ar.w, (int)Ac.z, (int)Ac.w);
         }
@@ -562,11 +582,11 @@ __device__ inline void bpq_exact(const BPDev &B, BPQWarp &W, int n, const CellGr
     // the bound: less the rounding of the positions (as thr), and less what the clamped cases overestimate for nearly
     // parallel edges or a sliver triangle (sin^2 of the angle under GeomEps<float>::par = 1e-5: at most L^2 par / (2 d), the
     // edges no longer than a cell's diagonal)
-    bpq_emit(B, W, nout, found, cnd, d - 4e-6f * g.s - 1.5e-5f * g.s * g.s / fmaxf(d, 1e-30f));
+    bpq_emit(B, W, nout, found, cnd, d - 4e-6f * s - 1.5e-5f * s * s / fmaxf(d, 1e-30f));
 }
 
 // queues the lanes' passing pairs (all lanes call); runs the exact tests once 32 are queued
-__device__ inline void bpq_push(const BPDev &B, BPQWarp &W, int &np, int &nout, const CellGrid &g, bool pass, unsigned int qr,
+__device__ inline void bpq_push(const BPDev &B, BPQWarp &W, int &np, int &nout, const Grids &g, bool pass, unsigned int qr,
                                 unsigned int qc)
 {
     const unsigned int m = __ballot_sync(0xffffffffu, pass);
@@ -589,7 +609,7 @@ __device__ inline void bpq_push(const BPDev &B, BPQWarp &W, int &np, int &nout, 
 
 // Work unit (b, r | c << 16) (all lanes call): rows 32 r .. 32 r + 31 of bucket b; columns 32 c .. 32 c + 31 of the
 // same bucket (edges, the pairs with the row before the column), or all entries of point bucket b + 2H (c = 0xffff).
-__device__ inline void bpq_unit(const BPDev &B, uint2 unit, const CellGrid &g, BPQWarp &W, int &np, int &nout)
+__device__ inline void bpq_unit(const BPDev &B, uint2 unit, const Grids &g, BPQWarp &W, int &np, int &nout)
 {
     const int lane = threadIdx.x & 31;
     const unsigned int b = unit.x, r = unit.y & 0xffffu, cc = unit.y >> 16;
@@ -637,7 +657,7 @@ __device__ inline void bpq_unit(const BPDev &B, uint2 unit, const CellGrid &g, B
 // Work units u = first, first + stride, ... (all lanes of the warp call; its batch area in W).  The candidate
 // threshold (bpq_exact) adds 4e-6 s to the exact-distance one: positions within a cell or two of a corner keep ~1e-7 s each
 // in float, and the differences and the distance formed from them stay well inside that.
-template <typename Next> __device__ inline void bpq_units(const BPDev &B, const CellGrid &g, BPQWarp &W, int first, Next next)
+template <typename Next> __device__ inline void bpq_units(const BPDev &B, const Grids &g, BPQWarp &W, int first, Next next)
 {
     const int nh = ((volatile Ctrl *)B.ctrl)->n_units_h, nl = ((volatile Ctrl *)B.ctrl)->n_units;
     const int nu = nh + nl;
@@ -659,7 +679,7 @@ static __global__ void __launch_bounds__(BP_B) bp_query(BPDev B)
     __shared__ BPQWarp W[BP_B / 32];
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
     int u = w;
-    bpq_units(B, grid_of(cell_size(B)), W[threadIdx.x >> 5], w, [&]() { return u += nw; });
+    bpq_units(B, grids_of(B), W[threadIdx.x >> 5], w, [&]() { return u += nw; });
 }
 
 } // namespace pncg

@@ -606,29 +606,19 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
             for (int j = tid; j < 3 * B.H; j += nthr) B.cnt[j] = 0u;
             for (int j = ov; j < vs.b1; j += PB) { B.xb[j] = ldcg4(B.x + j); if (B.xbh) B.xbh[j] = ldcg4(B.xh + j); }
             const Share ps = share_of(nprim);
-            for (int j = ps.b0 + (int)threadIdx.x; j < ps.b1; j += PB) {
-                int v[3];
-                int nvp;
-                if (j < B.nf) { const int4 t = B.tri[j]; v[0] = t.x; v[1] = t.y; v[2] = t.z; nvp = 3; }
-                else { const int4 e = B.edge[j - B.nf]; v[0] = e.x; v[1] = e.y; nvp = 2; }
-                float4 lo, hi;
-                box_of(B.x, v, nvp, B.infl, lo, hi);
-                B.blo[j] = lo;
-                B.bhi[j] = hi;
-                ext_max = fmaxf(ext_max, fmaxf(__fsub_ru(hi.x, lo.x), fmaxf(__fsub_ru(hi.y, lo.y), __fsub_ru(hi.z, lo.z))));
-            }
+            for (int j = ps.b0 + (int)threadIdx.x; j < ps.b1; j += PB) ext_max = fmaxf(ext_max, bp_box(B, j));
             const float ext = (float)grid_max<R, PB, CL>(R(ext_max), rb.max_region<PT, R>(), sh, br, c);
             if (lead) c->cell_bits = __float_as_uint(ext);
             st.mark(1);   // K_BP_BOXES
-            const CellGrid cg = grid_of(ext * 1.0001f);   // as cell_size() forms it from cell_bits
+            const Grids cg = grids_of(B, ext);
             br.phase = 2;   // K_BP_COUNT
             for (int j = ps.b0 + (int)threadIdx.x; j < ps.b1; j += PB)
-                for_cells(B, __ldcg(B.blo + j), __ldcg(B.bhi + j), cg, [&](int i, int jj, int kk) { atomicAdd(&B.cnt[prim_bucket(B, j, i, jj, kk)], 1u); });
+                for_cells(B, __ldcg(B.blo + j), __ldcg(B.bhi + j), cg.of(j >= B.nf), [&](int i, int jj, int kk) { atomicAdd(&B.cnt[prim_bucket(B, j, i, jj, kk)], 1u); });
             const Share ss = share_of(B.ns);
             for (int j = ss.b0 + (int)threadIdx.x; j < ss.b1; j += PB) {
                 int v, cc[3];
                 double4_32a X;
-                if (point_cell(B, j, cg, v, X, cc)) atomicAdd(&B.cnt[point_bucket(B, cc[0], cc[1], cc[2])], 1u);
+                if (point_cell(B, j, cg.t, v, X, cc)) atomicAdd(&B.cnt[point_bucket(B, cc[0], cc[1], cc[2])], 1u);
                 else atomicOr(&c->err, ERR_RANGE);
             }
             grid_barrier<CL>(br, c);
@@ -701,7 +691,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
             {
                 auto slot_of = [&](unsigned int b) { return choff[b >> cs] + __ldcg(B.off + b) + atomicAdd(&B.cnt[b], 1u); };
                 for (int j = ps.b0 + (int)threadIdx.x; j < ps.b1; j += PB) fill_prim(B, j, cg, slot_of);
-                for (int j = ss.b0 + (int)threadIdx.x; j < ss.b1; j += PB) fill_point(B, j, cg, slot_of);
+                for (int j = ss.b0 + (int)threadIdx.x; j < ss.b1; j += PB) fill_point(B, j, cg.t, slot_of);
             }
             grid_barrier<CL>(br, c);
             st.mark(4);   // K_BP_FILL
@@ -742,11 +732,10 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
                 // the block's share of the tets, then candidates 32 at a time per warp from a grid-wide cursor: the
                 // active ones (float-float geometry) cluster in the candidate order, and a fixed share per block
                 // left the blocks holding a contact patch 40 us behind the median one
-                const int nts = ts.b1 - ts.b0;
-                for (int q = threadIdx.x; q < nts; q += PB) {
+                for (int e = ts.b0 + (int)threadIdx.x; e < ts.b1; e += PB) {
                     TetIn<R> in;
-                    load_tet_in<R, CO>(D, ts.b0 + q, in);
-                    tet_grad<R, CO>(D, ts.b0 + q, par, in);
+                    load_tet_in<R, CO>(D, e, in);
+                    tet_grad<R, CO>(D, e, par, in);
                 }
                 if (lead) c->ticket[TK_PAIRS + ((k + 1) & 1)] = 0u;   // the next iteration's cursor
                 unsigned int *cur = &c->ticket[TK_PAIRS + (k & 1)];
