@@ -91,8 +91,6 @@ __device__ inline void tet_hvp_edges(const Dev<R> &D, int e, const int4 &tv, con
                 H[a][i] = dp[a][0] * S[0][i] + dp[a][1] * S[1][i] + dp[a][2] * S[2][i] + E[a][0] * Z[0][i] + E[a][1] * Z[1][i] +
                           E[a][2] * Z[2][i];
     } else {
-        R mu, lam;
-        tet_material<R>(D, e, mu, lam);
         const double4_32a a = D.td[e], b = D.td[n + e];
         const R k33 = __ldcg(D.tk + e), k3 = __ldcg(D.tk + n + e);
         R s[3][3], c[3][3];
@@ -104,7 +102,7 @@ __device__ inline void tet_hvp_edges(const Dev<R> &D, int e, const int4 &tv, con
 #pragma unroll
             for (int i = 0; i < 3; ++i) { g3 += c[r][i] * dp[r][i]; s[r][i] *= k3; }
         g3 *= k33;
-        const R M[3][3] = {{mu * a.x, mu * a.y, mu * a.z}, {mu * a.y, mu * a.w, mu * b.x}, {mu * a.z, mu * b.x, mu * b.y}};
+        const R M[3][3] = {{a.x, a.y, a.z}, {a.y, a.w, b.x}, {a.z, b.x, b.y}};
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             const int u = (i + 1) % 3, w = (i + 2) % 3;
@@ -362,14 +360,20 @@ __global__ void k_adj_out(Dev<R> D, const double4_32a *lam, const double *av, do
     }
 }
 // dE_e -= lambda_e . d g_e / d E_e: the tet's elastic gradient is linear in E_e (mu and lambda are), so its
-// derivative is the gradient evaluated with E_e = 1 (D carries mu and lambda of E = 1 and no per-tet scale)
+// derivative is the gradient evaluated with E_e = 1 (D carries mu and lambda of E = 1 and no per-tet scale; mu0 and es0
+// are the ones that the tets' constants were formed with)
 template <typename R, bool CO = false>
-__global__ void __launch_bounds__(EB) k_adj_youngs(Dev<R> D, const double4_32a *lam, double *dE)
+__global__ void __launch_bounds__(EB) k_adj_youngs(Dev<R> D, R mu0, const R *es0, const double4_32a *lam, double *dE)
 {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= D.nt) return;
     TetIn<R> in;
     load_tet_in<R, CO>(D, e, in);
+    if constexpr (!CO) {
+        const R f = D.mu / (es0 ? mu0 * es0[e] : mu0);
+#pragma unroll
+        for (int q = 0; q < 6; ++q) in.m[q] *= f;
+    }
     R gv[4][3], dv[4][3];
     if (!tet_grad_eval<R, CO>(D, in, gv, dv)) return;
     const int vid[4] = {in.tv.x, in.tv.y, in.tv.z, in.tv.w};

@@ -27,10 +27,10 @@ template <typename R> struct Dev {
     const float *G0;                   // FP32 corotated densities: [14][nt] rest metric Dm^T Dm of each tet as
                                        // float-float (six heads, six tails: entries 00 01 02 11 12 22), then det Dm
                                        // as float-float; null otherwise
-    const float4 *tc;                  // FP32 form: [5][nt] constants of each tet: the 14 values of G0, then h^2 V M
-                                       // (entries 00 01 02 11 12 22), M = Dm^-1 Dm^-T
-    const double4_32a *td;             // FP64 form: [2][nt] constants of each tet: h^2 V M (the six entries), det Dm^-1,
-                                       // h^2 V
+    const float4 *tc;                  // FP32 form: [5][nt] constants of each tet: the 14 values of G0, then mu h^2 V M
+                                       // (entries 00 01 02 11 12 22), M = Dm^-1 Dm^-T, mu the tet's own
+    const double4_32a *td;             // FP64 form: [2][nt] constants of each tet: mu h^2 V M (the six entries), det
+                                       // Dm^-1, h^2 V
     float4 *tS;                        // FP32 form: [4][nt] record of the last gradient pass per tet for tet_pHp_vec:
                                        // Z = Ds^-T (row-major), h^2 V Ds^-1 P Dm^-T (00 01 02 11 12 22), h^2 V k2
     R *tk;                             // the record's scalars: FP32 form [nt] h^2 V k1; FP64 form [2][nt]
@@ -411,7 +411,7 @@ template <typename R> __device__ inline void tet_material(const Dev<R> &D, int e
 template <typename R> struct TetIn {
     int4 tv;
     R w[3][3];      // FCR, ARAP: rows of D_m^-1
-    R m[6];         // h^2 V M, M = D_m^-1 D_m^-T, entries 00 01 02 11 12 22
+    R m[6];         // mu h^2 V M, M = D_m^-1 D_m^-T, entries 00 01 02 11 12 22
     R dw;           // FP64 form: det D_m^-1
     R hv, es;       // h^2 V, the Young's modulus scale
     float g0[14];   // FP32 form: rest metric entries 00 01 02 11 12 22, heads then tails; det Dm head, tail
@@ -706,10 +706,6 @@ __device__ inline bool tet_grad_edges(const Dev<R> &D, const TetIn<R> &in, R gv[
         }
         k33 *= in.hv;
         const float id = 1.0f / (J * in.g0[12]);   // 1 / det Ds
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int i = 0; i < 3; ++i) c[a][i] *= id;
         const float M[3][3] = {{in.m[0], in.m[1], in.m[2]}, {in.m[1], in.m[3], in.m[4]}, {in.m[2], in.m[4], in.m[5]}};
         const float hj = in.hv * mJ;
         float K[3][3];
@@ -720,12 +716,18 @@ __device__ inline bool tet_grad_edges(const Dev<R> &D, const TetIn<R> &in, R gv[
                 ffacc acc = ffacc::prod_f(G[i][0], M[0][b]);
 #pragma unroll
                 for (int j = 1; j < 3; ++j) acc.add_prod_f(G[i][j], M[j][b]);
-                K[i][b] = mu * acc.value() + (i == b ? hj : 0.0f);
+                K[i][b] = acc.value();
             }
+        // (the two parts are not added before they meet cof(Ds), and 1 / det Ds comes last: each sum and product
+        // rounded once more on the way cost a tenth of the gradient's accuracy)
 #pragma unroll
         for (int a = 0; a < 3; ++a)
 #pragma unroll
-            for (int i = 0; i < 3; ++i) H[a][i] = c[a][0] * K[0][i] + c[a][1] * K[1][i] + c[a][2] * K[2][i];
+            for (int i = 0; i < 3; ++i) H[a][i] = (hj * c[a][i] + c[a][0] * K[0][i] + c[a][1] * K[1][i] + c[a][2] * K[2][i]) * id;
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) c[a][i] *= id;
         if (e >= 0) {
             float S[3][3];
 #pragma unroll
@@ -759,15 +761,14 @@ __device__ inline bool tet_grad_edges(const Dev<R> &D, const TetIn<R> &in, R gv[
             D.tk[e] = k33;
             D.tk[(size_t)D.nt + e] = k3;
         }
-        const R M[3][3] = {{mu * in.m[0], mu * in.m[1], mu * in.m[2]}, {mu * in.m[1], mu * in.m[3], mu * in.m[4]},
-                           {mu * in.m[2], mu * in.m[4], mu * in.m[5]}};
+        const R M[3][3] = {{in.m[0], in.m[1], in.m[2]}, {in.m[1], in.m[3], in.m[4]}, {in.m[2], in.m[4], in.m[5]}};
 #pragma unroll
         for (int a = 0; a < 3; ++a)
 #pragma unroll
             for (int i = 0; i < 3; ++i) H[a][i] = s[a][0] * M[0][i] + s[a][1] * M[1][i] + s[a][2] * M[2][i] + k3 * c[a][i];
     }
-    const R m0 = mu * in.m[0], m1 = mu * in.m[3], m2 = mu * in.m[5];
-    const R ms = m0 + m1 + m2 + R(2) * mu * (in.m[1] + in.m[2] + in.m[4]);   // x_0's weights are minus the others' sum
+    const R m0 = in.m[0], m1 = in.m[3], m2 = in.m[5];
+    const R ms = m0 + m1 + m2 + R(2) * (in.m[1] + in.m[2] + in.m[4]);   // x_0's weights are minus the others' sum
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         gv[1][a] = H[a][0]; gv[2][a] = H[a][1]; gv[3][a] = H[a][2];
@@ -1420,8 +1421,6 @@ __device__ inline R tet_pHp_edges(const Dev<R> &D, int e, const int4 &tv, const 
                          2.0f * (q2.z * g[0][1] + q2.w * g[0][2] + q3.y * g[1][2]);
         return SD + k1 * tr * tr + q3.w * t2;
     } else {
-        R mu, lam;
-        tet_material<R>(D, e, mu, lam);
         const double4_32a a = D.td[e], b = D.td[n + e];
         const R k33 = __ldcg(D.tk + e), k3 = __ldcg(D.tk + n + e);
         R s[3][3], c[3][3];
@@ -1444,7 +1443,7 @@ __device__ inline R tet_pHp_edges(const Dev<R> &D, int e, const int4 &tv, const 
 #pragma unroll
             for (int j = i; j < 3; ++j) g[i][j] = dp[0][i] * dp[0][j] + dp[1][i] * dp[1][j] + dp[2][i] * dp[2][j];
         const R md = a.x * g[0][0] + a.w * g[1][1] + b.y * g[2][2] + R(2) * (a.y * g[0][1] + a.z * g[0][2] + b.x * g[1][2]);
-        return mu * md + k33 * (g3 * g3) + (R(2) * k3) * h3;
+        return md + k33 * (g3 * g3) + (R(2) * k3) * h3;
     }
 }
 

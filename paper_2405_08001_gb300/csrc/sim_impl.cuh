@@ -792,8 +792,8 @@ public:
             D1.mu = R(1.0 / (2.0 * (1.0 + M.nu)));
             D1.lam = R(M.nu / ((1.0 + M.nu) * (1.0 - 2.0 * M.nu)));
             D1.escale = nullptr;
-            if (corot) k_adj_youngs<R, true><<<(M.nt + EB - 1) / EB, EB, 0, s>>>(D1, adj_x, adj_dE);
-            else k_adj_youngs<R><<<(M.nt + EB - 1) / EB, EB, 0, s>>>(D1, adj_x, adj_dE);
+            if (corot) k_adj_youngs<R, true><<<(M.nt + EB - 1) / EB, EB, 0, s>>>(D1, D.mu, D.escale, adj_x, adj_dE);
+            else k_adj_youngs<R><<<(M.nt + EB - 1) / EB, EB, 0, s>>>(D1, D.mu, D.escale, adj_x, adj_dE);
             CK(cudaMemcpyAsync(dE, adj_dE, sizeof(double) * M.nt, cudaMemcpyDefault, s));
         }
         CK(cudaStreamSynchronize(s));
@@ -1189,14 +1189,15 @@ private:
         if ((st = up(B.edge, ed.data(), sizeof(int4) * M.ne))) return st;
         if ((st = up(B.obj, M.obj.data(), sizeof(int) * nv))) return st;
         if (B.excl && (st = up(B.excl, M.excl.data(), sizeof(unsigned long long) * M.excl.size()))) return st;
-        // h^2 V M with M = Dm^-1 Dm^-T (00 01 02 11 12 22) and det Dm^-1, in double
+        // mu h^2 V M with M = Dm^-1 Dm^-T (00 01 02 11 12 22) and det Dm^-1, in double
         auto weighted = [&](int e, double m[6], double &dw) {
+            const double f = M.hv[e] * M.mu * (M.escale.empty() ? 1.0 : M.escale[e]);
             double w[3][3];
             for (int r = 0; r < 3; ++r)
                 for (int c = 0; c < 3; ++c) w[r][c] = M.Dm[(size_t)(3 * r + c) * nt + e];
             int q = 0;
             for (int i = 0; i < 3; ++i)
-                for (int j = i; j < 3; ++j, ++q) m[q] = M.hv[e] * (w[i][0] * w[j][0] + w[i][1] * w[j][1] + w[i][2] * w[j][2]);
+                for (int j = i; j < 3; ++j, ++q) m[q] = f * (w[i][0] * w[j][0] + w[i][1] * w[j][1] + w[i][2] * w[j][2]);
             dw = w[0][0] * (w[1][1] * w[2][2] - w[1][2] * w[2][1]) - w[0][1] * (w[1][0] * w[2][2] - w[1][2] * w[2][0]) +
                  w[0][2] * (w[1][0] * w[2][1] - w[1][1] * w[2][0]);
         };
