@@ -61,11 +61,26 @@ template <typename R> __device__ inline void vadd(const Dev<R> &D, double4_32a *
 // of x_1..x_3 (x_0 gets minus their sum); p^T (H p) equals the p^T H p form of Sec. 3.1.  NH and SNH:
 //   FP64: Dp (2 Psi_2 h^2 V M) + h^2 V Psi_33 det(Dm^-1)^2 (cof(Ds) : Dp) cof(Ds) + h^2 V Psi_3 det(Dm^-1) d cof(Ds)[Dp], with
 // the scalars that the gradient pass at x left (tet_pHp_edges): about 135 FP64 operations where the form on F took 430
-// (82,944 tets: 70 us a pass).
+// (82,944 tets: 70 us a pass).  rec (or null): cof(Ds) and h^2 V Psi_3 det(Dm^-1) Ds kept by the solver, whose x stands
+// still (hvp_record): 99 operations.
 //   FP32: Dp (Dm^-1 S Dm^-T) + 2 (k1 tr(E) I + k2 E) Ds^-T, E = L + L^T, L = Dp Ds^-1, from the gradient pass's record: the
 // derivative of the quadratic form of tet_pHp_edges, in which the large terms of a rotating direction never meet.
+constexpr int HVP_REC = 5;   // double4 per tet of the record
+__device__ inline void hvp_record(const Dev<double> &D, int e, double4_32a *rec)
+{
+    const size_t n = (size_t)D.nt;
+    double s[3][3], c[3][3];
+    tet_ds<double>(D, D.tet[e], s);
+    cof3<double>(s, c);
+    const double k3 = __ldcg(D.tk + n + e);
+    rec[e] = make_double4_32a(c[0][0], c[0][1], c[0][2], c[1][0]);
+    rec[n + e] = make_double4_32a(c[1][1], c[1][2], c[2][0], c[2][1]);
+    rec[2 * n + e] = make_double4_32a(c[2][2], k3 * s[0][0], k3 * s[0][1], k3 * s[0][2]);
+    rec[3 * n + e] = make_double4_32a(k3 * s[1][0], k3 * s[1][1], k3 * s[1][2], k3 * s[2][0]);
+    rec[4 * n + e] = make_double4_32a(k3 * s[2][1], k3 * s[2][2], 0.0, 0.0);
+}
 template <typename R>
-__device__ inline void tet_hvp_edges(const Dev<R> &D, int e, const int4 &tv, const R dp[3][3], R H[3][3])
+__device__ inline void tet_hvp_edges(const Dev<R> &D, int e, const int4 &tv, const R dp[3][3], R H[3][3], const double4_32a *rec)
 {
     const size_t n = (size_t)D.nt;
     if constexpr (sizeof(R) == 4) {
@@ -92,16 +107,28 @@ __device__ inline void tet_hvp_edges(const Dev<R> &D, int e, const int4 &tv, con
                           E[a][2] * Z[2][i];
     } else {
         const double4_32a a = D.td[e], b = D.td[n + e];
-        const R k33 = __ldcg(D.tk + e), k3 = __ldcg(D.tk + n + e);
         R s[3][3], c[3][3];
-        tet_ds<R>(D, tv, s);
-        cof3<R>(s, c);
+        if (rec) {
+            const double4_32a q0 = rec[e], q1 = rec[n + e], q2 = rec[2 * n + e], q3 = rec[3 * n + e], q4 = rec[4 * n + e];
+            c[0][0] = q0.x; c[0][1] = q0.y; c[0][2] = q0.z; c[1][0] = q0.w; c[1][1] = q1.x; c[1][2] = q1.y;
+            c[2][0] = q1.z; c[2][1] = q1.w; c[2][2] = q2.x;
+            s[0][0] = q2.y; s[0][1] = q2.z; s[0][2] = q2.w; s[1][0] = q3.x; s[1][1] = q3.y; s[1][2] = q3.z;
+            s[2][0] = q3.w; s[2][1] = q4.x; s[2][2] = q4.y;
+        } else {
+            const R k3 = __ldcg(D.tk + n + e);
+            tet_ds<R>(D, tv, s);
+            cof3<R>(s, c);
+#pragma unroll
+            for (int r = 0; r < 3; ++r)
+#pragma unroll
+                for (int i = 0; i < 3; ++i) s[r][i] *= k3;
+        }
         R g3 = R(0);
 #pragma unroll
         for (int r = 0; r < 3; ++r)
 #pragma unroll
-            for (int i = 0; i < 3; ++i) { g3 += c[r][i] * dp[r][i]; s[r][i] *= k3; }
-        g3 *= k33;
+            for (int i = 0; i < 3; ++i) g3 += c[r][i] * dp[r][i];
+        g3 *= __ldcg(D.tk + e);
         const R M[3][3] = {{a.x, a.y, a.z}, {a.y, a.w, b.x}, {a.z, b.x, b.y}};
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
@@ -166,7 +193,7 @@ __device__ inline bool tet_hvp_rotated(const Dev<R> &D, int e, const int4 &tv, c
 
 // out += H_e v of tet e; returns v^T H_e v (in double)
 template <typename R, bool CO>
-__device__ inline double hvp_tet(const Dev<R> &D, int e, const double4_32a *v, double4_32a *out)
+__device__ inline double hvp_tet(const Dev<R> &D, int e, const double4_32a *v, double4_32a *out, const double4_32a *rec = nullptr)
 {
     const int4 tv = D.tet[e];
     const v3<R> V0 = vload(D, v, tv.x), V1 = vload(D, v, tv.y), V2 = vload(D, v, tv.z), V3 = vload(D, v, tv.w);
@@ -177,7 +204,7 @@ __device__ inline double hvp_tet(const Dev<R> &D, int e, const double4_32a *v, d
     if constexpr (CO) {
         if (!tet_hvp_rotated<R>(D, e, tv, dp, H)) return 0.0;
     } else {
-        tet_hvp_edges<R>(D, e, tv, dp, H);
+        tet_hvp_edges<R>(D, e, tv, dp, H, rec);
     }
     vadd<R>(D, out, tv.y, H[0][0], H[1][0], H[2][0]);
     vadd<R>(D, out, tv.z, H[0][1], H[1][1], H[2][1]);
@@ -243,6 +270,7 @@ constexpr int CG_STRIDE = 8;      // iterations between two looks at the residua
 enum { CG_RZ = 0, CG_BETA, CG_RR, CG_BB, CG_IT, CG_N };
 struct CgArgs {
     double4_32a *x, *r, *p, *q, *P;   // solution, residual (the right-hand side at iteration 0), direction, H p, Jacobi entries
+    double4_32a *rec;                 // FP64 form, NH and SNH: [HVP_REC][nt] (hvp_record); else null
     double *cg;                       // [CG_N] scalars carried between launches
     void *part;                       // reduction partials: 16 x gridDim.x doubles
     unsigned int *count;              // barrier arrival counter (zeroed before the launch)
@@ -272,7 +300,10 @@ __global__ void __launch_bounds__(CG_PB, CL ? 1 : 2) k_cg(Dev<R> D, CgArgs A)
         if (threadIdx.x == 0) { sh.o[0] = a; sh.o[1] = b; }
         __syncthreads();
     };
+    constexpr bool REC = sizeof(R) == 8 && !CO;
     if (A.it0 == 0) {
+        if constexpr (REC)
+            for (int e = ts.b0 + (int)threadIdx.x; e < ts.b1; e += CG_PB) hvp_record(D, e, A.rec);
         Acc<double> s[2];
         for (int i = vs.b0 + (int)threadIdx.x; i < vs.b1; i += CG_PB) {
             const typename V4<R>::T Dg = ldcg4(D.dg[par] + i);
@@ -308,7 +339,7 @@ __global__ void __launch_bounds__(CG_PB, CL ? 1 : 2) k_cg(Dev<R> D, CgArgs A)
         }
         grid_barrier<CL>(br, c);
         for (int j = threadIdx.x; j < nit; j += CG_PB)
-            pq[0].v += j < nts ? hvp_tet<R, CO>(D, ts.b0 + j, A.p, A.q) : hvp_pair<R>(D, as.b0 + j - nts, A.p, A.q);
+            pq[0].v += j < nts ? hvp_tet<R, CO>(D, ts.b0 + j, A.p, A.q, REC ? A.rec : nullptr) : hvp_pair<R>(D, as.b0 + j - nts, A.p, A.q);
         grid_reduce<double, CG_PB, CL, 1, false>(pq, 0.0, rb.sum_region<double>(), sh, br, c);
         share(threadIdx.x == 0 && sh.res[0] != 0.0 ? rz / sh.res[0] : 0.0, 0.0);
         const double al = sh.o[0];

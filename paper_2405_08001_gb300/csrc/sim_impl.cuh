@@ -690,6 +690,7 @@ public:
     {
         if (adj_p) return SIM_OK;
         const size_t n3 = 3 * (size_t)M.nv;
+        if (sizeof(R) == 8 && !corot) AL3(adj_rec, HVP_REC * (size_t)M.nt);
         AL3(adj_x, M.nv); AL3(adj_r, M.nv); AL3(adj_P, M.nv); AL3(adj_q, M.nv);
         AL3(adj_av, n3); AL3(adj_ax, n3); AL3(adj_cg, (size_t)CG_N);
         AL3(adj_dE, (size_t)M.nt);
@@ -714,7 +715,7 @@ public:
     // CG iterations it0 .. it1 - 1 at the positions of the last eval_setup
     cudaError_t launch_cg(int it0, int it1, double tol)
     {
-        CgArgs A{adj_x, adj_r, adj_p, adj_q, adj_P, adj_cg, cg_part, cg_count, it0, it1, tol * tol};
+        CgArgs A{adj_x, adj_r, adj_p, adj_q, adj_P, adj_rec, adj_cg, cg_part, cg_count, it0, it1, tol * tol};
         Dev<R> d = D;
         void *args[] = {(void *)&d, (void *)&A};
         if (cg_cluster > 0) {
@@ -848,7 +849,7 @@ private:
     unsigned long long *stamp_buf = nullptr;
     // differentiation: the solver's vectors, its launch and its scalars
     static constexpr int CG_LAUNCH = 1024;   // iterations per launch, a multiple of CG_STRIDE
-    double4_32a *adj_x = nullptr, *adj_r = nullptr, *adj_p = nullptr, *adj_q = nullptr, *adj_P = nullptr;
+    double4_32a *adj_x = nullptr, *adj_r = nullptr, *adj_p = nullptr, *adj_q = nullptr, *adj_P = nullptr, *adj_rec = nullptr;
     double *adj_av = nullptr, *adj_ax = nullptr, *adj_cg = nullptr, *adj_dE = nullptr, *cg_part = nullptr;
     unsigned int *cg_count = nullptr;
     int cg_cluster = 0, cg_grid = 1;
