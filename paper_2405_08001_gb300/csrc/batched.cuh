@@ -277,7 +277,7 @@ __device__ inline R batched_tail(const Dev<R> &D, Ctrl *c, PShared<R, PB, CL> &s
                         mp += G.w * np * np;
                     }
                     a2[1].add(mp);
-                    pmv = D.pnorm == 0 ? sqrt(px * px + py * py + pz * pz) : fmax(fabs(px), fmax(fabs(py), fabs(pz)));
+                    pmv = D.pnorm == 0 ? px * px + py * py + pz * pz : fmax(fabs(px), fmax(fabs(py), fabs(pz)));
                 }
                 D.pnext[i] = Pn;
             }
@@ -352,7 +352,8 @@ __device__ inline R batched_tail(const Dev<R> &D, Ctrl *c, PShared<R, PB, CL> &s
             const double gp = __ldcg(acc + (size_t)s * 8), pMp = __ldcg(acc + (size_t)s * 8 + 1);
             const bool empty = __ldcg(acc + (size_t)s * 8 + 2) == 0.0;
             const double pHp = __ldcg(acc + (size_t)s * 8 + 4) + __ldcg(acc + (size_t)s * 8 + 3) + pMp;
-            const double pmax = max_value<R>(__ldcg(mx + s));
+            const R pm = max_value<R>(__ldcg(mx + s));   // the squared length, or the component
+            const double pmax = D.pnorm == 0 ? (double)sqrt(pm) : (double)pm;
             const double au = pmax > 0.0 ? D.dhat / (2.0 * pmax) : 0.0;
             const double ab = -gp / pHp;
             double a;

@@ -8,6 +8,13 @@
 // needed).  In the FP32 form partial sums are carried as float-float (about 48 bits) on the FP32 pipes; in the FP64
 // form they are doubles.
 //
+// A double operation holds its scheduler's FP64 unit for 64 cycles, however few of the warp's lanes take part (measured:
+// division 450 cycles, square root 690, log 2,100), so the scalar work between two phases, which every thread waits for,
+// is kept short: in one thread per block, with no more than one division; what the next phase does not need (the reciprocal
+// for the next beta, Delta E, the eps rule, the records) is left to the last warp, which has the least to do there.
+// Measured with it against every scalar in thread 0 one after another: the 50-iteration step of the 2.5K-tet cube 767 ->
+// 711 us (FP32), the 25-iteration step of the twisted bar 985 -> 955 us (FP32), 5,450 -> 5,310 us (FP64, 50 iterations).
+//
 // One iteration has four grid barriers: gradient | beta dots | direction + p^T H p | update.  The direction
 // p_{k+1} = -P g + beta p_k is not a phase of its own: the beta pass stores P g per vertex, and the p^T H p pass
 // forms p_{k+1} of every vertex it touches from P g and p_k (one rounding order everywhere, so the values agree
@@ -141,7 +148,7 @@ template <> struct Acc<double> {
     __device__ inline void add(double x) { v += x; }
     __device__ inline void add_d(double x) { v += x; }
     __device__ inline void add(const Acc &o) { v += o.v; }
-    __device__ inline void add_ff(double h, double l) { v += h + l; }
+    __device__ inline void add_ff(double h, double) { v += h; }   // the FP64 form's terms have no tails
     __device__ inline Acc shfl_down(int o) const { Acc r; r.v = __shfl_down_sync(0xffffffffu, v, o); return r; }
     __device__ inline Acc shfl_up(int o) const { Acc r; r.v = __shfl_up_sync(0xffffffffu, v, o); return r; }
     __device__ inline double value() const { return v; }
@@ -234,8 +241,11 @@ template <typename R, int PB, bool CL> struct PShared {
     // cluster form: every block's partials; consecutive reductions alternate between the halves (RedBufs)
     unsigned long long cp[2][NQ + 1][CL ? CLUSTER_MAX : 1];
     double res[NQ + 1];   // reduced results: sums, then the max
-    double o[4];          // scalars computed by thread 0 and broadcast to the block
-    int oi[2];
+    double o[3];          // scalars computed by thread 0 and broadcast to the block: beta, g^T P g, alpha
+    double ab;            // -g.p / p^T H p
+    double ig, e0;        // kept by the last warp: 1 / g^T P g of this iteration (0 below 1e-300), Delta E_0
+    int oi[2];            // restarted, capped
+    int cv;               // kept by the last warp: the eps rule fired
     int fi;
     uint32_t fe;
 };
@@ -268,8 +278,10 @@ template <typename P> struct PartDst {
     int half;
 };
 
+// nq <= N: the sums in use; rows: the warps that have anything to add (the others' values are zero)
 template <typename R, int PB, bool CL, int N, bool MX>
-__device__ inline void block_publish(Acc<R> (&a)[N], R mx, const PartDst<typename PartT<R>::T> &dst, PShared<R, PB, CL> &sh)
+__device__ inline void block_publish(Acc<R> (&a)[N], R mx, const PartDst<typename PartT<R>::T> &dst, PShared<R, PB, CL> &sh,
+                                     int nq = N, int rows = PB / 32)
 {
     typename PartT<R>::T *part = dst.g;
     static_assert(N <= NQ && N + (MX ? 1 : 0) <= PB / 32, "one warp per quantity");
@@ -278,17 +290,15 @@ __device__ inline void block_publish(Acc<R> (&a)[N], R mx, const PartDst<typenam
     for (int q = 0; q < N; ++q) sh.t[q][threadIdx.x] = a[q];
     if (MX) sh.mx[threadIdx.x] = mx;
     __syncthreads();
-    if (warp < N) {
+    if (warp < nq) {
         Acc<R> s = sh.t[warp][lane];
-#pragma unroll
-        for (int j = 1; j < PB / 32; ++j) s.add(sh.t[warp][lane + 32 * j]);
+        for (int j = 1; j < rows; ++j) s.add(sh.t[warp][lane + 32 * j]);
         for (int o = 16; o > 0; o >>= 1) s.add(s.shfl_down(o));
         if constexpr (CL) peer_publish<R, PB, CL>(s, warp, dst.half, sh);
         else if (lane == 0) put_part(part + warp * gridDim.x + blockIdx.x, s);
     } else if (MX && warp == N) {
         R m = sh.mx[lane];
-#pragma unroll
-        for (int j = 1; j < PB / 32; ++j) m = fmax(m, sh.mx[lane + 32 * j]);
+        for (int j = 1; j < rows; ++j) m = fmax(m, sh.mx[lane + 32 * j]);
         for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
         Acc<R> b;
         b.add(m);
@@ -301,8 +311,11 @@ __device__ inline void block_publish(Acc<R> (&a)[N], R mx, const PartDst<typenam
 // L2), then the block reduces them transposed like block_publish (warp q sums quantity q, warp N takes the max, in
 // block order within each lane's stride); the results land in sh.res (sums in double), and thread 0 reads the
 // fetched scalars.  Every block computes bitwise the same results.  Ends with a CTA barrier.
-template <typename R, int PB, bool CL, int N, bool MX>
-__device__ inline void grid_collect(const PartDst<typename PartT<R>::T> &dst, PShared<R, PB, CL> &sh, const Fetch *f)
+// nq as in block_publish; post(max) runs in the thread that has it, before the results are handed on.
+struct NoPost { template <typename R> __device__ inline void operator()(R) const {} };
+template <typename R, int PB, bool CL, int N, bool MX, typename Post = NoPost>
+__device__ inline void grid_collect(const PartDst<typename PartT<R>::T> &dst, PShared<R, PB, CL> &sh, const Fetch *f, int nq = N,
+                                    Post post = Post())
 {
     const typename PartT<R>::T *part = dst.g;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -313,7 +326,7 @@ __device__ inline void grid_collect(const PartDst<typename PartT<R>::T> &dst, PS
             if (f->pi) sh.fi = (volatile const int &)*f->pi;
             if (f->pe) sh.fe = (volatile const uint32_t &)*f->pe;
         }
-        if (warp < N + (MX ? 1 : 0)) {
+        if (warp < nq || (MX && warp == N)) {
             Acc<R> s;
             if (lane < G) acc_from(sh.cp[dst.half][warp][lane], s);
             if (warp < N) {
@@ -322,7 +335,7 @@ __device__ inline void grid_collect(const PartDst<typename PartT<R>::T> &dst, PS
             } else {
                 R m = s.head();
                 for (int o = CLUSTER_MAX / 2; o > 0; o >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
-                if (lane == 0) sh.res[N] = (double)m;
+                if (lane == 0) { sh.res[N] = (double)m; post(m); }
             }
         }
         __syncthreads();
@@ -339,12 +352,14 @@ __device__ inline void grid_collect(const PartDst<typename PartT<R>::T> &dst, PS
         const int b = threadIdx.x + j * PB;
         if (b < G) {
 #pragma unroll
-            for (int q = 0; q < N; ++q) get_part(part + q * G + b, v[q][j]);
+            for (int q = 0; q < N; ++q)
+                if (q < nq) get_part(part + q * G + b, v[q][j]);
             if (MX) { Acc<R> w; get_part(part + N * G + b, w); m = fmax(m, w.head()); }
         }
     }
 #pragma unroll
     for (int q = 0; q < N; ++q) {
+        if (q >= nq) break;
         Acc<R> s = v[q][0];
 #pragma unroll
         for (int j = 1; j < (MAXG + PB - 1) / PB; ++j) s.add(v[q][j]);
@@ -352,7 +367,7 @@ __device__ inline void grid_collect(const PartDst<typename PartT<R>::T> &dst, PS
     }
     if (MX) sh.mx[threadIdx.x] = m;
     __syncthreads();
-    if (warp < N) {
+    if (warp < nq) {
         Acc<R> s = sh.t[warp][lane];
 #pragma unroll
         for (int j = 1; j < PB / 32; ++j) s.add(sh.t[warp][lane + 32 * j]);
@@ -363,7 +378,7 @@ __device__ inline void grid_collect(const PartDst<typename PartT<R>::T> &dst, PS
 #pragma unroll
         for (int j = 1; j < PB / 32; ++j) mm = fmax(mm, sh.mx[lane + 32 * j]);
         for (int o = 16; o > 0; o >>= 1) mm = fmax(mm, __shfl_down_sync(0xffffffffu, mm, o));
-        if (lane == 0) sh.res[N] = (double)mm;
+        if (lane == 0) { sh.res[N] = (double)mm; post(mm); }
     }
     __syncthreads();
 }
@@ -371,11 +386,11 @@ __device__ inline void grid_collect(const PartDst<typename PartT<R>::T> &dst, PS
 // Grid-wide sums of N accumulators (and a max): block part, barrier, collection into sh.res.
 template <typename R, int PB, bool CL, int N, bool MX>
 __device__ inline void grid_reduce(Acc<R> (&a)[N], R mx, const PartDst<typename PartT<R>::T> &part, PShared<R, PB, CL> &sh,
-                                   Bar &br, Ctrl *c, const Fetch *f = nullptr)
+                                   Bar &br, Ctrl *c, const Fetch *f = nullptr, int nq = N, int rows = PB / 32)
 {
-    block_publish<R, PB, CL, N, MX>(a, mx, part, sh);
+    block_publish<R, PB, CL, N, MX>(a, mx, part, sh, nq, rows);
     grid_barrier<CL>(br, c);
-    grid_collect<R, PB, CL, N, MX>(part, sh, f);
+    grid_collect<R, PB, CL, N, MX>(part, sh, f, nq);
 }
 
 // Grid-wide max of non-negative values of the element type (exact); one grid barrier.  `part` holds gridDim.x
@@ -429,6 +444,9 @@ __device__ inline R grid_max(R v, const PartDst<R> &dst, PShared<R, PB, CL> &sh,
     __syncthreads();
     return r;
 }
+
+// isfinite without the FP64 unit
+__device__ inline bool finite_bits(double a) { return (__double2hiint(a) & 0x7ff00000) != 0x7ff00000; }
 
 // a value that thread 0 reads once for the whole block
 __device__ inline int block_read(const int *p, int *sh)
@@ -540,9 +558,14 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
     // state every block reads before anyone can change it
     int rebuild = (volatile int &)c->rebuild;
     const bool skip_step = (volatile uint32_t &)c->err != 0u;
-    double gPg_prev = (volatile double &)c->gPg_prev;
-    double dE0 = (volatile double &)c->dE0;
-    int converged = (volatile int &)c->converged;
+    const bool keeper = threadIdx.x == PB - 32;   // the last warp's first thread keeps ig, e0 and cv
+    if (keeper) {
+        const double g = (volatile double &)c->gPg_prev;
+        sh.ig = g > 1e-300 ? 1.0 / g : 0.0;
+        sh.e0 = (volatile double &)c->dE0;
+        sh.cv = (volatile int &)c->converged;
+    }
+    const int vrows = min(PB / 32, max(1, (vs.b1 - vs.b0 + 31) >> 5));   // warps with vertices
     int npt = (volatile int &)c->n_cand[0], ncand = npt + (volatile int &)c->n_cand[1];
     R disp_max = R(-1);   // largest squared displacement of a vertex since the last candidate build; < 0: not known
     const double disp_lim = 0.5 * D.pad_r * (1.0 - 1e-4);
@@ -581,9 +604,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
         const R m = grid_max<R, PB, CL>(md, rb.max_region<PT, R>(), sh, br, c);
         disp_max = m;
         if (!skip_step && (double)m >= disp_lim * disp_lim) rebuild = 1;
-        gPg_prev = 0.0;
-        dE0 = 0.0;
-        converged = 0;
+        if (keeper) { sh.e0 = 0.0; sh.cv = 0; }
         if (lead) {
             c->k = 0; c->n_rebuilds = 0; c->n_capped = 0; c->n_near64 = 0; c->iters_done = 0; c->converged = 0;
             c->n_active = 0; c->dE0 = 0.0; c->gPg_prev = 0.0;
@@ -820,12 +841,12 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
         }
         // ------------------------------------------------------------ a4: beta (and P g for the direction)
         double beta = 0.0;
-        int restarted = 0;
         int na;
         R4 oG, oDg, oPG, oP0;   // this thread's own vertex (i == ov), kept for the direction pass
         br.phase = 8;   // K_DOTS
         {
             Acc<R> s5[5];
+            const int nq = D.beta_rule == 0 ? 3 : 5;   // the sums that the rule uses
             // complete since the gradient pass's barrier, as are its error bits: read here, where the vertices' loads
             // hide the round trip
             if (threadIdx.x == 0) { sh.fi = (volatile const int &)c->n_active; sh.fe = (volatile const uint32_t &)c->err; }
@@ -838,7 +859,8 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
                     R th[5], tl[5], pg[3];
                     beta_terms<R>(gv, dv, g0, p0, Dg.w, D.beta_rule, th, tl, pg);
 #pragma unroll
-                    for (int q = 0; q < 5; ++q) s5[q].add_ff(th[q], tl[q]);
+                    for (int q = 0; q < 5; ++q)
+                        if (q < nq) s5[q].add_ff(th[q], tl[q]);
                     PG = mk4<R>(pg[0], pg[1], pg[2], R(0));
                 } else if (P0.x != R(0) || P0.y != R(0) || P0.z != R(0)) {
                     D.p[i] = PG;   // a kinematic vertex never moves along p
@@ -847,7 +869,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
                 D.pg[i] = PG;
                 if (i == ov) { oG = G; oDg = Dg; oPG = PG; oP0 = P0; }
             }
-            grid_reduce<R, PB, CL, 5, false>(s5, R(0), rb.sum_region<PT>(), sh, br, c);
+            grid_reduce<R, PB, CL, 5, false>(s5, R(0), rb.sum_region<PT>(), sh, br, c, nullptr, nq, vrows);
             st.mark(8);   // K_DOTS
             // beta and the restart test: scalar FP64 work, done by one thread and broadcast
             if (threadIdx.x == 0) {
@@ -856,24 +878,25 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
                 int rs = 0;
                 if (D.beta_rule == 0) {
                     gPg = t[1];
-                    if (k > 0) { bt = gPg_prev > 0.0 ? t[0] / gPg_prev : 0.0; if (bt < 0.0) bt = 0.0; }
+                    if (k > 0) { bt = t[0] * sh.ig; if (bt < 0.0) bt = 0.0; }
                     gp_new = -gPg + bt * t[2];
                 } else {
                     gPg = t[4];
-                    if (k > 0) bt = fabs(t[2]) < 1e-30 ? 0.0 : t[0] / t[2] - (t[1] / t[2]) * (t[3] / t[2]);
+                    if (k > 0 && !(fabs(t[2]) < 1e-30)) {
+                        const double iy = 1.0 / t[2];
+                        bt = t[0] * iy - (t[1] * iy) * (t[3] * iy);
+                    }
                     gp_new = -gPg + bt * t[3];
                 }
                 if (gp_new >= 0.0 && bt != 0.0) { bt = 0.0; rs = 1; }
                 sh.o[0] = bt;
                 sh.o[1] = gPg;
                 sh.oi[0] = rs;
-                sh.oi[1] = sh.fi;
             }
             __syncthreads();
             beta = sh.o[0];
-            gPg_prev = sh.o[1];
-            restarted = sh.oi[0];
-            na = sh.oi[1];
+            na = sh.fi;
+            if (keeper) sh.ig = sh.o[1] > 1e-300 ? 1.0 / sh.o[1] : 0.0;
         }
         // ------------------------------------------------------------ a5-a7: direction, p^T H p and the step
         double alpha;
@@ -901,7 +924,8 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
                         mp += G.w * np * np;
                     }
                     s3[1].add(mp);
-                    const R pn = D.pnorm == 0 ? sqrt(px * px + py * py + pz * pz) : fmax(fabs(px), fmax(fabs(py), fabs(pz)));
+                    // squared lengths (the largest is the largest length's square; one root at the end), or components
+                    const R pn = D.pnorm == 0 ? px * px + py * py + pz * pz : fmax(fabs(px), fmax(fabs(py), fabs(pz)));
                     pm = fmax(pm, pn);
                 }
                 D.pnext[i] = Pn;
@@ -928,7 +952,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
             Fetch f;
             f.pe = CL ? nullptr : &c->err;   // with bounded waits: a time-out since then counts too
             const PartDst<PT> part = rb.sum_region<PT>();
-            block_publish<R, PB, CL, 3, true>(s3, pm, part, sh);
+            block_publish<R, PB, CL, 3, true>(s3, pm, part, sh, 3, max(vrows, min(PB / 32, (nit + 31) >> 5)));
             grid_barrier<CL>(br, c);
             // the update's loads of this thread's own vertex go out before the partial collection and the step rule
             if (ov < vs.b1) {
@@ -937,59 +961,64 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
                 if constexpr (sizeof(R) == 8) uXT = ldcg4(D.xtil + ov);
                 uXB = disp_ref<R>(D, ov);
             }
-            grid_collect<R, PB, CL, 3, true>(part, sh, &f);
+            // the cap dhat / (2 max |p|), by the thread that has the maximum, beside the sums
+            grid_collect<R, PB, CL, 3, true>(part, sh, &f, 3, [&](R m) {
+                const double pmax = D.pnorm == 0 ? (double)sqrt(m) : (double)m;
+                sh.res[3] = pmax;
+                sh.res[4] = pmax > 0.0 ? D.dhat / (2.0 * pmax) : 0.0;
+            });
             st.mark(10);  // K_PHP (direction included)
-            // the step rule (Sec. 4.3) and the predicted decrease: scalar FP64 work, done by one thread
+            // the step rule (Sec. 4.3): scalar FP64 work, done by one thread
             if (threadIdx.x == 0) {
-                const double gp = sh.res[0], pHp_vert = sh.res[1], pmax = sh.res[3];
-                uint32_t err = sh.fe;
-                const double pHp = sh.res[2] + pHp_vert;
-                const double au = pmax > 0.0 ? D.dhat / (2.0 * pmax) : 0.0;
+                const double gp = sh.res[0], au = sh.res[4], pHp = sh.res[2] + sh.res[1];
                 const double ab = -gp / pHp;
-                double a;
-                int capped;
-                if (!(pHp > 0.0) || !isfinite(ab)) { a = au; capped = 1; }
-                else if (ab < au) { a = ab; capped = 0; }
-                else { a = au; capped = 1; }
-                const double dE = -a * gp - 0.5 * a * a * pHp;
-                if (!isfinite(a) || !isfinite(gp)) {
+                const int cap = !(pHp > 0.0) || !finite_bits(ab) || !(ab < au);
+                const double a = cap ? au : ab;
+                if (!finite_bits(a) || !finite_bits(gp)) {
                     if (lead) flag_error(c, ERR_NONFINITE);
-                    err |= ERR_NONFINITE;
-                    a = 0.0;
+                    sh.fe |= ERR_NONFINITE;
                 }
-                if (err != 0u || converged) a = 0.0;
-                if (lead) {
-                    c->beta = beta; c->restarted = restarted; c->gp = gp; c->pmax = pmax; c->pHp_vert = pHp_vert;
-                    c->pHp = pHp; c->alpha_bar = ab; c->alpha_up = au; c->alpha = a; c->dE = dE; c->capped = capped;
+                sh.oi[1] = cap;
+                sh.ab = ab;
+                sh.o[2] = sh.fe != 0u || sh.cv ? 0.0 : a;
+            }
+            __syncthreads();
+            alpha = sh.o[2];
+            // the predicted decrease, the eps rule (Sec. 4.4) and the records: for the next iteration and the host
+            if (keeper && (blockIdx.x == 0 || D.eps > 0.0)) {
+                const double gp = sh.res[0], pHp_vert = sh.res[1], pmax = sh.res[3], au = sh.res[4], ab = sh.ab;
+                const double pHp = sh.res[2] + pHp_vert;
+                const int capped = sh.oi[1];
+                const bool ok = sh.fe == 0u, was = sh.cv != 0;
+                const double a = capped ? au : ab;
+                const double dE = -a * gp - 0.5 * a * a * pHp;
+                double e0 = sh.e0;
+                int cv = was;
+                if (!was && ok) {
+                    if (k == 0) e0 = dE;
+                    if (D.eps > 0.0 && dE < D.eps * e0) cv = 1;
+                }
+                sh.e0 = e0;
+                sh.cv = cv;
+                if (blockIdx.x == 0) {
+                    c->beta = beta; c->restarted = sh.oi[0]; c->gp = gp; c->pmax = pmax; c->pHp_vert = pHp_vert;
+                    c->pHp = pHp; c->alpha_bar = ab; c->alpha_up = au; c->alpha = alpha; c->dE = dE; c->capped = capped;
                     c->n_active_last = na;
-                    c->gPg_prev = gPg_prev;
-                    if (!converged && err == 0u) {
-                        if (k == 0) c->dE0 = dE;
+                    c->gPg_prev = sh.o[1];
+                    if (!was && ok) {
                         c->n_capped += capped;
                         c->iters_done = k + 1;
                         if (D.trace && k < D.iters) {
                             double *tr = D.trace + (size_t)k * TRACE_COLS;
-                            tr[0] = beta; tr[1] = gp; tr[2] = pHp; tr[3] = pmax; tr[4] = a; tr[5] = dE;
+                            tr[0] = beta; tr[1] = gp; tr[2] = pHp; tr[3] = pmax; tr[4] = alpha; tr[5] = dE;
                             tr[6] = na; tr[7] = capped;
                         }
                     }
                     c->k = k + 1;
+                    c->dE0 = e0;
+                    c->converged = cv;
                 }
-                int cv = converged;
-                double e0 = dE0;
-                if (!cv && err == 0u) {
-                    if (k == 0) e0 = dE;
-                    if (D.eps > 0.0 && dE < D.eps * e0) cv = 1;
-                }
-                if (lead) { c->dE0 = e0; c->converged = cv; }
-                sh.o[2] = a;
-                sh.o[3] = e0;
-                sh.oi[0] = cv;
             }
-            __syncthreads();
-            alpha = sh.o[2];
-            dE0 = sh.o[3];
-            converged = sh.oi[0];
         }
         // ------------------------------------------------------------ a8: update
         br.phase = 11;   // K_UPDATE
