@@ -753,7 +753,7 @@ __device__ inline bool tet_grad_edges(const Dev<R> &D, const TetIn<R> &in, R gv[
             k3 = hd * (lam * (J - R(1)) - mu);
             k33 = hd * in.dw * lam;
         } else {
-            const R L = log(J), ij = R(1) / J, q = hd * ij;
+            const R L = log_tab(J), ij = R(1) / J, q = hd * ij;
             k3 = q * (lam * L - mu);
             k33 = q * (in.dw * ij) * (mu + lam * (R(1) - L));
         }

@@ -17,6 +17,8 @@
 // corot_terms), so that the stress keeps its relative accuracy near a rotation.
 #pragma once
 
+#include "log_tab.cuh"
+
 namespace pncg {
 
 enum { MAT_NH = 0, MAT_SNH = 1, MAT_FCR = 2, MAT_ARAP = 3 };
@@ -42,7 +44,7 @@ template <typename R> __host__ __device__ inline MatTerms<R> mat_terms(int model
         t.Psi3 = model == MAT_FCR ? lam * (J - R(1)) : R(0);
         t.Psi33 = model == MAT_FCR ? lam : R(0);
     } else {
-        const R L = log(J);
+        const R L = log_pos(J);
         t.c2 = mu;
         t.Psi3 = (lam * L - mu) / J;
         t.Psi33 = (mu + lam * (R(1) - L)) / (J * J);
