@@ -5,6 +5,8 @@
 
 #include <math.h>
 
+#include "log_tab.cuh"
+
 namespace pncg {
 
 template <typename R> struct v3 { R x, y, z; };
@@ -24,6 +26,20 @@ template <> struct GeomEps<float> { static constexpr double par = 1e-5; };
 template <typename R> __host__ __device__ inline v3<R> operator-(v3<R> a, v3<R> b) { return mkv(a.x - b.x, a.y - b.y, a.z - b.z); }
 template <typename R> __host__ __device__ inline v3<R> operator+(v3<R> a, v3<R> b) { return mkv(a.x + b.x, a.y + b.y, a.z + b.z); }
 template <typename R> __host__ __device__ inline v3<R> operator*(R s, v3<R> a) { return mkv(s * a.x, s * a.y, s * a.z); }
+// a / d for several a.  F64, here and below: the FP64 form's pairs, where a division holds the FP64 unit as long as seven
+// other operations (log1p as long as 33), so one reciprocal serves several quotients: the 20-iteration step of two small
+// blocks in contact 888 -> 828 us.  In the FP32 form the same only costs registers (the stack's gradient pass 106 -> 111 us;
+// in its rare evaluations in double, the batched step 2.5 %).
+template <bool F64, typename R> struct Quot {
+    R d;
+    __host__ __device__ explicit Quot(R d_) : d(d_) {}
+    __host__ __device__ R operator()(R a) const { return a / d; }
+};
+template <typename R> struct Quot<true, R> {
+    R i;
+    __host__ __device__ explicit Quot(R d) : i(R(1) / d) {}
+    __host__ __device__ R operator()(R a) const { return a * i; }
+};
 template <typename R> __host__ __device__ inline R dot(v3<R> a, v3<R> b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
 template <typename R> __host__ __device__ inline v3<R> cross(v3<R> a, v3<R> b)
 {
@@ -47,13 +63,14 @@ template <typename R> __host__ __device__ inline R seg_closest(v3<R> q, v3<R> a,
 // Minimises |x0 - (a x1 + b x2 + g x3)| over the simplex (Eq. PT); c = (1, -a, -b, -g).  Interior projection from
 // the 2x2 normal equations when it lies in the triangle, else the closest of the three clamped edges in the
 // order (x1,x2), (x2,x3), (x3,x1) (first wins ties).  Returns d and writes c and t = x0 - x_b.
-template <typename R> __host__ __device__ inline R pt_coeffs(v3<R> r, v3<R> e1, v3<R> e2, R c[4], v3<R> &t)
+template <typename R, bool F64 = false> __host__ __device__ inline R pt_coeffs(v3<R> r, v3<R> e1, v3<R> e2, R c[4], v3<R> &t)
 {
     R a = dot(e1, e1), b = dot(e1, e2), cq = dot(e2, e2);
     R det = a * cq - b * b;
     if (det > R(GeomEps<R>::par) * a * cq) {
         R p = dot(r, e1), q = dot(r, e2);
-        R be = (cq * p - b * q) / det, ga = (a * q - b * p) / det;
+        const Quot<F64, R> by(det);
+        R be = by(cq * p - b * q), ga = by(a * q - b * p);
         if (be >= R(0) && ga >= R(0) && be + ga <= R(1)) {
             c[0] = R(1); c[1] = -(R(1) - be - ga); c[2] = -be; c[3] = -ga;
             t = r - (be * e1 + ga * e2);
@@ -80,14 +97,15 @@ template <typename R> __host__ __device__ inline R pt_coeffs(v3<R> r, v3<R> e1, 
 // Minimises |(1-s) x0 + s x1 - ((1-u) x2 + u x3)| over [0,1]^2 (Eq. EE); c = (1-s, s, -(1-u), -u).  Interior
 // solution of the 2x2 system when it lies in the square (and the edges are not parallel), else the closest of the
 // four clamped cases s = 0, s = 1, u = 0, u = 1 in that order.  Returns d and writes c and t.
-template <typename R> __host__ __device__ inline R ee_coeffs(v3<R> r, v3<R> a1, v3<R> e1, R c[4], v3<R> &t)
+template <typename R, bool F64 = false> __host__ __device__ inline R ee_coeffs(v3<R> r, v3<R> a1, v3<R> e1, R c[4], v3<R> &t)
 {
     v3<R> e0 = a1 - r;
     R a = dot(e0, e0), b = dot(e0, e1), cq = dot(e1, e1), dd = dot(e0, r), ee = dot(e1, r);
     R det = a * cq - b * b;
     bool done = false;
     if (det > R(GeomEps<R>::par) * a * cq) {
-        R s = (b * ee - cq * dd) / det, u = (a * ee - b * dd) / det;
+        const Quot<F64, R> by(det);
+        R s = by(b * ee - cq * dd), u = by(a * ee - b * dd);
         if (s >= R(0) && s <= R(1) && u >= R(0) && u <= R(1)) {
             c[0] = R(1) - s; c[1] = s; c[2] = -(R(1) - u); c[3] = -u;
             done = true;
@@ -118,15 +136,22 @@ template <typename R> __host__ __device__ inline v3<R> rel(double ax, double ay,
 // b(d) = -(d - dhat)^2 log(d/dhat) for 0 < d < dhat: first and second derivative in d, from d and r = d - dhat.
 // log(d/dhat) is formed as log1p(r/dhat), which keeps its relative accuracy as d -> dhat when r is accurate (the
 // FP32 form passes r from its float-float distance: a float d has lost r's low bits near the cut-off).
-template <typename R> __host__ __device__ inline void barrier_d12r(R d, R r, R dhat, R &b1, R &b2)
+template <typename R, bool F64 = false> __host__ __device__ inline void barrier_d12r(R d, R r, R dhat, R &b1, R &b2)
 {
-    const R L = log1p(r / dhat);
-    b1 = R(-2) * r * L - r * r / d;
-    b2 = R(-2) * L - R(4) * r / d + (r * r) / (d * d);
+    if constexpr (F64) {
+        const R L = log1p_tab(r / dhat);
+        const R q = r / d;
+        b1 = -r * (R(2) * L + q);
+        b2 = R(-2) * L - R(4) * q + q * q;
+    } else {
+        const R L = log1p(r / dhat);
+        b1 = R(-2) * r * L - r * r / d;
+        b2 = R(-2) * L - R(4) * r / d + (r * r) / (d * d);
+    }
 }
-template <typename R> __host__ __device__ inline void barrier_d12(R d, R dhat, R &b1, R &b2)
+template <typename R, bool F64 = false> __host__ __device__ inline void barrier_d12(R d, R dhat, R &b1, R &b2)
 {
-    barrier_d12r<R>(d, d - dhat, dhat, b1, b2);
+    barrier_d12r<R, F64>(d, d - dhat, dhat, b1, b2);
 }
 
 template <typename R> __host__ __device__ inline R barrier_b(R d, R dhat)

@@ -177,7 +177,7 @@ __device__ inline void init_vertex(const Dev<R> &D, int i, const double4_32a &X,
                 flag_error(D.ctrl, ERR_PENETRATION);
             } else {
                 double b1, b2;
-                barrier_d12<double>(d, D.dhat, b1, b2);
+                barrier_d12<double, true>(d, D.dhat, b1, b2);
                 double k1 = D.kappa * b1, k2 = D.kappa * b2;
                 gx += k1 * D.pn[0]; gy += k1 * D.pn[1]; gz += k1 * D.pn[2];
                 dx += k2 * D.pn[0] * D.pn[0]; dy += k2 * D.pn[1] * D.pn[1]; dz += k2 * D.pn[2] * D.pn[2];
@@ -1022,16 +1022,16 @@ __device__ inline void tet_grad_chunk(const Dev<R> &D, int ch, int par, R *sacc)
 
 // Closest-point coefficients and t of a candidate.  Relative coordinates come from the double positions (FP64
 // form, and the FP32 form's double re-evaluation) or from the float-float positions (FP32 form).
-template <typename R>
+template <typename R, bool F64 = false>
 __device__ inline R pair_geom(bool ee, const double4_32a &X0, const double4_32a &X1, const double4_32a &X2, const double4_32a &X3,
                               R c[4], v3<R> &t)
 {
     if (!ee) {
-        return pt_coeffs<R>(rel<R>(X0.x, X0.y, X0.z, X1.x, X1.y, X1.z), rel<R>(X2.x, X2.y, X2.z, X1.x, X1.y, X1.z),
-                            rel<R>(X3.x, X3.y, X3.z, X1.x, X1.y, X1.z), c, t);
+        return pt_coeffs<R, F64>(rel<R>(X0.x, X0.y, X0.z, X1.x, X1.y, X1.z), rel<R>(X2.x, X2.y, X2.z, X1.x, X1.y, X1.z),
+                                 rel<R>(X3.x, X3.y, X3.z, X1.x, X1.y, X1.z), c, t);
     }
-    return ee_coeffs<R>(rel<R>(X0.x, X0.y, X0.z, X2.x, X2.y, X2.z), rel<R>(X1.x, X1.y, X1.z, X2.x, X2.y, X2.z),
-                        rel<R>(X3.x, X3.y, X3.z, X2.x, X2.y, X2.z), c, t);
+    return ee_coeffs<R, F64>(rel<R>(X0.x, X0.y, X0.z, X2.x, X2.y, X2.z), rel<R>(X1.x, X1.y, X1.z, X2.x, X2.y, X2.z),
+                             rel<R>(X3.x, X3.y, X3.z, X2.x, X2.y, X2.z), c, t);
 }
 
 __device__ inline v3<float> rel_ff(const Dev<float> &D, int a, int b)
@@ -1101,7 +1101,7 @@ __device__ inline void pair_grad(const Dev<R> &D, const int4 &q, int par, bool n
             r = __fadd_rn(rf.h, rf.l);
         }
     } else {
-        d = pair_geom<R>(ee, ldcg4(D.x + v.x), ldcg4(D.x + v.y), ldcg4(D.x + v.z), ldcg4(D.x + v.w), c, t);
+        d = pair_geom<R, true>(ee, ldcg4(D.x + v.x), ldcg4(D.x + v.y), ldcg4(D.x + v.z), ldcg4(D.x + v.w), c, t);
         if (!(d < R(D.dhat))) return;
         r = d - R(D.dhat);
     }
@@ -1123,9 +1123,15 @@ __device__ inline void pair_grad(const Dev<R> &D, const int4 &q, int par, bool n
     } else {
         if (!(d > R(0))) { flag_error(D.ctrl, ERR_PENETRATION); return; }
         R b1, b2;
-        barrier_d12r<R>(d, r, R(D.dhat), b1, b2);
-        A = R(D.kappa) * (b2 / (d * d) - b1 / (d * d * d));
-        B = R(D.kappa) * b1 / d;
+        barrier_d12r<R, sizeof(R) == 8>(d, r, R(D.dhat), b1, b2);
+        if constexpr (sizeof(R) == 8) {   // one division (Quot says why)
+            const R i = R(1) / d, bd = b1 * i;
+            A = R(D.kappa) * ((b2 - bd) * i * i);
+            B = R(D.kappa) * bd;
+        } else {
+            A = R(D.kappa) * (b2 / (d * d) - b1 / (d * d * d));
+            B = R(D.kappa) * b1 / d;
+        }
     }
     const int slot = atomicAdd(&D.ctrl->n_active, 1);
     if (slot >= D.cand_cap) { flag_error(D.ctrl, ERR_CAPACITY); return; }
