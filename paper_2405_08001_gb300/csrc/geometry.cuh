@@ -46,6 +46,21 @@ template <typename R> __host__ __device__ inline v3<R> cross(v3<R> a, v3<R> b)
     return mkv(a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x);
 }
 
+// cof(S) : D and cof(D) : S (the first and half the second derivative of det at S along D; columns s_i, d_i).  Written as
+// triple products with s_1 or d_1, the two share w = s_2 x d_0 - s_0 x d_2: 36 operations, where the two cofactor matrices
+// take 54.
+template <typename R> __host__ __device__ inline void det_forms(const R (&s)[3][3], const R (&d)[3][3], R &g, R &h)
+{
+    g = h = R(0);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const int y = (a + 1) % 3, z = (a + 2) % 3;
+        const R w = (s[y][2] * d[z][0] - s[z][2] * d[y][0]) - (s[y][0] * d[z][2] - s[z][0] * d[y][2]);
+        g += s[a][1] * w + d[a][1] * (s[y][2] * s[z][0] - s[z][2] * s[y][0]);
+        h += d[a][1] * w + s[a][1] * (d[y][2] * d[z][0] - d[z][2] * d[y][0]);
+    }
+}
+
 // Closest point of segment [a, b] to q: returns the squared distance and the parameter u in [0, 1].
 template <typename R> __host__ __device__ inline R seg_closest(v3<R> q, v3<R> a, v3<R> b, R &u)
 {

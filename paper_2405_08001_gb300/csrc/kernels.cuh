@@ -1405,14 +1405,14 @@ __global__ void __launch_bounds__(VB) k_dir(Dev<R> D, int par)
 // tr(S)), at the x of the last gradient pass, whose record it reads.  On the direction's edge vectors Dp (columns p_i -
 // p_0) for NH and SNH, so that neither D_m^-1 nor dF is needed:
 //   FP64: 2 Psi_2 h^2 V M : Dp^T Dp + h^2 V Psi_33 det(Dm^-1)^2 (cof(Ds) : Dp)^2 + h^2 V Psi_3 det(Dm^-1) 2 cof(Dp) : Ds
-// (about 115 FP64 operations; on F and with the scalars formed anew it took 330).
+// (97 FP64 operations; on F and with the scalars formed anew it took 330: 54 -> 31 us an iteration for 98K tets).
 //   FP32: the second derivative of Psi written in C = F^T F, S : dF^T dF + k1 (tr C^-1 E)^2 + k2 tr(C^-1 E C^-1 E), E =
 // dF^T F + F^T dF.  With L = dF F^-1 = Dp Ds^-1, tr C^-1 E = tr(L + L^T) and tr(C^-1 E C^-1 E) = |L + L^T|^2, and S : dF^T dF =
 // (Dm^-1 S Dm^-T) : Dp^T Dp.  A direction that rotates the tet cancels inside L + L^T, so the large terms mu |dF|^2 and
 // Psi_3 d2det(F)[dF, dF] of the I2/I3 form, which cancel for it, never meet in float.  The record (68 bytes: Ds^-T, the
 // weighted stress, k1, k2) stands in for the positions' eight gathers and D_m^-1.
 template <typename R>
-__device__ inline R tet_pHp_edges(const Dev<R> &D, int e, const int4 &tv, const R dp[3][3])
+__device__ inline R tet_pHp_edges(const Dev<R> &D, int e, const int4 &tv, const R (&dp)[3][3])
 {
     const size_t n = (size_t)D.nt;
     if constexpr (sizeof(R) == 4) {
@@ -1440,20 +1440,9 @@ __device__ inline R tet_pHp_edges(const Dev<R> &D, int e, const int4 &tv, const 
     } else {
         const double4_32a a = D.td[e], b = D.td[n + e];
         const R k33 = __ldcg(D.tk + e), k3 = __ldcg(D.tk + n + e);
-        R s[3][3], c[3][3];
+        R s[3][3], g3, h3;
         tet_ds<R>(D, tv, s);
-        cof3<R>(s, c);
-        R g3 = R(0);
-#pragma unroll
-        for (int r = 0; r < 3; ++r)
-#pragma unroll
-            for (int i = 0; i < 3; ++i) g3 += c[r][i] * dp[r][i];
-        cof3<R>(dp, c);
-        R h3 = R(0);
-#pragma unroll
-        for (int r = 0; r < 3; ++r)
-#pragma unroll
-            for (int i = 0; i < 3; ++i) h3 += c[r][i] * s[r][i];
+        det_forms<R>(s, dp, g3, h3);
         R g[3][3];
 #pragma unroll
         for (int i = 0; i < 3; ++i)

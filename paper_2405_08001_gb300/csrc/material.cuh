@@ -58,7 +58,7 @@ __host__ __device__ inline double mat_psi(int model, double mu, double lam, doub
     if (model == MAT_SNH) return 0.5 * mu * (I2 - 3.0) - mu * (J - 1.0) + 0.5 * lam * (J - 1.0) * (J - 1.0);
     if (model == MAT_FCR) return mu * (I2 - 2.0 * I1 + 3.0) + 0.5 * lam * (J - 1.0) * (J - 1.0);
     if (model == MAT_ARAP) return mu * (I2 - 2.0 * I1 + 3.0);
-    const double L = log(J);
+    const double L = log_pos(J);
     return 0.5 * mu * (I2 - 3.0) - mu * L + 0.5 * lam * L * L;
 }
 

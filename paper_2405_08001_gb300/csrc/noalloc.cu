@@ -9,6 +9,7 @@
 
 #include "../../include/pncg.h"
 #include "common.cuh"
+#include "geometry.cuh"
 
 namespace {
 
@@ -54,21 +55,13 @@ __device__ inline Mat3 cofactors(const Mat3 &d)
     }
     return c;
 }
-__device__ inline double inner(const Mat3 &a, const Mat3 &b)
-{
-    double s = 0.0;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) s += a.m[i][j] * b.m[i][j];
-    return s;
-}
 
 // p^T M p + h^2 sum_e V_e [mu |dF|^2 + Psi_33 (cof F : dF)^2 + Psi_3 d2det(F)[dF, dF]] in double precision, one
 // thread per tet (and per vertex for the inertia term).  With the edge vectors of the rest, current and direction
 // values Dm, Ds, Dp (columns): J = det Ds / det Dm, cof F : dF = cof(Ds) : Dp / det Dm, d2det(F)[dF, dF] = 2 cof(Dp) : Ds /
 // det Dm and dF = Dp cof(Dm)^T / det Dm, so that neither D_m^-1 nor F is formed.  Bound by FP64 issue (1.65 lanes per
-// clock and SM): about 205 operations a tet with two divisions, where the form on F took about 400 with nine.
+// clock and SM): about 175 operations a tet with two divisions, where the form on F took about 400 with nine.  998,250 tets:
+// on F 768 us, on edge vectors 411, with det_forms and log_tab 354.
 __global__ void __launch_bounds__(NA_THREADS) k_pHp_noalloc(NoAllocScratch *scr, int nv, int nt, const double *x,
                                                              const double *p, const double *X, const int *tets,
                                                              const double *mass, double mu, double lam, double h2,
@@ -84,12 +77,16 @@ __global__ void __launch_bounds__(NA_THREADS) k_pHp_noalloc(NoAllocScratch *scr,
     if (i < nt) {
         const int v[4] = {tets[4 * i], tets[4 * i + 1], tets[4 * i + 2], tets[4 * i + 3]};
         const Mat3 A = edges(X, v), Ds = edges(x, v), Dp = edges(p, v);
-        const Mat3 ca = cofactors(A), cs = cofactors(Ds);
+        const Mat3 ca = cofactors(A);
         const double det = A.m[0][0] * ca.m[0][0] + A.m[1][0] * ca.m[1][0] + A.m[2][0] * ca.m[2][0];
-        const double ds = Ds.m[0][0] * cs.m[0][0] + Ds.m[1][0] * cs.m[1][0] + Ds.m[2][0] * cs.m[2][0];
+        double ds = 0.0, g3, h3;
+#pragma unroll
+        for (int a = 0; a < 3; ++a)     // s_1 . (s_2 x s_0), whose cross product det_forms has too
+            ds += Ds.m[a][1] * (Ds.m[(a + 1) % 3][2] * Ds.m[(a + 2) % 3][0] - Ds.m[(a + 2) % 3][2] * Ds.m[(a + 1) % 3][0]);
+        pncg::det_forms<double>(Ds.m, Dp.m, g3, h3);
         if (ds > 0.0 && det > 0.0) {
             const double idet = 1.0 / det, J = ds * idet, iJ = det / ds;
-            const double L = log(J);
+            const double L = pncg::log_tab(J);
             const double Psi3 = (lam * L - mu) * iJ, Psi33 = (mu + lam * (1.0 - L)) * iJ * iJ;
             double n2 = 0.0;
 #pragma unroll
@@ -99,8 +96,8 @@ __global__ void __launch_bounds__(NA_THREADS) k_pHp_noalloc(NoAllocScratch *scr,
                     const double f = Dp.m[a][0] * ca.m[b][0] + Dp.m[a][1] * ca.m[b][1] + Dp.m[a][2] * ca.m[b][2];
                     n2 += f * f;
                 }
-            const double g3 = inner(cs, Dp) * idet;
-            const double h3 = 2.0 * inner(cofactors(Dp), Ds) * idet;
+            g3 *= idet;
+            h3 *= 2.0 * idet;
             s[0] += h2 * (det * (1.0 / 6.0)) * (mu * (n2 * idet * idet) + Psi33 * (g3 * g3) + Psi3 * h3);
         } else {
             s[0] = nan("");     // an inverted current tet, or a rest tet of non-positive volume
