@@ -135,9 +135,11 @@ typedef struct {
                              above (a tet or pair spanning groups adds to each group's p^T H p with the other groups'
                              entries of p zero).  Group g = 2 object + (1 for the collision part); a group without
                              vertices takes no step.  Works without scene_of_vert (one object, two groups). */
-    int32_t block_shape;  /* block shape of the persistent form: 0 (default) = 256 threads x 2 blocks per SM, or for a
-                             small mesh (8,192 tets in the FP32 form, 4,096 in FP64; not with SIM_SCATTER_BLOCK) one
-                             thread-block cluster of 16 blocks of 256 threads;
+    int32_t block_shape;  /* block shape of the persistent form: 0 (default) = by the mesh's size: one thread-block
+                             cluster of 16 blocks of 256 threads up to 8,192 tets in the FP32 form, 4,096 in FP64; 256
+                             threads x 1 block per SM up to three tets a thread (several scenes or objects: one); else,
+                             with SIM_SCATTER_BLOCK, and for FCR and ARAP in the FP32 form above the cluster's size,
+                             256 threads x 2 blocks per SM;
                              1 = 512 x 1, 2 = 256 x 3, 3 = 256 x 1, 4 = 384 x 1 (the compiler fits the registers
                              per thread to the shape: 128, 128, 85, 255, 168); -1 = autotuned: from the second time
                              step on, each shape runs two time steps (interleaved), timed on the GPU (those steps

@@ -902,6 +902,19 @@ private:
     // tets 0.40 / 0.54, 6,000 0.46 / 0.55, 10,368 0.55 / 0.55, 16,464 0.68 / 0.55; FP64 (whose arithmetic needs the SMs)
     // 1,296 tets 0.66 / 0.91, 3,072 0.80 / 0.95, 6,000 1.19 / 0.98.
     bool small_mesh() const { return M.nt <= (sizeof(R) == 4 ? 8192 : 4096); }
+    // Where one block of 256 threads an SM, with 255 registers, is faster than two with 128 (the default shape's): half the
+    // blocks at the barriers and no spills, against twice the warps to hide latency.  A round is one tet a thread of the
+    // smaller grid.  Measured, time of a step with two / with one, 152 SMs (a round is 38,912 tets):
+    //   up to one round    FP32 10K tets 1.11, 29K 1.12; FP64 4.4K 1.17, 35K 1.13; batched FP32 19K 1.08, FP64 1.07
+    //   up to three        FP32 48K 1.03, 83K 1.07, 98K 1.05; FP64 56K 1.06, 83K 1.06, 98K 1.05 (FCR, ARAP 1.07), but FP64
+    //                      41K to 48K 0.98: a second round that hardly any thread has costs FP64 as much as a full one
+    //   above              FP32 132K 0.99, 236K 0.94; FP64 0.98 to 1.05, in no order; batched 52K 0.99 (FP32), 1.01 (FP64)
+    bool one_block() const
+    {
+        const long long nt = M.nt, round = (long long)PSHAPE_PB[3] * nsm;
+        if (M.nseg > 1) return nt <= round;
+        return nt <= 3 * round && !(sizeof(R) == 8 && nt > round && 3 * nt <= 4 * round);
+    }
     void set_shape(int sh)
     {
         shape = sh;
@@ -937,6 +950,8 @@ private:
             if (corot) CK((cluster_blocks<R, true>(&cluster)));
             else CK((cluster_blocks<R, false>(&cluster)));
         }
+        // (the autotuner's shape 0 stays two blocks an SM; the corotated FP32 kernel has that shape only)
+        if (M.opt.block_shape == 0 && !block_scatter && cluster <= 0 && one_block() && shape_grid[3] > 0) shape = 3;
         set_shape(shape);
         unsigned int *sync;
         AL2(sync, 32);                    // the barrier arrival counter on a 128-byte line of its own

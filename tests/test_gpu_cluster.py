@@ -10,8 +10,12 @@ from test_gpu_parity import B, CHECKED, O, TOL, lockstep  # noqa: F401  (B and O
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("prec,cells,blocks", [(1, (1, 1, 1), 1), (1, (9, 11, 13), 1), (1, (11, 11, 12), 2),
-                                               (0, (1, 2, 1), 1), (0, (8, 8, 10), 1), (0, (8, 9, 10), 2)])
+# ... and of the next rule: one block of 256 threads an SM up to three rounds of 256 x 152 tets, two above (and in FP64 just
+# above one round)
+@pytest.mark.parametrize("prec,cells,blocks", [(1, (1, 1, 1), 1), (1, (9, 11, 13), 1), (1, (11, 11, 12), 1),
+                                               (0, (1, 2, 1), 1), (0, (8, 8, 10), 1), (0, (8, 9, 10), 1),
+                                               (0, (23, 12, 23), 1), (0, (19, 18, 19), 2), (0, (21, 20, 21), 1),
+                                               (1, (27, 26, 27), 1), (1, (27, 27, 27), 2)])
 def test_both_sides_of_the_size_rule(B, O, prec, cells, blocks):  # noqa: F811
     sc = S.cube_drop(n=max(cells), cells=cells, drop=0.0)
     sc.x0 = sc.x0 + np.array([0.0, 0.0, 0.6 * sc.dhat])
@@ -32,11 +36,12 @@ def test_both_sides_of_the_size_rule(B, O, prec, cells, blocks):  # noqa: F811
                                      (lambda: S.batched(3, n_min=2, n_max=4), {})])
 def test_same_step_as_the_whole_grid(B, make, kw):  # noqa: F811
     """One FP64 step in the cluster form and in 256 x 1 blocks on the whole grid (the same arithmetic, another order of
-    the sums): equal within the growth of rounding over the step's iterations, about 1e3 to 1e5 on these scenes."""
+    the sums): equal within the growth of rounding over the step's iterations, up to 1e4 over four on these scenes (1e7 over
+    eight)."""
     sc = make()
     out = []
     for shape in (0, 3):
-        sim = B.Sim(sc, precision=0, block_shape=shape, iters=8, **kw)
+        sim = B.Sim(sc, precision=0, block_shape=shape, iters=4, **kw)
         sim.step(1, sc.targets(0))
         out.append(sim.state()[0])
         sim.close()
