@@ -694,14 +694,16 @@ public:
         AL3(adj_x, M.nv); AL3(adj_r, M.nv); AL3(adj_P, M.nv); AL3(adj_q, M.nv);
         AL3(adj_av, n3); AL3(adj_ax, n3); AL3(adj_cg, (size_t)CG_N);
         AL3(adj_dE, (size_t)M.nt);
-        // the solver's launch: one cluster on a small mesh, else as many resident blocks as the device takes together
+        // the solver's launch: one cluster on a small mesh, else one or two blocks an SM by the time step's rule (us an
+        // iteration with two / one: FP64 8K tets 18.1 / 16.3, 25K 21.5 / 19.7, 83K 39.2 / 37.8; FP32, whose sums are double
+        // here too, 25K 16.6 / 15.0, 41K 18.9 / 19.2, 83K 25.4 / 22.6)
         int coop = 0, per_sm = 0;
         CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
         cg_cluster = 0;
         if (small_mesh()) CK(largest_cluster(cg_kernel(true), &cg_cluster));
         cg_coop = cg_cluster == 0 && coop;
         if (cg_coop) CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cg_kernel(false), CG_PB, 0));
-        cg_grid = cg_cluster > 0 ? cg_cluster : std::max(1, std::min(std::min(per_sm, 2) * nsm, MAXG));
+        cg_grid = cg_cluster > 0 ? cg_cluster : std::max(1, std::min(std::min(per_sm, one_block(true) ? 1 : 2) * nsm, MAXG));
         AL3(cg_part, 16 * (size_t)cg_grid);
         AL3(cg_count, 32);
         AL3(adj_p, M.nv);
@@ -909,11 +911,11 @@ private:
     //   up to three        FP32 48K 1.03, 83K 1.07, 98K 1.05; FP64 56K 1.06, 83K 1.06, 98K 1.05 (FCR, ARAP 1.07), but FP64
     //                      41K to 48K 0.98: a second round that hardly any thread has costs FP64 as much as a full one
     //   above              FP32 132K 0.99, 236K 0.94; FP64 0.98 to 1.05, in no order; batched 52K 0.99 (FP32), 1.01 (FP64)
-    bool one_block() const
+    bool one_block(bool f64 = sizeof(R) == 8) const
     {
         const long long nt = M.nt, round = (long long)PSHAPE_PB[3] * nsm;
         if (M.nseg > 1) return nt <= round;
-        return nt <= 3 * round && !(sizeof(R) == 8 && nt > round && 3 * nt <= 4 * round);
+        return nt <= 3 * round && !(f64 && nt > round && 3 * nt <= 4 * round);
     }
     void set_shape(int sh)
     {
