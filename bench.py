@@ -142,25 +142,27 @@ def algorithmic_bytes(kernel: str, prec: int, sizes: dict, n_cand: int, n_active
 
     Vertex state: x (double4, 32 B) and, in the FP32 form, its float-float copy (2 x float4); accumulators g, diag
     and the directions are 4-vectors of the element type (16 B float, 32 B double).  Per tet: 4 indices (16 B),
-    D_m^-1 (9 values), h^2 V (1 value) and, in the FP32 form, the float-float rest metric (12 floats).  Candidates:
+    the constants on edge vectors (FP32: 20 floats, the float-float rest metric and mu h^2 V Dm^-1 Dm^-T; FP64: 8
+    doubles; the p^T H p pass reads them in the FP64 form, the record instead in FP32).  Candidates:
     int4 (16 B); active pairs (64 B float form, 112 B double form) written by the gradient pass and read by p^T H p.
-    The persistent step stores P g in the beta pass and forms the direction inside the p^T H p pass.  The FP32
-    form's per-tet p^T H p record (64 B written by the gradient pass, read by the p^T H p pass) is an
-    implementation choice for accuracy, not a quantity of the method, and is not counted."""
+    The persistent step stores P g in the beta pass and forms the direction inside the p^T H p pass.  The per-tet
+    p^T H p record (68 B in FP32, 16 B in FP64: written by the gradient pass, read by the p^T H p pass) is counted in
+    both."""
     T, V = sizes["n_tets"], sizes["n_verts"]
     r = 4 if prec == 1 else 8
     v4 = 4 * r
-    tet = 16 + 10 * r
+    rec = 68 if prec == 1 else 16
     act = 64 if prec == 1 else 112
     xpos = 32                                # gathered positions per vertex (ff pair, or double4)
     if kernel == "k_grad":
-        return T * (tet + (48 if prec == 1 else 0)) + V * (xpos + 4 * v4) + n_cand * 16 + n_active * act
+        return T * (16 + (80 if prec == 1 else 64) + rec) + V * (xpos + 4 * v4) + n_cand * 16 + n_active * act
     if kernel == "k_dots":
         return V * (5 if persistent else 4) * v4
     if kernel == "k_dir":
         return V * 4 * v4
     if kernel == "k_pHp":
-        return T * tet + V * (xpos + (5 if persistent else 1) * v4) + n_active * act
+        return (T * (16 + rec + (0 if prec == 1 else 64)) + V * ((0 if prec == 1 else xpos) + (5 if persistent else 1) * v4) +
+                n_active * act)
     if kernel == "k_update":
         disp = 32 if prec == 1 else 32      # FP32: float copy now + at the build; FP64: x at the build
         return V * (64 + 32 + (4 if persistent else 3) * v4 + (32 if prec == 1 else 0) + disp)
