@@ -391,19 +391,24 @@ __global__ void k_adj_out(Dev<R> D, const double4_32a *lam, const double *av, do
     }
 }
 // dE_e -= lambda_e . d g_e / d E_e: the tet's elastic gradient is linear in E_e (mu and lambda are), so its
-// derivative is the gradient evaluated with E_e = 1 (D carries mu and lambda of E = 1 and no per-tet scale; mu0 and es0
-// are the ones that the tets' constants were formed with)
+// derivative is the gradient evaluated with E_e = 1 (D carries mu and lambda of E = 1 and no per-tet scale).  The tets' constants
+// hold mu_e, which may be 0: mu h^2 V M is formed anew, from D_m^-1.
 template <typename R, bool CO = false>
-__global__ void __launch_bounds__(EB) k_adj_youngs(Dev<R> D, R mu0, const R *es0, const double4_32a *lam, double *dE)
+__global__ void __launch_bounds__(EB) k_adj_youngs(Dev<R> D, const double4_32a *lam, double *dE)
 {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= D.nt) return;
     TetIn<R> in;
     load_tet_in<R, CO>(D, e, in);
     if constexpr (!CO) {
-        const R f = D.mu / (es0 ? mu0 * es0[e] : mu0);
+        R w[3][3];
+        load_w<R>(D, e, w);
+        const R f = D.mu * D.hv[e];
+        int q = 0;
 #pragma unroll
-        for (int q = 0; q < 6; ++q) in.m[q] *= f;
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = i; j < 3; ++j, ++q) in.m[q] = f * (w[i][0] * w[j][0] + w[i][1] * w[j][1] + w[i][2] * w[j][2]);
     }
     R gv[4][3], dv[4][3];
     if (!tet_grad_eval<R, CO>(D, in, gv, dv)) return;

@@ -795,8 +795,8 @@ public:
             D1.mu = R(1.0 / (2.0 * (1.0 + M.nu)));
             D1.lam = R(M.nu / ((1.0 + M.nu) * (1.0 - 2.0 * M.nu)));
             D1.escale = nullptr;
-            if (corot) k_adj_youngs<R, true><<<(M.nt + EB - 1) / EB, EB, 0, s>>>(D1, D.mu, D.escale, adj_x, adj_dE);
-            else k_adj_youngs<R><<<(M.nt + EB - 1) / EB, EB, 0, s>>>(D1, D.mu, D.escale, adj_x, adj_dE);
+            if (corot) k_adj_youngs<R, true><<<(M.nt + EB - 1) / EB, EB, 0, s>>>(D1, adj_x, adj_dE);
+            else k_adj_youngs<R><<<(M.nt + EB - 1) / EB, EB, 0, s>>>(D1, adj_x, adj_dE);
             CK(cudaMemcpyAsync(dE, adj_dE, sizeof(double) * M.nt, cudaMemcpyDefault, s));
         }
         CK(cudaStreamSynchronize(s));

@@ -1,0 +1,45 @@
+"""The differentiation calls at the edges of what they accept."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+from paper_2405_08001_gb300 import scenes as S
+from test_gpu_parity import B, O  # noqa: F401  (fixtures)
+
+pytestmark = pytest.mark.gpu
+
+
+def strained(cells, seed):
+    sc = S.cube_drop(n=max(cells), cells=cells, drop=0.05)
+    rng = np.random.default_rng(seed)
+    c = sc.x0.mean(axis=0)
+    A = np.array([[1.03, 0.02, 0.0], [0.0, 0.99, 0.015], [0.0, 0.0, 1.0]])
+    return sc, (sc.x0 - c) @ A.T + c + 2e-5 * rng.normal(size=sc.x0.shape), rng
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("model", [0, 1, 2, 3])
+@pytest.mark.parametrize("uniform", [False, True])
+def test_zero_moduli(B, O, uniform, model, prec):  # noqa: F811
+    """dL/dE_e of tets with E_e = 0 (some of them, or all by youngs = 0) is finite and equals the oracle's with a modulus
+    of 1e-11 in their place (whose Hessian is about 1e-12 of the mass: lambda and the gradient change by no more than that).
+    The FP32 product's error is below 1e-5 (its hvp tests) and H's condition number here about 1e3."""
+    sc, x, rng = strained((3, 3, 3), 7)
+    E = np.full(sc.n_tets, 0.0 if uniform else 1e5)
+    E[::3] = 0.0
+    tiny = np.where(E == 0.0, 1e-11, E)
+    if uniform:
+        sim = B.Sim(dataclasses.replace(sc, youngs=0.0), precision=prec, model=model)
+    else:
+        sim = B.Sim(dataclasses.replace(sc, youngs=1.0, youngs_per_tet=E), precision=prec, model=model)
+    o = O.Oracle.from_scene(dataclasses.replace(sc, youngs=1.0, youngs_per_tet=tiny), model=model)
+    ax, av = rng.normal(size=x.shape), rng.normal(size=x.shape)
+    dE, dEo = np.zeros(sc.n_tets), np.zeros(sc.n_tets)
+    a, v, _, _ = B.sim_adjoint_step(sim.h, x, ax, av, dE=dE, tol=1e-13 if prec == 0 else 1e-9, max_iters=5000)
+    ao, vo, _, _ = o.adjoint_step(x, ax, av, dE=dEo, tol=1e-13, max_iters=5000)
+    assert np.isfinite(dE).all()
+    tol = 1e-9 if prec == 0 else 1e-2
+    for g, r in ((a, ao), (v, vo), (dE, dEo), (dE[::3], dEo[::3])):
+        assert np.linalg.norm(g - r) <= tol * np.linalg.norm(r)
+    sim.close()
