@@ -539,7 +539,7 @@ __device__ inline void bpq_exact(const BPDev &B, BPQWarp &W, int n, const Grids 
 {
     const int lane = threadIdx.x & 31;
     bool found = false;
-    float d = 0.0f, s = gs.e.s;   // the pair's cell size
+    float dlow = 0.0f, s = gs.e.s;   // the bound; the pair's cell size
     int4 cnd = make_int4(0, 0, 0, 0);
     if (lane < n) do {
         const uint2 pd = W.pend[lane];
@@ -558,8 +558,10 @@ __device__ inline void bpq_exact(const BPDev &B, BPQWarp &W, int n, const Grids 
                 const int f = __ldcg(B.eprim + qr), jp = __ldcg(B.eprim + qc);
                 if (B.tri[f].w == B.obj[v] && is_excluded(B, ((unsigned long long)jp << 31) | (unsigned long long)f)) break;
             }
-            d = pt_coeffs<float>(f3sub(c0, r0), f3sub(r1, r0), f3sub(r2, r0), cc, tv);
+            const v3<float> e1 = f3sub(r1, r0), e2 = f3sub(r2, r0);
+            const float d = pt_coeffs<float>(f3sub(c0, r0), e1, e2, cc, tv);
             if (!(d < B.thr + 4e-6f * s)) break;
+            dlow = cand_bound(d, dot(e1, e1), dot(e1, e2), dot(e2, e2), s);
             found = true;
             cnd = make_int4(v, (int)Ar.z, (int)Ar.w, t2);
         } else {
@@ -573,16 +575,15 @@ __device__ inline void bpq_exact(const BPDev &B, BPQWarp &W, int n, const Grids 
                     is_excluded(B, (1ull << 62) | ((unsigned long long)a << 31) | (unsigned long long)b))
                     break;
             }
-            d = ee_coeffs<float>(f3sub(r0, c0), f3sub(r1, c0), f3sub(c1, c0), cc, tv);
+            const float d = ee_coeffs<float>(f3sub(r0, c0), f3sub(r1, c0), f3sub(c1, c0), cc, tv);
             if (!(d < B.thr + 4e-6f * s)) break;
+            const v3<float> e0 = f3sub(r1, r0), e1 = f3sub(c1, c0);
+            dlow = cand_bound(d, dot(e0, e0), dot(e0, e1), dot(e1, e1), s);
             found = true;
             cnd = make_int4(-1 - (int)Ar.z, (int)Ar.w, (int)Ac.z, (int)Ac.w);
         }
     } while (false);
-    // the bound: less the rounding of the positions (as thr), and less what the clamped cases overestimate for nearly
-    // parallel edges or a sliver triangle (sin^2 of the angle under GeomEps<float>::par = 1e-5: at most L^2 par / (2 d), the
-    // edges no longer than a cell's diagonal)
-    bpq_emit(B, W, nout, found, cnd, d - 4e-6f * s - 1.5e-5f * s * s / fmaxf(d, 1e-30f));
+    bpq_emit(B, W, nout, found, cnd, dlow);
 }
 
 // queues the lanes' passing pairs (all lanes call); runs the exact tests once 32 are queued
