@@ -152,7 +152,7 @@ template <typename R> __host__ __device__ inline v3<R> rel(double ax, double ay,
 // within a cell or two, of size s, of their origin; a, b, c: the products e1.e1, e1.e2, e2.e2 of the two vectors whose
 // normal equations were solved, q = sin^2 of their angle.  d^2 exceeds the minimum by at most
 //   the rounding of the closest point, squared, where the interior solution is tried: a few 2^-24 s / q along either vector,
-//     as the right-hand sides lose by cancellation what the determinant does (4e-13 is 20 times the largest of 40 million
+//     as the right-hand sides lose by cancellation what the determinant does (4e-13 is eleven times the largest of 20 million
 //     sampled pairs, edges of 1 : 1 to 100 : 1);
 //   what the clamped cases miss of a minimum inside, q times the shorter vector's square (a sliver's width, squared), where
 //     only they are tried (q below GeomEps<float>::par, less its rounding);
