@@ -533,13 +533,31 @@ __device__ inline void bpq_emit(const BPDev &B, BPQWarp &W, int &n, bool found, 
 __device__ inline v3<float> f3sub(const float4 &a, const float4 &b) { return mkv(a.x - b.x, a.y - b.y, a.z - b.z); }
 __device__ inline unsigned long long key_of(const uint4 &A) { return (unsigned long long)A.y << 32 | A.x; }
 
+// cand_bound of a queued pair at distance d.  Its vertices are loaded anew, which the compiler must not undo: the products
+// kept over the closest-point code cost the whole kernel registers (the batched step 1.5 %).
+__device__ inline v3<float> load_again(const float4 *p)
+{
+    v3<float> a;
+    float w;
+    asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(w) : "l"(p));
+    return a;
+}
+__device__ inline float pair_bound(const BPDev &B, uint2 pd, float d, float s)
+{
+    const unsigned int qr = pd.x, qc = pd.y & ~BPQ_PT;
+    const bool pt = (pd.y & BPQ_PT) != 0u;
+    const v3<float> r0 = load_again(B.ev + qr), e0 = load_again(B.ev + B.ecap + qr) - r0;
+    const v3<float> e1 = pt ? load_again(B.ev + 2 * (size_t)B.ecap + qr) - r0 : load_again(B.ev + B.ecap + qc) - load_again(B.ev + qc);
+    return cand_bound(d, dot(e0, e0), dot(e0, e1), dot(e1, e1), s);
+}
+
 // exact tests of the first n queued pairs (all lanes call); both entries of a pair are in the same cell, so their
 // positions are relative to the same corner
 __device__ inline void bpq_exact(const BPDev &B, BPQWarp &W, int n, const Grids &gs, int &nout)
 {
     const int lane = threadIdx.x & 31;
     bool found = false;
-    float dlow = 0.0f, s = gs.e.s;   // the bound; the pair's cell size
+    float d = 0.0f, s = gs.e.s;   // the pair's cell size
     int4 cnd = make_int4(0, 0, 0, 0);
     if (lane < n) do {
         const uint2 pd = W.pend[lane];
@@ -558,10 +576,8 @@ __device__ inline void bpq_exact(const BPDev &B, BPQWarp &W, int n, const Grids 
                 const int f = __ldcg(B.eprim + qr), jp = __ldcg(B.eprim + qc);
                 if (B.tri[f].w == B.obj[v] && is_excluded(B, ((unsigned long long)jp << 31) | (unsigned long long)f)) break;
             }
-            const v3<float> e1 = f3sub(r1, r0), e2 = f3sub(r2, r0);
-            const float d = pt_coeffs<float>(f3sub(c0, r0), e1, e2, cc, tv);
+            d = pt_coeffs<float>(f3sub(c0, r0), f3sub(r1, r0), f3sub(r2, r0), cc, tv);
             if (!(d < B.thr + 4e-6f * s)) break;
-            dlow = cand_bound(d, dot(e1, e1), dot(e1, e2), dot(e2, e2), s);
             found = true;
             cnd = make_int4(v, (int)Ar.z, (int)Ar.w, t2);
         } else {
@@ -575,15 +591,13 @@ __device__ inline void bpq_exact(const BPDev &B, BPQWarp &W, int n, const Grids 
                     is_excluded(B, (1ull << 62) | ((unsigned long long)a << 31) | (unsigned long long)b))
                     break;
             }
-            const float d = ee_coeffs<float>(f3sub(r0, c0), f3sub(r1, c0), f3sub(c1, c0), cc, tv);
+            d = ee_coeffs<float>(f3sub(r0, c0), f3sub(r1, c0), f3sub(c1, c0), cc, tv);
             if (!(d < B.thr + 4e-6f * s)) break;
-            const v3<float> e0 = f3sub(r1, r0), e1 = f3sub(c1, c0);
-            dlow = cand_bound(d, dot(e0, e0), dot(e0, e1), dot(e1, e1), s);
             found = true;
             cnd = make_int4(-1 - (int)Ar.z, (int)Ar.w, (int)Ac.z, (int)Ac.w);
         }
     } while (false);
-    bpq_emit(B, W, nout, found, cnd, dlow);
+    bpq_emit(B, W, nout, found, cnd, found ? pair_bound(B, W.pend[lane], d, s) : 0.0f);
 }
 
 // queues the lanes' passing pairs (all lanes call); runs the exact tests once 32 are queued
