@@ -156,6 +156,29 @@ __device__ inline void box_of(const double4_32a *x, const int *v, int n, double 
     hi = make_float4(__double2float_ru(h[0] + infl), __double2float_ru(h[1] + infl), __double2float_ru(h[2] + infl), 0.f);
 }
 
+// Vertex j's position kept as the build's (x_b, and in the FP32 form its float head), and the bits of its largest |coordinate|:
+// a float's of the heads, or a double's upper half (conversions of doubles are as scarce as their arithmetic).
+__device__ inline unsigned int keep_x(const BPDev &B, int j)
+{
+    const double4_32a X = ldcg4(B.x + j);
+    B.xb[j] = X;
+    if (B.xbh) {
+        const float4 H = ldcg4(B.xh + j);
+        B.xbh[j] = H;
+        return __float_as_uint(fmaxf(fabsf(H.x), fmaxf(fabsf(H.y), fabsf(H.z))));
+    }
+    return max(__double2hiint(X.x) & 0x7fffffff, max(__double2hiint(X.y) & 0x7fffffff, __double2hiint(X.z) & 0x7fffffff));
+}
+// the warp's largest keep_x, rounded up to a float, into Ctrl::xmax_bits (all lanes call)
+__device__ inline void put_xmax(const BPDev &B, unsigned int m)
+{
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) != 0) return;
+    if (!B.xbh) m = __float_as_uint(__double2float_ru(__hiloint2double((int)m, -1)));
+    if (m > __ldcg(&B.ctrl->xmax_bits)) atomicMax(&B.ctrl->xmax_bits, m);
+}
+__device__ inline float get_xmax(const Ctrl *c) { return __uint_as_float(__ldcg(&c->xmax_bits)); }
+
 // a position relative to the lower corner of hash cell (ix, iy, iz) of size s, formed in double and rounded once to
 // float: positions within a cell or two of the corner keep ~1e-7 s in float wherever the scene sits
 __device__ inline float4 rel_corner(const double4_32a &X, int ix, int iy, int iz, float s, int w)
@@ -351,16 +374,18 @@ static __global__ void __launch_bounds__(BP_B) bp_boxes(BPDev B)
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         B.ctrl->n_cand[0] = B.ctrl->n_cand[1] = 0; B.ctrl->n_units = 0; B.ctrl->n_units_h = 0; B.ctrl->n_rebuilds += 1;
     }
+    unsigned int xm = 0u;
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += stride) {
         if (j < 3 * B.H) B.cnt[j] = 0u;
         if (j < B.nv) {
-            B.xb[j] = B.x[j];
-            if (B.xbh) B.xbh[j] = B.xh[j];
+            xm = max(xm, keep_x(B, j));
         }
         if (j < B.nf + B.ne) {
             atomicMax(&B.ctrl->cell_bits, __float_as_uint(bp_box(B, j)));
         }
     }
+    __syncwarp();
+    put_xmax(B, xm);
 }
 
 // one thread per triangle or edge (j < nf + ne) and per surface point (j < ns)

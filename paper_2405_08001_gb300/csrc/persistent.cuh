@@ -246,6 +246,7 @@ template <typename R, int PB, bool CL> struct PShared {
     double ig, e0;        // kept by the last warp: 1 / g^T P g of this iteration (0 below 1e-300), Delta E_0
     int oi[2];            // restarted, capped
     int cv;               // kept by the last warp: the eps rule fired
+    float xmax;           // Ctrl::xmax_bits
     int fi;
     uint32_t fe;
 };
@@ -564,6 +565,7 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
         sh.ig = g > 1e-300 ? 1.0 / g : 0.0;
         sh.e0 = (volatile double &)c->dE0;
         sh.cv = (volatile int &)c->converged;
+        sh.xmax = get_xmax(c);
     }
     const int vrows = min(PB / 32, max(1, (vs.b1 - vs.b0 + 31) >> 5));   // warps with vertices
     int npt = (volatile int &)c->n_cand[0], ncand = npt + (volatile int &)c->n_cand[1];
@@ -625,11 +627,15 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
             const int nprim = B.nf + B.ne;
             float ext_max = 0.0f;
             for (int j = tid; j < 3 * B.H; j += nthr) B.cnt[j] = 0u;
-            for (int j = ov; j < vs.b1; j += PB) { B.xb[j] = ldcg4(B.x + j); if (B.xbh) B.xbh[j] = ldcg4(B.xh + j); }
+            unsigned int xm = 0u;
+            for (int j = ov; j < vs.b1; j += PB) xm = max(xm, keep_x(B, j));
+            __syncwarp();
+            put_xmax(B, xm);
             const Share ps = share_of(nprim);
             for (int j = ps.b0 + (int)threadIdx.x; j < ps.b1; j += PB) ext_max = fmaxf(ext_max, bp_box(B, j));
             const float ext = (float)grid_max<R, PB, CL>(R(ext_max), rb.max_region<PT, R>(), sh, br, c);
             if (lead) c->cell_bits = __float_as_uint(ext);
+            if (threadIdx.x == 0) sh.xmax = get_xmax(c);
             st.mark(1);   // K_BP_BOXES
             const Grids cg = grids_of(B, ext);
             br.phase = 2;   // K_BP_COUNT
@@ -763,9 +769,11 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
                 const int nc = min(ncand, D.cand_cap), lane = threadIdx.x & 31;
                 // d changes by at most twice the largest displacement, so a candidate whose distance at the build was
                 // above `reach` cannot be active: it is passed over on that number alone, without its positions
-                // (1e-3 of the displacement and of dhat + r cover the floats' rounding)
+                // (1e-3 of the displacement and of dhat + r cover the floats' rounding; the FP32 form's displacement is one
+                // between float heads, each rounded by up to 2^-24 of its coordinate: 2 sqrt(3) 2^-23 xmax)
                 const float reach = disp_max < R(0) ? 3.0e38f
-                                                    : (float)D.dhat + 2.002f * sqrtf((float)disp_max) + (B.thr - (float)B.infl);
+                                                    : (float)D.dhat + 2.002f * sqrtf((float)disp_max) + (B.thr - (float)B.infl) +
+                                                          (sizeof(R) == 4 ? 4.3e-7f * sh.xmax : 0.0f);
                 // the candidates within reach queue in shared memory, per warp, and are worked on 32 at a time, so that
                 // the geometry runs with full warps; in the FP32 form they take the float filter first, and those that
                 // pass it queue once more for the float-float geometry

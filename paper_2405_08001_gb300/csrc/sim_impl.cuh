@@ -60,7 +60,7 @@ template <typename R4, typename R> __global__ void k_precond_out(const R4 *dg, d
 template <typename R> __global__ void k_set_state(Dev<R> D, const double *x, const double *v)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0) { D.ctrl->rebuild = 1; D.ctrl->cell_bits = 0u; }
+    if (i == 0) { D.ctrl->rebuild = 1; D.ctrl->cell_bits = 0u; D.ctrl->xmax_bits = 0u; }
     if (i >= D.nv) return;
     if (x) put_x<R>(D, i, make_double4_32a(x[3 * i], x[3 * i + 1], x[3 * i + 2], 0.0));
     if (v) D.v[i] = make_double4_32a(v[3 * i], v[3 * i + 1], v[3 * i + 2], 0.0);
@@ -80,7 +80,7 @@ template <typename R> __global__ void k_eval_in(Dev<R> D, const double *x, const
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0) {
         Ctrl *c = D.ctrl;
-        c->rebuild = 1; c->cell_bits = 0u; c->n_active = 0; c->n_near64 = 0;
+        c->rebuild = 1; c->cell_bits = 0u; c->xmax_bits = 0u; c->n_active = 0; c->n_near64 = 0;
     }
     if (i >= D.nv) return;
     const double4_32a T = D.xtil[i];
@@ -99,7 +99,7 @@ template <typename R> __global__ void k_eval_out(Dev<R> D, const double4_32a *xs
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0) {
         Ctrl *c = D.ctrl;
-        c->rebuild = 1; c->cell_bits = 0u; c->n_active_last = c->n_active; c->n_active = 0;
+        c->rebuild = 1; c->cell_bits = 0u; c->xmax_bits = 0u; c->n_active_last = c->n_active; c->n_active = 0;
     }
     if (i >= D.nv) return;
     const double4_32a T = xtsave[i];

@@ -82,3 +82,38 @@ def test_nearly_parallel_pairs_are_not_passed_over(B, ratio, kind):  # noqa: F81
     assert int(B.sim_get_trace(a.h)[0, B.TRACE_COLUMNS.index("n_active")]) == n
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("far", [150.0, 1000.0, 5000.0])
+def test_fp32_far_from_the_origin(B, far):  # noqa: F811
+    """The FP32 form measures displacements between float heads, whose rounding grows with the distance from the origin.  Two
+    tets there come 0.84 units of the heads' last place closer and within dhat, each by less than half a unit, so that
+    no head moves: the pair that a single iteration finds is found in a whole step.  (No stiffness: the first iteration
+    ends at x~.)"""
+    u = float(np.spacing(np.float32(far)))
+    d0 = round(1e-3 / u) * u
+    dhat = d0 - 0.6 * u
+    a = 0.1 * np.array([[0, 0, 0], [0.1, 0, 0], [0, 0.1, 0], [0.03, 0.03, -0.1]])
+    b = 0.1 * np.array([[0.03, 0.03, 0], [0.13, 0.03, 0.1], [0.03, 0.13, 0.1], [-0.07, -0.07, 0.1]])
+    b[:, 2] += d0
+    X = np.concatenate([a, b]) + [0, 0, far]
+    X[:, 2] = np.round(X[:, 2] / u) * u
+    v = np.zeros_like(X)
+    v[:4, 2], v[4:, 2] = 0.42 * u * 60, -0.42 * u * 60
+    T = np.array([[0, 2, 1, 3], [4, 5, 6, 7]], np.int32)
+    for t in T:
+        if np.linalg.det(X[t[1:]] - X[t[0]]) < 0:
+            t[[1, 2]] = t[[2, 1]]
+    sc = S.Scene(name="far", rest_x=X, tets=T, x0=X, v0=v, youngs=0.0, poisson=0.4, density=1000.0, dt=1.0 / 60.0, dhat=dhat, kappa=1e4,
+                 iters=3, steps=1)
+    s, w = (B.Sim(sc, precision=1, pad_r=2 * dhat) for _ in range(2))
+    B.sim_begin_step(s.h)
+    active = []
+    for _ in range(sc.iters):
+        B.sim_iterate(s.h, 1)
+        active.append(B.sim_get_iterate(s.h)[5]["n_active"])
+    assert active[0] == 0 and max(active) > 0, active
+    w.step(1)
+    assert B.sim_get_trace(w.h)[:, B.TRACE_COLUMNS.index("n_active")].astype(int).tolist() == active
+    s.close()
+    w.close()
