@@ -104,7 +104,8 @@ __device__ inline CellGrid grid_of(float s) { return {s, 1.0f / s}; }
 // The build's two grids from the largest extent of a box inflated by dhat + r (bp_box): the cells are that large for the
 // triangles and points, and smaller by dhat + r for the edges, whose boxes are inflated by half as much (with one grid and
 // one inflation for both, a cell held about 1.8 times the edges).  The margins keep the rounding of q / s from making a box
-// span three cells along an axis, as far from the origin on the finer grid (at least half as large) as on the other.
+// span three cells along an axis, as far from the origin on the finer grid (at least half as large) as on the other.  Where the
+// farthest vertex's finer cell would come near the last number, the edges too have the coarser cells.
 struct Grids {
     CellGrid t, e;
     __device__ inline const CellGrid &of(bool edge) const { return edge ? e : t; }
@@ -138,11 +139,12 @@ __device__ inline bool cell_of(float q, const CellGrid &g, int &i)
     return true;
 }
 
-__device__ inline Grids grids_of(const BPDev &B, float ext)
+__device__ inline Grids grids_of(const BPDev &B, float ext, float xmax)
 {
-    return {grid_of(ext * 1.0001f), grid_of(__fsub_ru(ext, __double2float_rd(B.infl)) * 1.0002f)};
+    const float t = ext * 1.0001f, e = __fsub_ru(ext, __double2float_rd(B.infl)) * 1.0002f;
+    return {grid_of(t), grid_of(xmax < float(CELL_BIAS / 2) * e ? e : t)};
 }
-__device__ inline Grids grids_of(const BPDev &B) { return grids_of(B, __uint_as_float(B.ctrl->cell_bits)); }
+__device__ inline Grids grids_of(const BPDev &B) { return grids_of(B, __uint_as_float(B.ctrl->cell_bits), __uint_as_float(B.ctrl->xmax_bits)); }
 
 __device__ inline void box_of(const double4_32a *x, const int *v, int n, double infl, float4 &lo, float4 &hi)
 {
@@ -173,7 +175,7 @@ __device__ inline unsigned int keep_x(const BPDev &B, int j)
 __device__ inline void put_xmax(const BPDev &B, unsigned int m)
 {
     m = __reduce_max_sync(0xffffffffu, m);
-    if ((threadIdx.x & 31) != 0) return;
+    if ((threadIdx.x & 31) != 0 || m == 0u) return;
     if (!B.xbh) m = __float_as_uint(__double2float_ru(__hiloint2double((int)m, -1)));
     if (m > __ldcg(&B.ctrl->xmax_bits)) atomicMax(&B.ctrl->xmax_bits, m);
 }

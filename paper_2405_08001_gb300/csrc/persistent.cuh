@@ -635,9 +635,10 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
             for (int j = ps.b0 + (int)threadIdx.x; j < ps.b1; j += PB) ext_max = fmaxf(ext_max, bp_box(B, j));
             const float ext = (float)grid_max<R, PB, CL>(R(ext_max), rb.max_region<PT, R>(), sh, br, c);
             if (lead) c->cell_bits = __float_as_uint(ext);
-            if (threadIdx.x == 0) sh.xmax = get_xmax(c);
+            const float xmax = get_xmax(c);
+            if (threadIdx.x == 0) sh.xmax = xmax;
             st.mark(1);   // K_BP_BOXES
-            const Grids cg = grids_of(B, ext);
+            const Grids cg = grids_of(B, ext, xmax);
             br.phase = 2;   // K_BP_COUNT
             for (int j = ps.b0 + (int)threadIdx.x; j < ps.b1; j += PB)
                 for_cells(B, __ldcg(B.blo + j), __ldcg(B.bhi + j), cg.of(j >= B.nf), [&](int i, int jj, int kk) { atomicAdd(&B.cnt[prim_bucket(B, j, i, jj, kk)], 1u); });

@@ -117,3 +117,16 @@ def test_fp32_far_from_the_origin(B, far):  # noqa: F811
     assert B.sim_get_trace(w.h)[:, B.TRACE_COLUMNS.index("n_active")].astype(int).tolist() == active
     s.close()
     w.close()
+
+
+def test_a_scene_near_the_grids_limit(B):  # noqa: F811
+    """Cells are numbered up to 2^20 from the origin.  A tet so far out that the triangles' cells are within that and the
+    edges' smaller ones would not be: the step runs."""
+    X = np.array([[0.0, 0.0, 0.0], [1.0, 0.0, 0.0], [0.0, 1.0, 0.0], [0.0, 0.0, 1.0]])
+    x0 = X + np.array([3.2e6, 0.0, 0.0])
+    sc = S.Scene(name="far", rest_x=X, tets=np.array([[0, 1, 2, 3]], np.int32), x0=x0, v0=np.zeros_like(X), youngs=1e3, poisson=0.4,
+                 density=1000.0, dt=1.0 / 60.0, dhat=1.0, kappa=1e4, iters=2)
+    sim = B.Sim(sc, precision=0, pad_r=1.0)
+    sim.step(1)
+    assert np.abs(sim.state()[0] - x0).max() < 1e-6
+    sim.close()
