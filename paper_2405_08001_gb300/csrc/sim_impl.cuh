@@ -73,21 +73,23 @@ template <typename R4> __global__ void k_out2(const R4 *a, const R4 *b, double *
     if (oa) { const R4 v = a[i]; oa[3 * i] = double(v.x); oa[3 * i + 1] = double(v.y); oa[3 * i + 2] = double(v.z); }
     if (ob) { const R4 v = b[i]; ob[3 * i] = double(v.x); ob[3 * i + 1] = double(v.y); ob[3 * i + 2] = double(v.z); }
 }
-// Before an evaluation at x (and x~ = xt; null keeps it): the state's x and x~ set aside, every vertex free, iteration 0's
-// accumulators initialised, a candidate build requested and the counters cleared.
-template <typename R> __global__ void k_eval_in(Dev<R> D, const double *x, const double *xt, double4_32a *xsave, double4_32a *xtsave)
+// Before an evaluation at x (and x~ = xt; null keeps it): the state's x and x~ set aside, every vertex free or (kin) those
+// that are kinematic marked so, iteration 0's accumulators initialised, a candidate build requested and the counters cleared.
+template <typename R>
+__global__ void k_eval_in(Dev<R> D, const double *x, const double *xt, bool kin, double4_32a *xsave, double4_32a *xtsave)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0) {
         Ctrl *c = D.ctrl;
-        c->rebuild = 1; c->cell_bits = 0u; c->xmax_bits = 0u; c->n_active = 0; c->n_near64 = 0;
+        c->rebuild = 1; c->cell_bits = 0u; c->n_active = 0; c->n_near64 = 0;
     }
     if (i >= D.nv) return;
     const double4_32a T = D.xtil[i];
     xsave[i] = D.x[i];
     xtsave[i] = T;
     const double4_32a X = make_double4_32a(x[3 * i], x[3 * i + 1], x[3 * i + 2], 0.0);
-    const double4_32a XT = xt ? make_double4_32a(xt[3 * i], xt[3 * i + 1], xt[3 * i + 2], D.mass[i]) : make_double4_32a(T.x, T.y, T.z, D.mass[i]);
+    const double w = kin && D.fix_slot[i] >= 0 ? -1.0 : D.mass[i];
+    const double4_32a XT = xt ? make_double4_32a(xt[3 * i], xt[3 * i + 1], xt[3 * i + 2], w) : make_double4_32a(T.x, T.y, T.z, w);
     D.xtil[i] = XT;
     put_x<R>(D, i, X);
     put_xt<R>(D, i, XT);
@@ -99,7 +101,7 @@ template <typename R> __global__ void k_eval_out(Dev<R> D, const double4_32a *xs
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0) {
         Ctrl *c = D.ctrl;
-        c->rebuild = 1; c->cell_bits = 0u; c->xmax_bits = 0u; c->n_active_last = c->n_active; c->n_active = 0;
+        c->rebuild = 1; c->cell_bits = 0u; c->n_active_last = c->n_active; c->n_active = 0;
     }
     if (i >= D.nv) return;
     const double4_32a T = xtsave[i];
@@ -398,14 +400,15 @@ public:
     }
 
     // ------------------------------------------------------------------------------------------ evaluations
-    // Runs the candidate build and the gradient pass at the given x (and xtilde) with all vertices free.
-    sim_status eval_setup(const double *x, const double *xt)
+    // Runs the candidate build and the gradient pass at the given x (and xtilde) with all vertices free, or (kin) with the
+    // kinematic ones as such.
+    sim_status eval_setup(const double *x, const double *xt, bool kin = false)
     {
         const double *dx = nullptr, *dt = nullptr;
         sim_status r = on_device(x, stage, dx);
         if (r) return r;
         if (xt) { r = on_device(xt, stage + 3 * (size_t)M.nv, dt); if (r) return r; }
-        k_eval_in<R><<<(M.nv + 255) / 256, 256, 0, s>>>(D, dx, dt, xsave, xtsave);
+        k_eval_in<R><<<(M.nv + 255) / 256, 256, 0, s>>>(D, dx, dt, kin && M.nfix > 0, xsave, xtsave);
         launch_bp();
         launch_grad(0);
         CK(cudaGetLastError());
@@ -744,7 +747,7 @@ public:
         if (!x || !v || !out) return fail(SIM_ERR_INVALID_ARG, "x, v and out are required");
         sim_status r = adj_alloc();
         if (r) return r;
-        r = eval_setup(x, nullptr);
+        r = eval_setup(x, nullptr, true);
         if (r) return r;
         const double *dv = nullptr;
         r = on_device(v, stage, dv);
@@ -764,7 +767,7 @@ public:
             return fail(SIM_ERR_INVALID_ARG, "x1, the adjoints and a positive tolerance and iteration cap are required");
         sim_status r = adj_alloc();
         if (r) return r;
-        r = eval_setup(x1, nullptr);   // H at x_{t+1}: candidates, active pairs and the gradient pass there
+        r = eval_setup(x1, nullptr, true);   // H at x_{t+1}: candidates, active pairs and the gradient pass there
         if (r) return r;
         const size_t bytes = sizeof(double) * 3 * (size_t)M.nv;
         const int nb = (M.nv + VB - 1) / VB;

@@ -43,3 +43,35 @@ def test_zero_moduli(B, O, uniform, model, prec):  # noqa: F811
     for g, r in ((a, ao), (v, vo), (dE, dEo), (dE[::3], dEo[::3])):
         assert np.linalg.norm(g - r) <= tol * np.linalg.norm(r)
     sim.close()
+
+
+# 432 tets: one cluster; 8,640: the whole grid in both precisions
+@pytest.mark.parametrize("cells", [(3, 3, 8), (12, 12, 10)])
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("model", [0, 2])
+def test_kinematic_rows_and_columns_are_dropped(B, O, model, prec, cells):  # noqa: F811
+    """H v and the reverse step on a bar whose two end caps are kinematic, against the oracle, which drops their rows and
+    columns: their entries of H v are 0, their ax0 is -av1 / h and their av0 is 0, all exactly."""
+    sc = S.twisted_bar(*cells)
+    fx = sc.fixed.astype(bool)
+    rng = np.random.default_rng(17)
+    x = sc.x0 + 1e-4 * rng.normal(size=sc.x0.shape)
+    sim = B.Sim(sc, precision=prec, model=model)
+    o = O.Oracle.from_scene(sc, model=model)
+    v = rng.normal(size=x.shape)
+    hv, ref = B.sim_eval_hvp(sim.h, x, v), o.hvp(x, v)
+    assert (hv[fx] == 0.0).all()
+    assert np.linalg.norm(hv - ref) <= (1e-10 if prec == 0 else 1e-5) * np.linalg.norm(ref)
+    ax, av = rng.normal(size=x.shape), 1e-2 * rng.normal(size=x.shape)
+    dE, dEo = np.zeros(sc.n_tets), np.zeros(sc.n_tets)
+    a, b, _, _ = B.sim_adjoint_step(sim.h, x, ax, av, dE=dE, tol=1e-13 if prec == 0 else 1e-9, max_iters=20000)
+    ao, bo, _, _ = o.adjoint_step(x, ax, av, dE=dEo, tol=1e-13, max_iters=20000)
+    assert (b[fx] == 0.0).all() and np.array_equal(a[fx], -av[fx] / sc.dt)
+    tol = 1e-9 if prec == 0 else 1e-2       # FP32: the product's 1e-5 at most, times H's condition number of about 1e3
+    for g, r in ((a, ao), (b, bo), (dE, dEo)):
+        assert np.linalg.norm(g - r) <= tol * np.linalg.norm(r), np.linalg.norm(g - r) / np.linalg.norm(r)
+    # the state's own flags are as they were: the next step holds the caps at their targets
+    t = sc.targets(0)
+    sim.step(1, t)
+    assert np.abs(sim.state()[0][fx] - t).max() < 1e-12
+    sim.close()
