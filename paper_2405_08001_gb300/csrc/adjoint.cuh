@@ -270,7 +270,7 @@ constexpr int CG_STRIDE = 8;      // iterations between two looks at the residua
 enum { CG_RZ = 0, CG_BETA, CG_RR, CG_BB, CG_IT, CG_N };
 struct CgArgs {
     double4_32a *x, *r, *p, *q, *P;   // solution, residual (the right-hand side at iteration 0), direction, H p, Jacobi entries
-    double4_32a *rec;                 // FP64 form, NH and SNH: [HVP_REC][nt] (hvp_record); else null
+    double4_32a *rec;                 // FP64 form, NH and SNH: [HVP_REC][nt] (hvp_record); else, or without room for it, null
     double *cg;                       // [CG_N] scalars carried between launches
     void *part;                       // reduction partials: 16 x gridDim.x doubles
     unsigned int *count;              // barrier arrival counter (zeroed before the launch)
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(CG_PB, CL ? 1 : 2) k_cg(Dev<R> D, CgArgs A)
     constexpr bool REC = sizeof(R) == 8 && !CO;
     if (A.it0 == 0) {
         if constexpr (REC)
-            for (int e = ts.b0 + (int)threadIdx.x; e < ts.b1; e += CG_PB) hvp_record(D, e, A.rec);
+            for (int e = ts.b0 + (int)threadIdx.x; A.rec && e < ts.b1; e += CG_PB) hvp_record(D, e, A.rec);
         Acc<double> s[2];
         for (int i = vs.b0 + (int)threadIdx.x; i < vs.b1; i += CG_PB) {
             const typename V4<R>::T Dg = ldcg4(D.dg[par] + i);

@@ -565,7 +565,7 @@ __device__ inline unsigned long long key_of(const uint4 &A) { return (unsigned l
 __device__ inline v3<float> load_again(const float4 *p)
 {
     v3<float> a;
-    float w;
+    [[maybe_unused]] float w;
     asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(w) : "l"(p));
     return a;
 }

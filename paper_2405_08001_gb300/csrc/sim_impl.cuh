@@ -689,14 +689,26 @@ public:
     }
 
     // ------------------------------------------------------------------------------------------ differentiation
+    // the product's vectors; and the solver's, with its launch (each at its first use)
+    sim_status hvp_alloc()
+    {
+        if (!adj_p) AL3(adj_p, M.nv);
+        if (!adj_q) AL3(adj_q, M.nv);
+        return SIM_OK;
+    }
     sim_status adj_alloc()
     {
-        if (adj_p) return SIM_OK;
+        if (adj_ready) return SIM_OK;
         const size_t n3 = 3 * (size_t)M.nv;
-        if (sizeof(R) == 8 && !corot) AL3(adj_rec, HVP_REC * (size_t)M.nt);
-        AL3(adj_x, M.nv); AL3(adj_r, M.nv); AL3(adj_P, M.nv); AL3(adj_q, M.nv);
-        AL3(adj_av, n3); AL3(adj_ax, n3); AL3(adj_cg, (size_t)CG_N);
-        AL3(adj_dE, (size_t)M.nt);
+        sim_status st = hvp_alloc();
+        if (st) return st;
+        if (!adj_x) AL3(adj_x, M.nv);
+        if (!adj_r) AL3(adj_r, M.nv);
+        if (!adj_P) AL3(adj_P, M.nv);
+        if (!adj_av) AL3(adj_av, n3);
+        if (!adj_ax) AL3(adj_ax, n3);
+        if (!adj_cg) AL3(adj_cg, (size_t)CG_N);
+        if (!adj_dE) AL3(adj_dE, (size_t)M.nt);
         // the solver's launch: one cluster on a small mesh, else one or two blocks an SM by the time step's rule (us an
         // iteration with two / one: FP64 8K tets 18.1 / 16.3, 25K 21.5 / 19.7, 83K 39.2 / 37.8; FP32, whose sums are double
         // here too, 25K 16.6 / 15.0, 41K 18.9 / 19.2, 83K 25.4 / 22.6)
@@ -707,9 +719,15 @@ public:
         cg_coop = cg_cluster == 0 && coop;
         if (cg_coop) CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cg_kernel(false), CG_PB, 0));
         cg_grid = cg_cluster > 0 ? cg_cluster : std::max(1, std::min(std::min(per_sm, one_block(true) ? 1 : 2) * nsm, MAXG));
-        AL3(cg_part, 16 * (size_t)cg_grid);
-        AL3(cg_count, 32);
-        AL3(adj_p, M.nv);
+        if (!cg_part) AL3(cg_part, 16 * (size_t)cg_grid);
+        if (!cg_count) AL3(cg_count, 32);
+        // the tets' record last, and the solve without it (its product then as sim_eval_hvp's) where the device has no room
+        if (sizeof(R) == 8 && !corot && dalloc(adj_rec, HVP_REC * (size_t)M.nt) != SIM_OK) {
+            if (adj_rec) return SIM_ERR_CUDA;
+            cudaGetLastError();
+            err.clear();
+        }
+        adj_ready = true;
         return SIM_OK;
     }
     const void *cg_kernel(bool cl) const
@@ -745,7 +763,7 @@ public:
     {
         CK(cudaSetDevice(dev));
         if (!x || !v || !out) return fail(SIM_ERR_INVALID_ARG, "x, v and out are required");
-        sim_status r = adj_alloc();
+        sim_status r = hvp_alloc();
         if (r) return r;
         r = eval_setup(x, nullptr, true);
         if (r) return r;
@@ -858,7 +876,7 @@ private:
     double *adj_av = nullptr, *adj_ax = nullptr, *adj_cg = nullptr, *adj_dE = nullptr, *cg_part = nullptr;
     unsigned int *cg_count = nullptr;
     int cg_cluster = 0, cg_grid = 1;
-    bool cg_coop = false;
+    bool cg_coop = false, adj_ready = false;
     int *stamp_kind = nullptr;
 
     sim_status fail(sim_status st, const std::string &m) { err = m; return st; }

@@ -75,3 +75,45 @@ def test_kinematic_rows_and_columns_are_dropped(B, O, model, prec, cells):  # no
     sim.step(1, t)
     assert np.abs(sim.state()[0][fx] - t).max() < 1e-12
     sim.close()
+
+
+def free_bytes():
+    import torch
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+
+def test_hvp_needs_no_solver_memory(B):  # noqa: F811
+    """The first sim_eval_hvp of a handle allocates two vectors of 32 bytes a vertex, and none of the reverse step's (160
+    bytes a tet among them)."""
+    sc, x, rng = strained((30, 30, 30), 3)
+    v = rng.normal(size=x.shape)
+    used = []
+    for _ in range(2):                          # the first handle loads the kernels
+        sim = B.Sim(sc, precision=0)
+        f = free_bytes()
+        B.sim_eval_hvp(sim.h, x, v)
+        used.append(f - free_bytes())
+        sim.close()
+    assert used[1] <= 2 * 32 * sc.n_verts + (4 << 20), used   # and the driver's 2 MB pages
+
+
+def test_reverse_step_without_room_for_the_record(B):  # noqa: F811
+    """Where the device has no room for the tets' record (160 bytes each) the solve runs without it: the same result
+    within the solver's tolerance, no SIM_ERR_OOM."""
+    import torch
+    sc, x, rng = strained((30, 30, 30), 5)      # 162,000 tets: 26 MB of record, 9 MB of vectors
+    ax, av = rng.normal(size=x.shape), np.zeros_like(x)
+    out = []
+    for full in (False, True):
+        sim = B.Sim(sc, precision=0)
+        torch.cuda.empty_cache()
+        hog = torch.empty(free_bytes() - (20 << 20), dtype=torch.uint8, device="cuda") if full else None
+        a, v, it, res = B.sim_adjoint_step(sim.h, x, ax, av, tol=1e-11, max_iters=5000)
+        assert res <= 1e-11
+        out.append((a, v))
+        del hog
+        torch.cuda.empty_cache()
+        sim.close()
+    for p, q in zip(*out):
+        assert np.linalg.norm(p - q) <= 1e-8 * np.linalg.norm(q)   # 1e-11 times the condition number of about 1e3
