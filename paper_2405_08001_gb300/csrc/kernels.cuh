@@ -27,9 +27,9 @@ template <typename R> struct Dev {
     const float *G0;                   // FP32 corotated densities: [14][nt] rest metric Dm^T Dm of each tet as
                                        // float-float (six heads, six tails: entries 00 01 02 11 12 22), then det Dm
                                        // as float-float; null otherwise
-    const float4 *tc;                  // FP32 form: [5][nt] constants of each tet: the 14 values of G0, then mu h^2 V M
+    const float4 *tc;                  // FP32 form, NH and SNH: [5][nt] constants of each tet: the 14 values of G0, then mu h^2 V M
                                        // (entries 00 01 02 11 12 22), M = Dm^-1 Dm^-T, mu the tet's own
-    const double4_32a *td;             // FP64 form: [2][nt] constants of each tet: mu h^2 V M (the six entries), det
+    const double4_32a *td;             // FP64 form, NH and SNH: [2][nt] constants of each tet: mu h^2 V M (the six entries), det
                                        // Dm^-1, h^2 V
     float4 *tS;                        // FP32 form: [4][nt] record of the last gradient pass per tet for tet_pHp_vec:
                                        // Z = Ds^-T (row-major), h^2 V Ds^-1 P Dm^-T (00 01 02 11 12 22), h^2 V k2

@@ -1035,6 +1035,7 @@ private:
         D.tc = nullptr;
         D.td = nullptr;
         D.tS = nullptr;
+        D.tk = nullptr;
         corot = M.model == MAT_FCR || M.model == MAT_ARAP;
         D.xbh = nullptr;
         D.pg = D.pnext = nullptr;
@@ -1044,13 +1045,14 @@ private:
                 float *g0;
                 AL(g0, 14 * (size_t)nt);
                 D.G0 = g0;
+            } else {
+                float4 *tc;
+                AL(tc, 5 * (size_t)nt);
+                D.tc = tc;
+                AL(D.tk, (size_t)nt);
             }
-            float4 *tc;
-            AL(tc, 5 * (size_t)nt);
-            D.tc = tc;
             AL(D.tS, 4 * (size_t)nt);
-            AL(D.tk, (size_t)nt);
-        } else {
+        } else if (!corot) {
             double4_32a *td;
             AL(td, 2 * (size_t)nt);
             D.td = td;
@@ -1089,8 +1091,8 @@ private:
             AL(c_tet, nt); AL(c_Dm, 9 * (size_t)nt); AL(c_hv, nt);
             if (!M.escale.empty()) AL(c_es, nt);
             if (D.G0) AL(c_G0, 14 * (size_t)nt);
-            if (sizeof(R) == 4) AL(c_tc, 5 * (size_t)nt);
-            else AL(c_td, 2 * (size_t)nt);
+            if (D.tc) AL(c_tc, 5 * (size_t)nt);
+            if (D.td) AL(c_td, 2 * (size_t)nt);
         }
         D.nseg = M.nseg;
         D.vscene = nullptr; D.seg = nullptr; D.sacc = nullptr; D.smax = nullptr; D.cmark = nullptr;
@@ -1250,10 +1252,10 @@ private:
             }
             if ((st = up(D.td, td.data(), sizeof(double4_32a) * 2 * (size_t)nt))) return st;
         }
-        if (D.tc) {
+        if (sizeof(R) == 4) {
             // rest metric Dm^T Dm and det Dm (six times the rest volume) per tet in double, stored as float-float
             std::vector<float> g0(14 * (size_t)nt);
-            std::vector<float4> tc(5 * (size_t)nt);
+            std::vector<float4> tc(D.tc ? 5 * (size_t)nt : 0);
             for (int e = 0; e < nt; ++e) {
                 double dm[3][3];
                 for (int c = 0; c < 3; ++c)
@@ -1272,6 +1274,7 @@ private:
                 const float dh = (float)det;
                 g0[(size_t)12 * nt + e] = dh;
                 g0[(size_t)13 * nt + e] = (float)(det - (double)dh);
+                if (!D.tc) continue;
                 double m[6], dw;
                 weighted(e, m, dw);
                 auto g = [&](int k) { return k < 14 ? g0[(size_t)k * nt + e] : (float)m[k - 14]; };
@@ -1279,7 +1282,7 @@ private:
                     tc[(size_t)k * nt + e] = make_float4(g(4 * k), g(4 * k + 1), g(4 * k + 2), g(4 * k + 3));
             }
             if (D.G0 && (st = up(D.G0, g0.data(), sizeof(float) * 14 * (size_t)nt))) return st;
-            if ((st = up(D.tc, tc.data(), sizeof(float4) * 5 * (size_t)nt))) return st;
+            if (D.tc && (st = up(D.tc, tc.data(), sizeof(float4) * 5 * (size_t)nt))) return st;
         }
         if (D.colored) {
             k_color_gather<R><<<(nt + 255) / 256, 256, 0, s>>>(D, c_tet, c_Dm, c_hv, c_es, c_G0, c_tc, c_td);
