@@ -63,7 +63,7 @@ template <typename R> __device__ inline void vadd(const Dev<R> &D, double4_32a *
 // the scalars that the gradient pass at x left (tet_pHp_edges): about 135 FP64 operations where the form on F took 430
 // (82,944 tets: 70 us a pass).  rec (or null): cof(Ds) and h^2 V Psi_3 det(Dm^-1) Ds kept by the solver, whose x stands
 // still (hvp_record): 99 operations.
-//   FP32: Dp (Dm^-1 S Dm^-T) + 2 (k1 tr(E) I + k2 E) Ds^-T, E = L + L^T, L = Dp Ds^-1, from the gradient pass's record: the
+//   FP32: (L P F^T + 2 (k1 tr(E) I + k2 E)) Ds^-T, E = L + L^T, L = Dp Ds^-1, from the gradient pass's record: the
 // derivative of the quadratic form of tet_pHp_edges, in which the large terms of a rotating direction never meet.
 constexpr int HVP_REC = 5;   // double4 per tet of the record
 __device__ inline void hvp_record(const Dev<double> &D, int e, double4_32a *rec)
@@ -98,13 +98,12 @@ __device__ inline void tet_hvp_edges(const Dev<R> &D, int e, const int4 &tv, con
 #pragma unroll
         for (int a = 0; a < 3; ++a)
 #pragma unroll
-            for (int b = 0; b < 3; ++b) E[a][b] = 2.0f * k2 * (L[a][b] + L[b][a]) + (a == b ? kt : 0.0f);
+            for (int b = 0; b < 3; ++b)
+                E[a][b] = 2.0f * k2 * (L[a][b] + L[b][a]) + (a == b ? kt : 0.0f) + L[a][0] * S[0][b] + L[a][1] * S[1][b] + L[a][2] * S[2][b];
 #pragma unroll
         for (int a = 0; a < 3; ++a)
 #pragma unroll
-            for (int i = 0; i < 3; ++i)
-                H[a][i] = dp[a][0] * S[0][i] + dp[a][1] * S[1][i] + dp[a][2] * S[2][i] + E[a][0] * Z[0][i] + E[a][1] * Z[1][i] +
-                          E[a][2] * Z[2][i];
+            for (int i = 0; i < 3; ++i) H[a][i] = E[a][0] * Z[0][i] + E[a][1] * Z[1][i] + E[a][2] * Z[2][i];
     } else {
         const double4_32a a = D.td[e], b = D.td[n + e];
         R s[3][3], c[3][3];
@@ -392,7 +391,7 @@ __global__ void k_adj_out(Dev<R> D, const double4_32a *lam, const double *av, do
 }
 // dE_e -= lambda_e . d g_e / d E_e: the tet's elastic gradient is linear in E_e (mu and lambda are), so its
 // derivative is the gradient evaluated with E_e = 1 (D carries mu and lambda of E = 1 and no per-tet scale).  The tets' constants
-// hold mu_e, which may be 0: mu h^2 V M is formed anew, from D_m^-1.
+// hold mu_e, which may be 0: mu h^2 V M (or its factor) is formed anew, from D_m^-1.
 template <typename R, bool CO = false>
 __global__ void __launch_bounds__(EB) k_adj_youngs(Dev<R> D, const double4_32a *lam, double *dE)
 {
@@ -404,11 +403,18 @@ __global__ void __launch_bounds__(EB) k_adj_youngs(Dev<R> D, const double4_32a *
         R w[3][3];
         load_w<R>(D, e, w);
         const R f = D.mu * D.hv[e];
-        int q = 0;
+        if constexpr (sizeof(R) == 4) {
+            double wd[3][3], k[6];
+            for (int i = 0; i < 9; ++i) wd[i / 3][i % 3] = w[i / 3][i % 3];
+            tri_factor(wd, sqrt((double)f), k);
+            for (int i = 0; i < 6; ++i) in.m[i] = (float)k[i];
+        } else {
+            int q = 0;
 #pragma unroll
-        for (int i = 0; i < 3; ++i)
+            for (int i = 0; i < 3; ++i)
 #pragma unroll
-            for (int j = i; j < 3; ++j, ++q) in.m[q] = f * (w[i][0] * w[j][0] + w[i][1] * w[j][1] + w[i][2] * w[j][2]);
+                for (int j = i; j < 3; ++j, ++q) in.m[q] = f * (w[i][0] * w[j][0] + w[i][1] * w[j][1] + w[i][2] * w[j][2]);
+        }
     }
     R gv[4][3], dv[4][3];
     if (!tet_grad_eval<R, CO>(D, in, gv, dv)) return;

@@ -27,12 +27,14 @@ template <typename R> struct Dev {
     const float *G0;                   // FP32 corotated densities: [14][nt] rest metric Dm^T Dm of each tet as
                                        // float-float (six heads, six tails: entries 00 01 02 11 12 22), then det Dm
                                        // as float-float; null otherwise
-    const float4 *tc;                  // FP32 form, NH and SNH: [5][nt] constants of each tet: the 14 values of G0, then mu h^2 V M
-                                       // (entries 00 01 02 11 12 22), M = Dm^-1 Dm^-T, mu the tet's own
+    const float4 *tc;                  // FP32 form, NH and SNH: [5][nt] constants of each tet: the 14 values of G0, then K
+                                       // (entries 00 10 20 11 21 22), K K^T = mu h^2 V M, M = Dm^-1 Dm^-T, mu the tet's own
     const double4_32a *td;             // FP64 form, NH and SNH: [2][nt] constants of each tet: mu h^2 V M (the six entries), det
                                        // Dm^-1, h^2 V
+    const double4_32a *tl;             // FP64 form, NH and SNH: [nt] K's entries 00 10 20 11,
+    const double2 *tl2;                // and [nt] 21 22
     float4 *tS;                        // FP32 form: [4][nt] record of the last gradient pass per tet for tet_pHp_vec:
-                                       // Z = Ds^-T (row-major), h^2 V Ds^-1 P Dm^-T (00 01 02 11 12 22), h^2 V k2
+                                       // Z = Ds^-T (row-major), h^2 V P F^T (00 01 02 11 12 22), h^2 V k2
     R *tk;                             // the record's scalars: FP32 form [nt] h^2 V k1; FP64 form [2][nt]
                                        // h^2 V Psi_33 det(Dm^-1)^2 and h^2 V Psi_3 det(Dm^-1)
     R4 *g[2], *dg[2];                  // ping-pong by iteration parity; g.w = plane curvature kappa b'', dg.w = xtil.w
@@ -406,12 +408,32 @@ template <typename R> __device__ inline void tet_material(const Dev<R> &D, int e
     if (D.escale) { R s = D.escale[e]; mu *= s; lam *= s; }
 }
 
+// The lower triangular factor K of f^2 W W^T (entries 00 10 20 11 21 22), W = D_m^-1, from W's rows by Gram-Schmidt (u
+// times W's condition number) and not from their products (its square).
+__host__ __device__ inline void tri_factor(const double w[3][3], double f, double k[6])
+{
+    double q[3][3], l[3][3];
+    for (int i = 0; i < 3; ++i) {
+        for (int c = 0; c < 3; ++c) q[i][c] = w[i][c];
+        for (int j = 0; j < i; ++j) {
+            const double d = l[i][j] = q[i][0] * q[j][0] + q[i][1] * q[j][1] + q[i][2] * q[j][2];
+            for (int c = 0; c < 3; ++c) q[i][c] -= d * q[j][c];
+        }
+        l[i][i] = sqrt(q[i][0] * q[i][0] + q[i][1] * q[i][1] + q[i][2] * q[i][2]);
+        if (i == 2) break;
+        const double r = 1.0 / l[i][i];
+        for (int c = 0; c < 3; ++c) q[i][c] *= r;
+    }
+    k[0] = f * l[0][0]; k[1] = f * l[1][0]; k[2] = f * l[2][0]; k[3] = f * l[1][1]; k[4] = f * l[2][1]; k[5] = f * l[2][2];
+}
+
 // The per-tet constants a gradient evaluation streams in (coalesced, structure-of-arrays in memory).  The densities
 // without an I1 term work on the edge vectors (tet_grad_edges) and need no D_m^-1; FCR and ARAP do.
 template <typename R> struct TetIn {
     int4 tv;
     R w[3][3];      // FCR, ARAP: rows of D_m^-1
-    R m[6];         // mu h^2 V M, M = D_m^-1 D_m^-T, entries 00 01 02 11 12 22
+    R m[6];         // FP64 form: mu h^2 V M, M = D_m^-1 D_m^-T, entries 00 01 02 11 12 22; FP32 form: its lower triangular
+                    // factor K, mu h^2 V M = K K^T, entries 00 10 20 11 21 22 (tri_factor)
     R dw;           // FP64 form: det D_m^-1
     R hv, es;       // h^2 V, the Young's modulus scale
     float g0[14];   // FP32 form: rest metric entries 00 01 02 11 12 22, heads then tails; det Dm head, tail
@@ -663,8 +685,8 @@ __device__ inline void tet_metric(const Dev<float> &D, const TetIn<float> &in, f
 // their products with Dm^-1 are formed.  The FP32 form takes the forces from the metric change,
 //   h^2 V Ds^-T (mu G M + (mu + Psi_3 J) I),    G = Ds^T Ds - Dm^T Dm,
 // which equals the line above exactly and stays accurate for small strains under any rotation (mu + Psi_3 J is lambda
-// log J for NH); G M is formed with compensated (Dot2) products from the float-float G, its terms being up to
-// cond(Dm)^2 times larger than the result.  Both leave the record that tet_pHp_vec reads (e >= 0).  Returns false (and
+// log J for NH).  mu h^2 V M enters as its factor, K K^T: G K is formed with compensated (Dot2) products from the
+// float-float G, its terms being up to cond(Dm) times larger than the result.  Both leave the record that tet_pHp_vec reads (e >= 0).  Returns false (and
 // flags the error) when det F <= 0.
 // FP64: 170 FP64 operations a tet where the form on F took about 430, at 1.65 FP64 lanes per clock and SM.
 template <typename R>
@@ -706,39 +728,56 @@ __device__ inline bool tet_grad_edges(const Dev<R> &D, const TetIn<R> &in, R gv[
         }
         k33 *= in.hv;
         const float id = 1.0f / (J * in.g0[12]);   // 1 / det Ds
-        const float M[3][3] = {{in.m[0], in.m[1], in.m[2]}, {in.m[1], in.m[3], in.m[4]}, {in.m[2], in.m[4], in.m[5]}};
+        const float K[3][3] = {{in.m[0], 0.0f, 0.0f}, {in.m[1], in.m[3], 0.0f}, {in.m[2], in.m[4], in.m[5]}};
         const float hj = in.hv * mJ;
-        float K[3][3];
+        float A[3][3];   // G K
 #pragma unroll
         for (int i = 0; i < 3; ++i)
 #pragma unroll
             for (int b = 0; b < 3; ++b) {
-                ffacc acc = ffacc::prod_f(G[i][0], M[0][b]);
+                ffacc acc = ffacc::prod_f(G[i][b], K[b][b]);
 #pragma unroll
-                for (int j = 1; j < 3; ++j) acc.add_prod_f(G[i][j], M[j][b]);
-                K[i][b] = acc.value();
+                for (int j = b + 1; j < 3; ++j) acc.add_prod_f(G[i][j], K[j][b]);
+                A[i][b] = acc.value();
             }
+        float Y[3][3];   // cof(Ds) G K
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) Y[a][b] = c[a][0] * A[0][b] + c[a][1] * A[1][b] + c[a][2] * A[2][b];
+        if (e >= 0) {
+            float S[3][3];   // h^2 V P F^T = h^2 V (mu + Psi_3 J) I + Ds^-T G K (Ds K)^T
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const float f[3] = {s[a][0] * K[0][0] + s[a][1] * K[1][0] + s[a][2] * K[2][0], s[a][1] * K[1][1] + s[a][2] * K[2][1],
+                                    s[a][2] * K[2][2]};
+#pragma unroll
+                for (int i = 0; i <= a; ++i)
+                    S[i][a] = (Y[i][0] * f[0] + Y[i][1] * f[1] + Y[i][2] * f[2]) * id + (i == a ? hj : 0.0f);
+            }
+            const size_t n = (size_t)D.nt;
+            D.tS[2 * n + e] = make_float4(c[2][2] * id, S[0][0], S[0][1], S[0][2]);
+            D.tS[3 * n + e] = make_float4(S[1][1], S[1][2], S[2][2], in.hv * k2);
+        }
         // (the two parts are not added before they meet cof(Ds), and 1 / det Ds comes last: each sum and product
         // rounded once more on the way cost a tenth of the gradient's accuracy)
 #pragma unroll
         for (int a = 0; a < 3; ++a)
 #pragma unroll
-            for (int i = 0; i < 3; ++i) H[a][i] = (hj * c[a][i] + c[a][0] * K[0][i] + c[a][1] * K[1][i] + c[a][2] * K[2][i]) * id;
+            for (int i = 0; i < 3; ++i) {
+                float h = hj * c[a][i];
+#pragma unroll
+                for (int b = 0; b <= i; ++b) h += Y[a][b] * K[i][b];
+                H[a][i] = h * id;
+            }
 #pragma unroll
         for (int a = 0; a < 3; ++a)
 #pragma unroll
             for (int i = 0; i < 3; ++i) c[a][i] *= id;
         if (e >= 0) {
-            float S[3][3];
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int j = i; j < 3; ++j) S[i][j] = c[0][i] * H[0][j] + c[1][i] * H[1][j] + c[2][i] * H[2][j];
             const size_t n = (size_t)D.nt;
             D.tS[e] = make_float4(c[0][0], c[0][1], c[0][2], c[1][0]);
             D.tS[n + e] = make_float4(c[1][1], c[1][2], c[2][0], c[2][1]);
-            D.tS[2 * n + e] = make_float4(c[2][2], S[0][0], S[0][1], S[0][2]);
-            D.tS[3 * n + e] = make_float4(S[1][1], S[1][2], S[2][2], in.hv * k2);
             D.tk[e] = in.hv * k1;
         }
     } else {
@@ -767,8 +806,16 @@ __device__ inline bool tet_grad_edges(const Dev<R> &D, const TetIn<R> &in, R gv[
 #pragma unroll
             for (int i = 0; i < 3; ++i) H[a][i] = s[a][0] * M[0][i] + s[a][1] * M[1][i] + s[a][2] * M[2][i] + k3 * c[a][i];
     }
-    const R m0 = in.m[0], m1 = in.m[3], m2 = in.m[5];
-    const R ms = m0 + m1 + m2 + R(2) * (in.m[1] + in.m[2] + in.m[4]);   // x_0's weights are minus the others' sum
+    R m0 = in.m[0], m1 = in.m[3], m2 = in.m[5], ms;   // x_0's weights are minus the others' sum
+    if constexpr (sizeof(R) == 4) {
+        const R k0 = in.m[0] + in.m[1] + in.m[2], k1 = in.m[3] + in.m[4];
+        ms = k0 * k0 + k1 * k1 + m2 * m2;
+        m0 *= m0;
+        m1 = m1 * m1 + in.m[1] * in.m[1];
+        m2 = m2 * m2 + in.m[4] * in.m[4] + in.m[2] * in.m[2];
+    } else {
+        ms = m0 + m1 + m2 + R(2) * (in.m[1] + in.m[2] + in.m[4]);
+    }
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         gv[1][a] = H[a][0]; gv[2][a] = H[a][1]; gv[3][a] = H[a][2];
@@ -1404,13 +1451,15 @@ __global__ void __launch_bounds__(VB) k_dir(Dev<R> D, int par)
 // Psi_3 d2det(F)[dF, dF] + Psi_1 d2I1(F)[dF, dF]] (Sec. 3.1 with H2 = 2I, H3 the det Hessian, H1 the Hessian of
 // tr(S)), at the x of the last gradient pass, whose record it reads.  On the direction's edge vectors Dp (columns p_i -
 // p_0) for NH and SNH, so that neither D_m^-1 nor dF is needed:
-//   FP64: 2 Psi_2 h^2 V M : Dp^T Dp + h^2 V Psi_33 det(Dm^-1)^2 (cof(Ds) : Dp)^2 + h^2 V Psi_3 det(Dm^-1) 2 cof(Dp) : Ds
+//   FP64: |Dp K|^2 + h^2 V Psi_33 det(Dm^-1)^2 (cof(Ds) : Dp)^2 + h^2 V Psi_3 det(Dm^-1) 2 cof(Dp) : Ds, with 2 Psi_2 h^2 V M =
+// K K^T, K lower triangular: as many operations as M : Dp^T Dp, whose terms are the aspect ratio's square larger than their
+// sum where dF is not (a tet 1,000 times wider than high, p affine: 2.4e4 roundings against 1e2).
 // (97 FP64 operations; on F and with the scalars formed anew it took 330: 54 -> 31 us an iteration for 98K tets).
 //   FP32: the second derivative of Psi written in C = F^T F, S : dF^T dF + k1 (tr C^-1 E)^2 + k2 tr(C^-1 E C^-1 E), E =
 // dF^T F + F^T dF.  With L = dF F^-1 = Dp Ds^-1, tr C^-1 E = tr(L + L^T) and tr(C^-1 E C^-1 E) = |L + L^T|^2, and S : dF^T dF =
-// (Dm^-1 S Dm^-T) : Dp^T Dp.  A direction that rotates the tet cancels inside L + L^T, so the large terms mu |dF|^2 and
-// Psi_3 d2det(F)[dF, dF] of the I2/I3 form, which cancel for it, never meet in float.  The record (68 bytes: Ds^-T, the
-// weighted stress, k1, k2) stands in for the positions' eight gathers and D_m^-1.
+// (P F^T) : L^T L (and not (Dm^-1 S Dm^-T) : Dp^T Dp, for the same reason as K).  A direction that rotates the tet cancels
+// inside L + L^T, so the large terms mu |dF|^2 and Psi_3 d2det(F)[dF, dF] of the I2/I3 form, which cancel for it, never meet
+// in float.  The record (68 bytes: Ds^-T, h^2 V P F^T, k1, k2) stands in for the positions' eight gathers and D_m^-1.
 template <typename R>
 __device__ inline R tet_pHp_edges(const Dev<R> &D, int e, const int4 &tv, const R (&dp)[3][3])
 {
@@ -1433,22 +1482,23 @@ __device__ inline R tet_pHp_edges(const Dev<R> &D, int e, const int4 &tv, const 
 #pragma unroll
         for (int i = 0; i < 3; ++i)
 #pragma unroll
-            for (int j = i; j < 3; ++j) g[i][j] = dp[0][i] * dp[0][j] + dp[1][i] * dp[1][j] + dp[2][i] * dp[2][j];
+            for (int j = i; j < 3; ++j) g[i][j] = L[0][i] * L[0][j] + L[1][i] * L[1][j] + L[2][i] * L[2][j];
         const float SD = q2.y * g[0][0] + q3.x * g[1][1] + q3.z * g[2][2] +
                          2.0f * (q2.z * g[0][1] + q2.w * g[0][2] + q3.y * g[1][2]);
         return SD + k1 * tr * tr + q3.w * t2;
     } else {
-        const double4_32a a = D.td[e], b = D.td[n + e];
+        const double4_32a a = D.tl[e];
+        const double2 b = D.tl2[e];
         const R k33 = __ldcg(D.tk + e), k3 = __ldcg(D.tk + n + e);
         R s[3][3], g3, h3;
         tet_ds<R>(D, tv, s);
         det_forms<R>(s, dp, g3, h3);
-        R g[3][3];
+        R md = R(0);
 #pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = i; j < 3; ++j) g[i][j] = dp[0][i] * dp[0][j] + dp[1][i] * dp[1][j] + dp[2][i] * dp[2][j];
-        const R md = a.x * g[0][0] + a.w * g[1][1] + b.y * g[2][2] + R(2) * (a.y * g[0][1] + a.z * g[0][2] + b.x * g[1][2]);
+        for (int i = 0; i < 3; ++i) {
+            const R y0 = dp[i][0] * a.x + dp[i][1] * a.y + dp[i][2] * a.z, y1 = dp[i][1] * a.w + dp[i][2] * b.x, y2 = dp[i][2] * b.y;
+            md += y0 * y0 + y1 * y1 + y2 * y2;
+        }
         return md + k33 * (g3 * g3) + (R(2) * k3) * h3;
     }
 }

@@ -1034,6 +1034,8 @@ private:
         D.G0 = nullptr;
         D.tc = nullptr;
         D.td = nullptr;
+        D.tl = nullptr;
+        D.tl2 = nullptr;
         D.tS = nullptr;
         D.tk = nullptr;
         corot = M.model == MAT_FCR || M.model == MAT_ARAP;
@@ -1056,6 +1058,12 @@ private:
             double4_32a *td;
             AL(td, 2 * (size_t)nt);
             D.td = td;
+            double4_32a *tl;
+            double2 *tl2;
+            AL(tl, (size_t)nt);
+            AL(tl2, (size_t)nt);
+            D.tl = tl;
+            D.tl2 = tl2;
             AL(D.tk, 2 * (size_t)nt);
         }
         double *mass; AL(mass, nv); D.mass = mass;
@@ -1230,27 +1238,33 @@ private:
         if ((st = up(B.edge, ed.data(), sizeof(int4) * M.ne))) return st;
         if ((st = up(B.obj, M.obj.data(), sizeof(int) * nv))) return st;
         if (B.excl && (st = up(B.excl, M.excl.data(), sizeof(unsigned long long) * M.excl.size()))) return st;
-        // mu h^2 V M with M = Dm^-1 Dm^-T (00 01 02 11 12 22) and det Dm^-1, in double
-        auto weighted = [&](int e, double m[6], double &dw) {
-            const double f = M.hv[e] * M.mu * (M.escale.empty() ? 1.0 : M.escale[e]);
-            double w[3][3];
+        // D_m^-1 and mu h^2 V, in double
+        auto inverse = [&](int e, double w[3][3]) {
             for (int r = 0; r < 3; ++r)
                 for (int c = 0; c < 3; ++c) w[r][c] = M.Dm[(size_t)(3 * r + c) * nt + e];
-            int q = 0;
-            for (int i = 0; i < 3; ++i)
-                for (int j = i; j < 3; ++j, ++q) m[q] = f * (w[i][0] * w[j][0] + w[i][1] * w[j][1] + w[i][2] * w[j][2]);
-            dw = w[0][0] * (w[1][1] * w[2][2] - w[1][2] * w[2][1]) - w[0][1] * (w[1][0] * w[2][2] - w[1][2] * w[2][0]) +
-                 w[0][2] * (w[1][0] * w[2][1] - w[1][1] * w[2][0]);
         };
+        auto weight = [&](int e) { return M.hv[e] * M.mu * (M.escale.empty() ? 1.0 : M.escale[e]); };
         if (D.td) {
-            std::vector<double4_32a> td(2 * (size_t)nt);
+            std::vector<double4_32a> td(2 * (size_t)nt), tl(nt);
+            std::vector<double2> tl2(nt);
             for (int e = 0; e < nt; ++e) {
-                double m[6], dw;
-                weighted(e, m, dw);
+                double w[3][3], m[6];
+                inverse(e, w);
+                const double f = weight(e);
+                for (int i = 0, q = 0; i < 3; ++i)
+                    for (int j = i; j < 3; ++j, ++q) m[q] = f * (w[i][0] * w[j][0] + w[i][1] * w[j][1] + w[i][2] * w[j][2]);
+                const double dw = w[0][0] * (w[1][1] * w[2][2] - w[1][2] * w[2][1]) - w[0][1] * (w[1][0] * w[2][2] - w[1][2] * w[2][0]) +
+                                  w[0][2] * (w[1][0] * w[2][1] - w[1][1] * w[2][0]);
                 td[e] = make_double4_32a(m[0], m[1], m[2], m[3]);
                 td[(size_t)nt + e] = make_double4_32a(m[4], m[5], dw, M.hv[e]);
+                double k[6];
+                tri_factor(w, std::sqrt(f), k);
+                tl[e] = make_double4_32a(k[0], k[1], k[2], k[3]);
+                tl2[e] = make_double2(k[4], k[5]);
             }
             if ((st = up(D.td, td.data(), sizeof(double4_32a) * 2 * (size_t)nt))) return st;
+            if ((st = up(D.tl, tl.data(), sizeof(double4_32a) * (size_t)nt))) return st;
+            if ((st = up(D.tl2, tl2.data(), sizeof(double2) * (size_t)nt))) return st;
         }
         if (sizeof(R) == 4) {
             // rest metric Dm^T Dm and det Dm (six times the rest volume) per tet in double, stored as float-float
@@ -1275,8 +1289,9 @@ private:
                 g0[(size_t)12 * nt + e] = dh;
                 g0[(size_t)13 * nt + e] = (float)(det - (double)dh);
                 if (!D.tc) continue;
-                double m[6], dw;
-                weighted(e, m, dw);
+                double w[3][3], m[6];
+                inverse(e, w);
+                tri_factor(w, std::sqrt(weight(e)), m);
                 auto g = [&](int k) { return k < 14 ? g0[(size_t)k * nt + e] : (float)m[k - 14]; };
                 for (int k = 0; k < 5; ++k)
                     tc[(size_t)k * nt + e] = make_float4(g(4 * k), g(4 * k + 1), g(4 * k + 2), g(4 * k + 3));

@@ -105,3 +105,32 @@ def test_separate_tets(B, O, aspect, prec):  # noqa: F811
         ref = o.pHp(x, q)
         assert abs(B.sim_eval_pHp(sim.h, x, q) - ref) <= tol[n, 2] + 8 * u * abs(ref), (J, "pHp")
     sim.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("aspect", [1.0, 30.0, 1000.0])
+def test_flat_tets_along_smooth_directions(B, O, aspect, prec):  # noqa: F811
+    """p^T H p of flat tets along p = A X, whose dF = A does not grow with the aspect ratio: forming dF from
+    the edges costs u times the aspect ratio, and no more than four times that may go into the sum of the terms' magnitudes.
+    (On M = Dm^-1 Dm^-T, whose entries are the ratio's square, it costs u times that.)"""
+    for seed in range(4):
+        rng = np.random.default_rng(10 * int(aspect) + seed)
+        sc = separate_tets(aspect, rng)
+        o = O.Oracle.from_scene(sc)
+        sim = B.Sim(sc, precision=prec)
+        u = 2.0**-53 if prec == 0 else 2.0**-24
+        for n, t in enumerate(sc.tets):
+            J = J_EDGE[n]
+            if not 0.4 < J < 2.1:
+                continue
+            Dm = (sc.rest_x[t[1:]] - sc.rest_x[t[0]]).T
+            F = (sc.x0[t[1:]] - sc.x0[t[0]]).T @ np.linalg.inv(Dm)
+            A = rng.normal(size=(3, 3))
+            p = np.zeros_like(sc.x0)
+            p[t] = (sc.rest_x[t] - sc.rest_x[t].mean(axis=0)) @ A.T
+            hv, L, a2, f = sc.dt**2 * np.linalg.det(Dm) / 6, abs(np.log(J)), np.sum(A * A), np.linalg.norm(F)
+            scale = hv * a2 * (MU + (MU + LAM * (1 + L)) / J**2 * f**4 + (LAM * L + MU) / J * 2 * f)
+            scale += 1000.0 * np.linalg.det(Dm) / 24 * np.sum(p * p)
+            err = abs(B.sim_eval_pHp(sim.h, sc.x0, p) - o.pHp(sc.x0, p))
+            assert err <= 4 * aspect * u * scale, (J, err / (aspect * u * scale))
+        sim.close()
