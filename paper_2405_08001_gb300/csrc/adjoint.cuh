@@ -43,11 +43,11 @@ __global__ void k_hvp_vert(Dev<R> D, int par, const double4_32a *v, double4_32a 
     if (i < D.nv) out[i] = hvp_vert<R>(D, par, i, v[i]);
 }
 
-template <typename R> __device__ inline v3<R> vload(const Dev<R> &D, const double4_32a *v, int i)
+template <typename R> __device__ inline v3<double> vload(const Dev<R> &D, const double4_32a *v, int i)
 {
-    if (dropped(D, i)) return mkv(R(0), R(0), R(0));
+    if (dropped(D, i)) return mkv(0.0, 0.0, 0.0);
     const double4_32a a = ldcg4(v + i);
-    return mkv(R(a.x), R(a.y), R(a.z));
+    return mkv(a.x, a.y, a.z);
 }
 template <typename R> __device__ inline void vadd(const Dev<R> &D, double4_32a *out, int i, double a, double b, double c)
 {
@@ -190,16 +190,17 @@ __device__ inline bool tet_hvp_rotated(const Dev<R> &D, int e, const int4 &tv, c
     return true;
 }
 
-// out += H_e v of tet e; returns v^T H_e v (in double)
+// out += H_e v of tet e; returns v^T H_e v, in double as every sum: in the FP32 form from v itself and the entries that were
+// added, so that it is the v^T (H v) of the vectors
 template <typename R, bool CO>
 __device__ inline double hvp_tet(const Dev<R> &D, int e, const double4_32a *v, double4_32a *out, const double4_32a *rec = nullptr)
 {
     const int4 tv = D.tet[e];
-    const v3<R> V0 = vload(D, v, tv.x), V1 = vload(D, v, tv.y), V2 = vload(D, v, tv.z), V3 = vload(D, v, tv.w);
+    const v3<double> V0 = vload(D, v, tv.x), V1 = vload(D, v, tv.y), V2 = vload(D, v, tv.z), V3 = vload(D, v, tv.w);
     R dp[3][3], H[3][3];
-    dp[0][0] = V1.x - V0.x; dp[1][0] = V1.y - V0.y; dp[2][0] = V1.z - V0.z;
-    dp[0][1] = V2.x - V0.x; dp[1][1] = V2.y - V0.y; dp[2][1] = V2.z - V0.z;
-    dp[0][2] = V3.x - V0.x; dp[1][2] = V3.y - V0.y; dp[2][2] = V3.z - V0.z;
+    dp[0][0] = R(V1.x) - R(V0.x); dp[1][0] = R(V1.y) - R(V0.y); dp[2][0] = R(V1.z) - R(V0.z);
+    dp[0][1] = R(V2.x) - R(V0.x); dp[1][1] = R(V2.y) - R(V0.y); dp[2][1] = R(V2.z) - R(V0.z);
+    dp[0][2] = R(V3.x) - R(V0.x); dp[1][2] = R(V3.y) - R(V0.y); dp[2][2] = R(V3.z) - R(V0.z);
     if constexpr (CO) {
         if (!tet_hvp_rotated<R>(D, e, tv, dp, H)) return 0.0;
     } else {
@@ -208,13 +209,23 @@ __device__ inline double hvp_tet(const Dev<R> &D, int e, const double4_32a *v, d
     vadd<R>(D, out, tv.y, H[0][0], H[1][0], H[2][0]);
     vadd<R>(D, out, tv.z, H[0][1], H[1][1], H[2][1]);
     vadd<R>(D, out, tv.w, H[0][2], H[1][2], H[2][2]);
-    vadd<R>(D, out, tv.x, -(H[0][0] + H[0][1] + H[0][2]), -(H[1][0] + H[1][1] + H[1][2]), -(H[2][0] + H[2][1] + H[2][2]));
-    R q = R(0);
+    const R h0 = -(H[0][0] + H[0][1] + H[0][2]), h1 = -(H[1][0] + H[1][1] + H[1][2]), h2 = -(H[2][0] + H[2][1] + H[2][2]);
+    vadd<R>(D, out, tv.x, h0, h1, h2);
+    double q = 0.0;
+    if constexpr (sizeof(R) == 4) {
+        q = V0.x * h0 + V0.y * h1 + V0.z * h2;
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
+        for (int i = 0; i < 3; ++i) {
+            const v3<double> &V = i == 0 ? V1 : i == 1 ? V2 : V3;
+            q += V.x * H[0][i] + V.y * H[1][i] + V.z * H[2][i];
+        }
+    } else {
 #pragma unroll
-        for (int i = 0; i < 3; ++i) q += dp[a][i] * H[a][i];
-    return double(q);
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) q += dp[a][i] * H[a][i];
+    }
+    return q;
 }
 template <typename R, bool CO>
 __global__ void __launch_bounds__(EB) k_hvp_tet(Dev<R> D, const double4_32a *v, double4_32a *out)
@@ -234,8 +245,8 @@ __device__ inline double hvp_pair(const Dev<R> &D, int k, const double4_32a *v, 
     double w[3] = {0.0, 0.0, 0.0};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        const v3<R> V = vload(D, v, vid[j]);
-        w[0] += double(ap.c[j]) * double(V.x); w[1] += double(ap.c[j]) * double(V.y); w[2] += double(ap.c[j]) * double(V.z);
+        const v3<double> V = vload(D, v, vid[j]);
+        w[0] += double(ap.c[j]) * V.x; w[1] += double(ap.c[j]) * V.y; w[2] += double(ap.c[j]) * V.z;
     }
     const double s = w[0] * double(ap.t[0]) + w[1] * double(ap.t[1]) + w[2] * double(ap.t[2]);
     const double A = ap.A, Bc = ap.B;

@@ -1,5 +1,6 @@
 """The differentiation calls at the edges of what they accept."""
 import dataclasses
+import math
 
 import numpy as np
 import pytest
@@ -117,3 +118,24 @@ def test_reverse_step_without_room_for_the_record(B):  # noqa: F811
         sim.close()
     for p, q in zip(*out):
         assert np.linalg.norm(p - q) <= 1e-8 * np.linalg.norm(q)   # 1e-11 times the condition number of about 1e3
+
+
+@pytest.mark.parametrize("cells", [(9, 11, 13), (20, 20, 20)])   # one cluster; the whole grid
+def test_fp32_step_length_is_summed_in_double(B, O, cells):  # noqa: F811
+    """One CG iteration: lambda = alpha P r with alpha = r.P r / p.H p.  H p is the FP32 form's (sim_eval_hvp), and alpha
+    the quotient of sums in double over it, whatever the order: N u of a sum of N positive terms, 30,000 u < 1e-11.  The
+    segmented scatter makes P the same from call to call."""
+    sc, x, rng = strained(cells, 23)
+    sim = B.Sim(sc, precision=1, scatter=B.SIM_SCATTER_SEGMENTED)
+    _, d = B.sim_eval_gradient(sim.h, x, x)
+    P = (np.float32(1.0) / d.astype(np.float32)).astype(np.float64)
+    r = rng.normal(size=x.shape)
+    p = P * r
+    q = B.sim_eval_hvp(sim.h, x, p)
+    alpha = math.fsum((r * p).ravel()) / math.fsum((p * q).ravel())
+    _, av, it, _ = B.sim_adjoint_step(sim.h, x, r, np.zeros_like(r), tol=1e-30, max_iters=1)
+    assert it == 1
+    lam = av / (sc.dt * O.Oracle.from_scene(sc).mass()[:, None])
+    got = np.median(lam / p)
+    assert abs(got / alpha - 1.0) < 1e-11, got / alpha - 1.0
+    sim.close()
