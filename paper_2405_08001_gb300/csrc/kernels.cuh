@@ -1172,8 +1172,9 @@ __device__ inline void pair_grad(const Dev<R> &D, const int4 &q, int par, bool n
         R b1, b2;
         barrier_d12r<R, sizeof(R) == 8>(d, r, R(D.dhat), b1, b2);
         if constexpr (sizeof(R) == 8) {   // one division (Quot says why)
-            const R i = R(1) / d, bd = b1 * i;
-            A = R(D.kappa) * ((b2 - bd) * i * i);
+            const Quot<true, R> by(d);
+            const R bd = by(b1);
+            A = R(D.kappa) * by(by(b2 - bd));
             B = R(D.kappa) * bd;
         } else {
             A = R(D.kappa) * (b2 / (d * d) - b1 / (d * d * d));
@@ -1305,20 +1306,9 @@ __device__ inline void beta_terms(const R gv[3], const R dv[3], const R g0[3], c
 {
 #pragma unroll
     for (int q = 0; q < 5; ++q) { th[q] = R(0); tl[q] = R(0); }
-    R Pv[3];
-    if constexpr (sizeof(R) == 4) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) Pv[a] = precond<R>(dv[a], m);
-    } else {   // one division for the three entries of precond
-        R d[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) d[a] = dv[a] > R(1e-3) * m ? dv[a] : m;
-        const R d12 = d[1] * d[2], i = R(1) / (d[0] * d12), i0 = i * d[0];
-        Pv[0] = i * d12; Pv[1] = i0 * d[2]; Pv[2] = i0 * d[1];
-    }
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const R P = Pv[a];
+        const R P = precond<R>(dv[a], m);
         const R g = gv[a], y = g - g0[a];
         pg[a] = g * P;
         if constexpr (sizeof(R) == 4) {

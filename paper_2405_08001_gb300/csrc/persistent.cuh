@@ -28,6 +28,8 @@
 // 2.1 us on 304 blocks and 1.5 us on 16) and the reductions' partials go straight into the other blocks' shared memory.
 #pragma once
 
+#include <float.h>
+
 #include "broadphase.cuh"
 #include "kernels.cuh"
 
@@ -243,7 +245,7 @@ template <typename R, int PB, bool CL> struct PShared {
     double res[NQ + 1];   // reduced results: sums, then the max
     double o[3];          // scalars computed by thread 0 and broadcast to the block: beta, g^T P g, alpha
     double ab;            // -g.p / p^T H p
-    double ig, e0;        // kept by the last warp: 1 / g^T P g of this iteration (0 below 1e-300), Delta E_0
+    double g0, ig, e0;    // kept by the last warp: g^T P g of the iteration before, its reciprocal (0 if subnormal), Delta E_0
     int oi[2];            // restarted, capped
     int cv;               // kept by the last warp: the eps rule fired
     float xmax;           // Ctrl::xmax_bits
@@ -562,7 +564,8 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
     const bool keeper = threadIdx.x == PB - 32;   // the last warp's first thread keeps ig, e0 and cv
     if (keeper) {
         const double g = (volatile double &)c->gPg_prev;
-        sh.ig = g > 1e-300 ? 1.0 / g : 0.0;
+        sh.g0 = g;
+        sh.ig = g >= DBL_MIN ? 1.0 / g : 0.0;
         sh.e0 = (volatile double &)c->dE0;
         sh.cv = (volatile int &)c->converged;
         sh.xmax = get_xmax(c);
@@ -887,13 +890,13 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
                 int rs = 0;
                 if (D.beta_rule == 0) {
                     gPg = t[1];
-                    if (k > 0) { bt = t[0] * sh.ig; if (bt < 0.0) bt = 0.0; }
+                    if (k > 0) { bt = Quot<true, double>(sh.g0, sh.ig)(t[0]); if (bt < 0.0) bt = 0.0; }
                     gp_new = -gPg + bt * t[2];
                 } else {
                     gPg = t[4];
                     if (k > 0 && !(fabs(t[2]) < 1e-30)) {
-                        const double iy = 1.0 / t[2];
-                        bt = t[0] * iy - (t[1] * iy) * (t[3] * iy);
+                        const Quot<true, double> by(t[2]);
+                        bt = by(t[0]) - by(t[1]) * by(t[3]);
                     }
                     gp_new = -gPg + bt * t[3];
                 }
@@ -905,7 +908,10 @@ __global__ void __launch_bounds__(PB, MINB) k_persistent(Dev<R> D, BPDev B, Pers
             __syncthreads();
             beta = sh.o[0];
             na = sh.fi;
-            if (keeper) sh.ig = sh.o[1] > 1e-300 ? 1.0 / sh.o[1] : 0.0;
+            if (keeper) {
+                sh.g0 = sh.o[1];
+                sh.ig = sh.o[1] >= DBL_MIN ? 1.0 / sh.o[1] : 0.0;
+            }
         }
         // ------------------------------------------------------------ a5-a7: direction, p^T H p and the step
         double alpha;

@@ -66,10 +66,25 @@ static void bounds(int ee, double ratio, double s0, double s1, int n)
     std::printf("%d %.3e\n", above, worst);
 }
 
+// Quot<true> against the division: prints how many of n quotients differ
+static void quotients(int n)
+{
+    std::mt19937_64 g(2);
+    std::uniform_real_distribution<double> U(1, 2), E(-60, 60);
+    int differ = 0;
+    for (int t = 0; t < n; ++t) {
+        const double a = (g() & 1 ? -1 : 1) * std::ldexp(U(g), (int)E(g)), d = std::ldexp(U(g), (int)E(g));
+        if (Quot<true, double>(d)(a) != a / d) ++differ;
+    }
+    std::printf("%d\n", differ);
+}
+
 int main(int argc, char **argv)
 {
     if (argc == 7 && !std::strcmp(argv[1], "bounds"))
         bounds(std::atoi(argv[2]), std::atof(argv[3]), std::atof(argv[4]), std::atof(argv[5]), std::atoi(argv[6]));
+    else if (argc == 3 && !std::strcmp(argv[1], "quotients"))
+        quotients(std::atoi(argv[2]));
     else return 2;
     return 0;
 }

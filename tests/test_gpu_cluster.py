@@ -46,3 +46,15 @@ def test_same_step_as_the_whole_grid(B, make, kw):  # noqa: F811
         out.append(sim.state()[0])
         sim.close()
     assert np.abs(out[0] - out[1]).max() <= 1e-9 * np.abs(out[1] - sc.x0).max()
+
+
+@pytest.mark.parametrize("persistent", [0, 1])
+def test_fp64_first_direction_is_the_rounded_quotient(B, persistent):  # noqa: F811
+    """p_1 = -P g with P = 1 / diag, each operation rounded once: bit by bit, in both launch forms."""
+    sc = S.two_blocks(0)
+    sim = B.Sim(sc, precision=0, persistent=persistent)
+    B.sim_begin_step(sim.h)
+    B.sim_iterate(sim.h, 1)
+    x, g, P, p, *_ = B.sim_get_iterate(sim.h)
+    assert np.array_equal(p, -(P * g))
+    sim.close()

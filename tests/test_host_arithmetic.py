@@ -27,3 +27,9 @@ def test_candidate_bound_is_below_the_distance(program, ee, ratio, sin2):
     """No candidate's stored bound exceeds its distance: nearly parallel edges and sliver triangles, edges of 5 to 300 dhat."""
     above, worst = program("bounds", ee, ratio, *sin2, 100000)
     assert above == "0", worst
+
+
+def test_quotients_by_one_reciprocal_are_the_divisions(program):
+    """The FP64 pairs' and beta's quotients, formed from one reciprocal and corrected by their residual, are those of the
+    division: by Markstein's theorem for every divisor but the one whose mantissa is all ones."""
+    assert program("quotients", 2000000) == ["0"]
