@@ -96,6 +96,67 @@ __device__ inline void seg_warp_max(R m, int key, unsigned long long *mx)
     if (key >= 0 && (lane == 31 || kn != key)) atomicMax(mx + key, max_bits<R>(m));
 }
 
+// A sum over lanes on its way: float-float over a whole stay is added up with a third float for the tails' rounding (five
+// levels of float-float there lost three times what 32 items a time lose; so it loses less).
+template <typename R> struct LaneSum;
+template <> struct LaneSum<double> {
+    double v;
+    __device__ inline static LaneSum of(const Acc<double> &a) { return {a.v}; }
+    __device__ inline LaneSum xor_lane(int o) const { return {__shfl_xor_sync(0xffffffffu, v, o)}; }
+    __device__ inline void add(const LaneSum &b) { v += b.v; }
+    __device__ inline double value() const { return v; }
+};
+template <> struct LaneSum<float> {
+    float h, l, m;
+    __device__ inline static LaneSum of(const Acc<float> &a) { return {a.h, a.l, 0.0f}; }
+    __device__ inline LaneSum xor_lane(int o) const
+    {
+        return {__shfl_xor_sync(0xffffffffu, h, o), __shfl_xor_sync(0xffffffffu, l, o), __shfl_xor_sync(0xffffffffu, m, o)};
+    }
+    __device__ inline static float two_sum(float x, float y, float &e)
+    {
+        const float s = __fadd_rn(x, y), b = __fsub_rn(s, x);
+        e = __fadd_rn(__fsub_rn(x, __fsub_rn(s, b)), __fsub_rn(y, b));
+        return s;
+    }
+    __device__ inline void add(const LaneSum &b)
+    {
+        float e, e1, e2;
+        h = two_sum(h, b.h, e);
+        l = two_sum(two_sum(l, b.l, e1), e, e2);
+        m = __fadd_rn(__fadd_rn(m, b.m), __fadd_rn(e1, e2));
+    }
+    __device__ inline double value() const { return (double)h + ((double)l + (double)m); }
+};
+// The warp's N sums, each in some lanes: at the first levels a lane hands half of its quantities over and keeps the other
+// half, and in the end converts and adds its one (a double operation costs as much for one lane as for 32).  Returns the
+// quantity of the calling lane's sum, or -1.
+template <typename R, int N> __device__ inline int warp_sums(const Acc<R> (&a)[N], LaneSum<R> &out)
+{
+    constexpr int P = N > 4 ? 8 : N > 2 ? 4 : N;
+    static_assert(N <= 8 && N != 2, "one, or padded to four or eight");
+    const int lane = threadIdx.x & 31;
+    LaneSum<R> t[P];
+#pragma unroll
+    for (int q = 0; q < P; ++q) t[q] = q < N ? LaneSum<R>::of(a[q < N ? q : 0]) : LaneSum<R>{};
+    int o = 16, q = 0;
+#pragma unroll
+    for (int n = P / 2; n > 0; n /= 2, o /= 2) {
+        const bool up = (lane & o) != 0;
+        if (up) q += n;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const LaneSum<R> give = up ? t[i] : t[i + n];
+            if (up) t[i] = t[i + n];
+            t[i].add(give.xor_lane(o));
+        }
+    }
+#pragma unroll
+    for (int n = 16 / P; n > 0; n /= 2, o /= 2) t[0].add(t[0].xor_lane(o));
+    out = t[0];
+    return (lane & (32 / P - 1)) == 0 && q < N ? q : -1;
+}
+
 // Running sums of a warp whose items mostly stay in one group: while all its lanes' items have the group of the sums so
 // far, each lane adds its own; a change of group sends the sums to the accumulator.  The scan of seg_warp_sum, about
 // 100 instructions a quantity, thus runs once per group that a warp meets instead of once per 32 items.
@@ -124,12 +185,11 @@ template <typename R, int N> struct SegRun {
     __device__ inline void flush(double *acc, int q0, unsigned long long *mx = nullptr)
     {
         if (key >= 0) {
+            LaneSum<R> t;
+            const int q = warp_sums<R, N>(a, t);
+            if (q >= 0) atomicAdd(acc + (size_t)key * 8 + q0 + q, t.value());
 #pragma unroll
-            for (int q = 0; q < N; ++q) {
-                for (int o = 16; o > 0; o >>= 1) a[q].add(a[q].shfl_down(o));
-                if ((threadIdx.x & 31) == 0) atomicAdd(acc + (size_t)key * 8 + q0 + q, a[q].value());
-                a[q] = Acc<R>();
-            }
+            for (int i = 0; i < N; ++i) a[i] = Acc<R>();
             if (mx) {
                 for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
                 if ((threadIdx.x & 31) == 0) atomicMax(mx + key, max_bits<R>(m));
