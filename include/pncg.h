@@ -137,13 +137,15 @@ typedef struct {
                              vertices takes no step.  Works without scene_of_vert (one object, two groups). */
     int32_t block_shape;  /* block shape of the persistent form: 0 (default) = by the mesh's size: one thread-block
                              cluster of 16 blocks of 256 threads up to 8,192 tets in the FP32 form, 4,096 in FP64; 256
-                             threads x 1 block per SM up to three tets a thread (several scenes or objects: one); else,
-                             with SIM_SCATTER_BLOCK, and for FCR and ARAP in the FP32 form above the cluster's size,
-                             256 threads x 2 blocks per SM;
+                             threads x 1 block per SM up to three tets a thread (several scenes or objects: one), in
+                             FP64 not between one and four thirds; else, with SIM_SCATTER_BLOCK, and for FCR and ARAP
+                             in the FP32 form above the cluster's size, 256 threads x 2 blocks per SM (which no value
+                             names: below those sizes the autotuner can choose it);
                              1 = 512 x 1, 2 = 256 x 3, 3 = 256 x 1, 4 = 384 x 1 (the compiler fits the registers
                              per thread to the shape: 128, 128, 85, 255, 168); -1 = autotuned: from the second time
                              step on, each shape runs two time steps (interleaved), timed on the GPU (those steps
-                             synchronise), and the shape of the fastest step runs from then on
+                             synchronise; on a mesh of the cluster's size the cluster and 256 x 2 both), and the shape
+                             of the fastest step runs from then on
                              (sim_stats.block_threads, blocks_per_sm).
                              With persistent = 2 the per-phase form is timed as one more candidate.
                              SIM_SCATTER_BLOCK keeps shape 0. */

@@ -237,14 +237,16 @@ public:
         if (gexec) { cudaGraphExecDestroy(gexec); gexec = nullptr; }
         if (graph) { cudaGraphDestroy(graph); graph = nullptr; }
     }
-    // candidate c: a shape index >= 0 (persistent form) or -1 (one kernel per phase)
+    // candidate c: a shape index >= 0 (persistent form), WHOLE_GRID (shape 0 on the whole grid of a mesh that has the cluster
+    // form) or -1 (one kernel per phase)
+    static constexpr int WHOLE_GRID = N_PSHAPES;
     void apply_config(int c)
     {
-        const bool want_persist = c >= 0;
-        const int want_shape = c >= 0 ? c : shape;
-        if (persist != want_persist || shape != want_shape) {
+        const bool want_persist = c >= 0, want_cluster = c == 0 && cluster > 0;
+        const int want_shape = c < 0 ? shape : c == WHOLE_GRID ? 0 : c;
+        if (persist != want_persist || (want_persist && (shape != want_shape || use_cluster != want_cluster))) {
             persist = want_persist;
-            set_shape(want_shape);
+            set_shape(want_shape, c != WHOLE_GRID);
             drop_graph();
         }
     }
@@ -938,10 +940,10 @@ private:
         if (M.nseg > 1) return nt <= round;
         return nt <= 3 * round && !(f64 && nt > round && 3 * nt <= 4 * round);
     }
-    void set_shape(int sh)
+    void set_shape(int sh, bool cl = true)
     {
         shape = sh;
-        use_cluster = sh == 0 && cluster > 0;
+        use_cluster = cl && sh == 0 && cluster > 0;
         pgrid = use_cluster ? cluster : shape_grid[sh];
     }
 
@@ -992,6 +994,7 @@ private:
         tune_cfg.clear();
         if (M.opt.block_shape < 0 && !block_scatter) {
             for (int sh = 0; sh < N_PSHAPES; ++sh) if (shape_grid[sh] > 0) tune_cfg.push_back(sh);
+            if (cluster > 0 && shape_grid[0] > 0) tune_cfg.push_back(WHOLE_GRID);
         } else {
             tune_cfg.push_back(shape);
         }

@@ -58,3 +58,16 @@ def test_fp64_first_direction_is_the_rounded_quotient(B, persistent):  # noqa: F
     x, g, P, p, *_ = B.sim_get_iterate(sim.h)
     assert np.array_equal(p, -(P * g))
     sim.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_autotuner_times_every_shape_on_a_small_mesh(B, prec):  # noqa: F811
+    """block_shape = -1 on a mesh that the default runs as one cluster: the tuned steps run 256 x 2 on the whole grid too."""
+    sim = B.Sim(S.two_blocks(0), precision=prec, block_shape=-1)
+    seen = set()
+    for _ in range(14):
+        sim.step(1)
+        st = sim.state()[2]
+        seen.add((st["block_threads"], st["blocks_per_sm"]))
+    assert {(256, 1), (256, 2), (256, 3), (512, 1), (384, 1)} <= seen, seen
+    sim.close()
