@@ -10,13 +10,28 @@ from test_gpu_parity import B, CHECKED, O, TOL, lockstep  # noqa: F401  (B and O
 pytestmark = pytest.mark.gpu
 
 
-# ... and of the next rule: one block of 256 threads an SM up to three rounds of 256 x 152 tets, two above (and in FP64 just
-# above one round)
+def cells_for(tets):
+    """Cell counts (ragged) of a box of at most that many tets, and of nearly as many."""
+    n = tets // 6
+    k = max(1, round(n ** (1.0 / 3.0)))
+    return max(((i, j, n // (i * j)) for i in range(k - 4, k + 5) for j in range(k - 4, i)), key=lambda c: c[0] * c[1] * c[2])
+
+
+def rounds(q):
+    """q tets a thread of one block of 256 threads an SM."""
+    import torch
+    return int(q * 256 * torch.cuda.get_device_properties(0).multi_processor_count)
+
+
+# ... and of the next rule: one block of 256 threads an SM up to three rounds of 256 x SMs tets, two above (and in FP64 up to
+# four thirds of a round above one)
 @pytest.mark.parametrize("prec,cells,blocks", [(1, (1, 1, 1), 1), (1, (9, 11, 13), 1), (1, (11, 11, 12), 1),
                                                (0, (1, 2, 1), 1), (0, (8, 8, 10), 1), (0, (8, 9, 10), 1),
-                                               (0, (23, 12, 23), 1), (0, (19, 18, 19), 2), (0, (21, 20, 21), 1),
-                                               (1, (27, 26, 27), 1), (1, (27, 27, 27), 2)])
+                                               (0, 0.99, 1), (0, 1.1, 2), (0, 1.32, 2), (0, 1.45, 1), (1, 2.98, 1), (1, 3.1, 2)])
 def test_both_sides_of_the_size_rule(B, O, prec, cells, blocks):  # noqa: F811
+    if isinstance(cells, float):
+        q, cells = cells, cells_for(rounds(cells))
+        assert abs(6 * np.prod(cells) / rounds(q) - 1.0) < 0.02     # within the side that q names
     sc = S.cube_drop(n=max(cells), cells=cells, drop=0.0)
     sc.x0 = sc.x0 + np.array([0.0, 0.0, 0.6 * sc.dhat])
     sim = B.Sim(sc, precision=prec)
