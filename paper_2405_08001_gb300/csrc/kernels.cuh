@@ -1146,6 +1146,7 @@ __device__ inline void pair_grad(const Dev<R> &D, const int4 &q, int par, bool n
             t = mkv(__fadd_rn(tf.x.h, tf.x.l), __fadd_rn(tf.y.h, tf.y.l), __fadd_rn(tf.z.h, tf.z.l));
             d = __fadd_rn(df.h, df.l);
             r = __fadd_rn(rf.h, rf.l);
+            near = d < R(1e-3) * R(D.dhat);   // the float distance may have been above it
         }
     } else {
         d = pair_geom<R, true>(ee, ldcg4(D.x + v.x), ldcg4(D.x + v.y), ldcg4(D.x + v.z), ldcg4(D.x + v.w), c, t);

@@ -130,3 +130,29 @@ def test_a_scene_near_the_grids_limit(B):  # noqa: F811
     sim.step(1)
     assert np.abs(sim.state()[0] - x0).max() < 1e-6
     sim.close()
+
+
+def test_fp32_pairs_below_the_line_are_evaluated_in_double(B):  # noqa: F811
+    """Below 1e-3 dhat the FP32 form evaluates a pair in double (n_near_fp64 counts them): also where the float
+    filter's distance lies above the line and the float-float one below.  Crossed edges 1e-6 to 1e-2 of the line below it."""
+    rng = np.random.default_rng(31)
+    dhat, L, X, T = 1e-3, 0.1, [], []
+    for k in range(512):
+        f = 1.0 - 10.0 ** rng.uniform(-6, -2)      # (1e-6 of the line is 1e-12 m; x is rounded to 1e-15)
+        th = rng.uniform(0.3, 1.2)
+        u = np.array([np.cos(th), np.sin(th), 0.0])
+        a = np.array([[-0.4 * L, 0, 0], [0.6 * L, 0, 0], [0.1 * L, -0.2 * L, -0.3 * L], [0.1 * L, 0.2 * L, -0.3 * L]])
+        b = np.array([-0.5 * L * u, 0.5 * L * u, [0, -0.2 * L, 0.3 * L], [0, 0.2 * L, 0.3 * L]]) + [0, 0, 1e-3 * f * dhat]
+        R, o = S.random_rotation(rng), 0.4 * np.array([k % 32, k // 32, 0])
+        for t in (a, b):
+            if np.linalg.det(t[1:] - t[0]) < 0:
+                t = t[[0, 2, 1, 3]]
+            X.append(t @ R.T + o)
+            T.append(np.arange(4) + 4 * len(T))
+    X = np.ascontiguousarray(np.concatenate(X))
+    sc = S.Scene(name="near", rest_x=X, tets=np.array(T, np.int32), x0=X, v0=np.zeros_like(X), youngs=1e5, poisson=0.4, density=1000.0,
+                 dt=1.0 / 60.0, dhat=dhat, kappa=1e-3, iters=1, steps=1)
+    sim = B.Sim(sc, precision=1)
+    B.sim_eval_gradient(sim.h, X, X)
+    assert sim.state()[2]["n_near_fp64"] == 512
+    sim.close()
