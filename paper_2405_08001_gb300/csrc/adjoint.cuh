@@ -62,7 +62,7 @@ template <typename R> __device__ inline void vadd(const Dev<R> &D, double4_32a *
 //   FP64: Dp (2 Psi_2 h^2 V M) + h^2 V Psi_33 det(Dm^-1)^2 (cof(Ds) : Dp) cof(Ds) + h^2 V Psi_3 det(Dm^-1) d cof(Ds)[Dp], with
 // the scalars that the gradient pass at x left (tet_pHp_edges): about 135 FP64 operations where the form on F took 430
 // (82,944 tets: 70 us a pass).  rec (or null): cof(Ds) and h^2 V Psi_3 det(Dm^-1) Ds kept by the solver, whose x stands
-// still (hvp_record): 99 operations.
+// still (hvp_record): 91 operations, and 15 for the corner sums and p^T H_e p.
 //   FP32: (L P F^T + 2 (k1 tr(E) I + k2 E)) Ds^-T, E = L + L^T, L = Dp Ds^-1, from the gradient pass's record: the
 // derivative of the quadratic form of tet_pHp_edges, in which the large terms of a rotating direction never meet.
 constexpr int HVP_REC = 5;   // double4 per tet of the record
@@ -273,8 +273,9 @@ __global__ void __launch_bounds__(EB) k_hvp_pair(Dev<R> D, const double4_32a *v,
 //   product    the tets and pairs add to q; p^T q accumulates beside it from the elements' own p^T H_e p, so that no pass
 //              of its own reads p and q for it
 //   update     alpha = r.z / p.q; x += alpha p, r -= alpha q, z = P r; the sums r.z and r.r
-// It replaces six launches an iteration and a host round trip every eight (82,944 tets: 98 us of kernels, with their gaps
-// 230 us an iteration).  Convergence is looked at every eighth iteration.
+// It replaces six launches an iteration and a host round trip every eight (82,944 tets, about 900 iterations: 100 us an
+// iteration, nearly all of it the kernels themselves, against 38 in one launch, of which the product is 28).  Convergence is
+// looked at every eighth iteration.  The waits at the grid barriers are bounded as the time step's; the cluster's need not be.
 constexpr int CG_PB = 256;
 constexpr int CG_STRIDE = 8;      // iterations between two looks at the residual
 enum { CG_RZ = 0, CG_BETA, CG_RR, CG_BB, CG_IT, CG_N };

@@ -688,7 +688,8 @@ __device__ inline void tet_metric(const Dev<float> &D, const TetIn<float> &in, f
 // log J for NH).  mu h^2 V M enters as its factor, K K^T: G K is formed with compensated (Dot2) products from the
 // float-float G, its terms being up to cond(Dm) times larger than the result.  Both leave the record that tet_pHp_vec reads (e >= 0).  Returns false (and
 // flags the error) when det F <= 0.
-// FP64: 170 FP64 operations a tet where the form on F took about 430, at 1.65 FP64 lanes per clock and SM.
+// FP64: about 140 FP64 operations a tet (the logarithm 17 of them) where the form on F took about 430, at 1.68 FP64 lanes
+// per clock and SM.
 template <typename R>
 __device__ inline bool tet_grad_edges(const Dev<R> &D, const TetIn<R> &in, R gv[4][3], R dv[4][3], int e)
 {

@@ -59,7 +59,7 @@ __device__ inline Mat3 cofactors(const Mat3 &d)
 // p^T M p + h^2 sum_e V_e [mu |dF|^2 + Psi_33 (cof F : dF)^2 + Psi_3 d2det(F)[dF, dF]] in double precision, one
 // thread per tet (and per vertex for the inertia term).  With the edge vectors of the rest, current and direction
 // values Dm, Ds, Dp (columns): J = det Ds / det Dm, cof F : dF = cof(Ds) : Dp / det Dm, d2det(F)[dF, dF] = 2 cof(Dp) : Ds /
-// det Dm and dF = Dp cof(Dm)^T / det Dm, so that neither D_m^-1 nor F is formed.  Bound by FP64 issue (1.65 lanes per
+// det Dm and dF = Dp cof(Dm)^T / det Dm, so that neither D_m^-1 nor F is formed.  Bound by FP64 issue (1.68 lanes per
 // clock and SM): about 175 operations a tet with two divisions, where the form on F took about 400 with nine.  998,250 tets:
 // on F 768 us, on edge vectors 411, with det_forms and log_tab 354.
 __global__ void __launch_bounds__(NA_THREADS) k_pHp_noalloc(NoAllocScratch *scr, int nv, int nt, const double *x,

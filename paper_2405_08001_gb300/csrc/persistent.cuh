@@ -8,9 +8,10 @@
 // needed).  In the FP32 form partial sums are carried as float-float (about 48 bits) on the FP32 pipes; in the FP64
 // form they are doubles.
 //
-// A double operation holds its scheduler's FP64 unit for 64 cycles, however few of the warp's lanes take part (measured:
-// division 450 cycles, square root 690, log 2,100), so the scalar work between two phases, which every thread waits for,
-// is kept short: in one thread per block, with no more than one division; what the next phase does not need (the reciprocal
+// A double operation holds its scheduler's FP64 unit for 64 cycles, however few of the warp's lanes take part (measured;
+// 76 with all four schedulers of an SM at it, 1.68 lanes per clock; division 450 cycles, square root 690, log 2,100), so
+// the scalar work between two phases, which every thread waits for, is kept short: in one thread per block, with no more
+// than one division; what the next phase does not need (the reciprocal
 // for the next beta, Delta E, the eps rule, the records) is left to the last warp, which has the least to do there.
 // Measured with it against every scalar in thread 0 one after another: the 50-iteration step of the 2.5K-tet cube 767 ->
 // 711 us (FP32), the 25-iteration step of the twisted bar 985 -> 955 us (FP32), 5,450 -> 5,310 us (FP64, 50 iterations).
@@ -20,12 +21,16 @@
 // forms p_{k+1} of every vertex it touches from P g and p_k (one rounding order everywhere, so the values agree
 // bitwise); the update pass then stores it as the current direction.
 //
-// Barrier waits are bounded: a block that waits longer than the limit sets ERR_TIMEOUT and carries on; later
-// barriers do not wait once the bit is set, so the launch always terminates and the host reports SIM_ERR_TIMEOUT.
+// Waits at the counter barrier (the whole-grid form) are bounded: a block that waits longer than the limit sets
+// ERR_TIMEOUT and carries on; later barriers do not wait once the bit is set, so the launch always terminates and the
+// host reports SIM_ERR_TIMEOUT.
 //
 // Small meshes run it as one thread-block cluster (the template parameter CL, at most CLUSTER_MAX blocks): the
-// barrier is the hardware's cluster barrier (0.23 us for 16 blocks of 512 threads where the counter barrier takes
+// barrier is the hardware's cluster barrier (0.19 us for 16 blocks of 256 threads where the counter barrier takes
 // 2.1 us on 304 blocks and 1.5 us on 16) and the reductions' partials go straight into the other blocks' shared memory.
+// That barrier has no limit and needs none: the hardware starts a cluster's blocks together or not at all, and every
+// block passes the same sequence of barriers, whatever errors it has flagged (the conditions around them are uniform
+// over the launch), so no arrival can be missing.
 #pragma once
 
 #include <float.h>
