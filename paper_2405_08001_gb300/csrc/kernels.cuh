@@ -408,23 +408,24 @@ template <typename R> __device__ inline void tet_material(const Dev<R> &D, int e
     if (D.escale) { R s = D.escale[e]; mu *= s; lam *= s; }
 }
 
-// The lower triangular factor K of f^2 W W^T (entries 00 10 20 11 21 22), W = D_m^-1, from W's rows by Gram-Schmidt (u
-// times W's condition number) and not from their products (its square).
+// The lower triangular factor K of f^2 W W^T (entries 00 10 20 11 21 22), W = D_m^-1, from W's rows w_i in the orthogonal
+// frame w_0, c x w_0, c = w_0 x w_1 (u times W's condition number) and not from their products (its square).
 __host__ __device__ inline void tri_factor(const double w[3][3], double f, double k[6])
 {
-    double q[3][3], l[3][3];
-    for (int i = 0; i < 3; ++i) {
-        for (int c = 0; c < 3; ++c) q[i][c] = w[i][c];
-        for (int j = 0; j < i; ++j) {
-            const double d = l[i][j] = q[i][0] * q[j][0] + q[i][1] * q[j][1] + q[i][2] * q[j][2];
-            for (int c = 0; c < 3; ++c) q[i][c] -= d * q[j][c];
-        }
-        l[i][i] = sqrt(q[i][0] * q[i][0] + q[i][1] * q[i][1] + q[i][2] * q[i][2]);
-        if (i == 2) break;
-        const double r = 1.0 / l[i][i];
-        for (int c = 0; c < 3; ++c) q[i][c] *= r;
-    }
-    k[0] = f * l[0][0]; k[1] = f * l[1][0]; k[2] = f * l[2][0]; k[3] = f * l[1][1]; k[4] = f * l[2][1]; k[5] = f * l[2][2];
+    auto dot = [](const double a[3], const double b[3]) { return a[0] * b[0] + a[1] * b[1] + a[2] * b[2]; };
+    auto cross = [](const double a[3], const double b[3], double o[3]) {
+        o[0] = a[1] * b[2] - a[2] * b[1]; o[1] = a[2] * b[0] - a[0] * b[2]; o[2] = a[0] * b[1] - a[1] * b[0];
+    };
+    double c[3], n[3];
+    cross(w[0], w[1], c);
+    cross(c, w[0], n);
+    const double r0 = sqrt(dot(w[0], w[0])), rc = sqrt(dot(c, c)), f0 = f / r0, fc = f / rc;
+    k[0] = f * r0;
+    k[1] = f0 * dot(w[1], w[0]);
+    k[2] = f0 * dot(w[2], w[0]);
+    k[3] = f0 * rc;
+    k[4] = fc / r0 * dot(w[2], n);
+    k[5] = fc * fabs(dot(w[2], c));
 }
 
 // The per-tet constants a gradient evaluation streams in (coalesced, structure-of-arrays in memory).  The densities
