@@ -177,6 +177,7 @@ __device__ inline void put_xmax(const BPDev &B, unsigned int m)
     m = __reduce_max_sync(0xffffffffu, m);
     if ((threadIdx.x & 31) != 0 || m == 0u) return;
     if (!B.xbh) m = __float_as_uint(__double2float_ru(__hiloint2double((int)m, -1)));
+    m = min(m, 0x7f800000u);   // NaN counts as infinite
     if (m > __ldcg(&B.ctrl->xmax_bits)) atomicMax(&B.ctrl->xmax_bits, m);
 }
 __device__ inline float get_xmax(const Ctrl *c) { return __uint_as_float(__ldcg(&c->xmax_bits)); }

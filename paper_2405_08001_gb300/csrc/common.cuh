@@ -47,7 +47,7 @@ struct Ctrl {
     int32_t rebuild;       // 1 = candidate build needed before the next gradient pass
     uint32_t cell_bits;    // float bits of the hash cell size of the current build (atomicMax of extents)
     uint32_t xmax_bits;    // float bits of the largest |coordinate| of a vertex (FP32 form: of its float head) at the candidate
-                           // builds since the state was set
+                           // builds since the state was set, or an evaluation's position
     int32_t k;             // index of the next iteration within the step
     int32_t n_rebuilds;
     int32_t n_capped;

@@ -81,7 +81,7 @@ __global__ void k_eval_in(Dev<R> D, const double *x, const double *xt, bool kin,
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0) {
         Ctrl *c = D.ctrl;
-        c->rebuild = 1; c->cell_bits = 0u; c->n_active = 0; c->n_near64 = 0;
+        c->rebuild = 1; c->cell_bits = 0u; c->xmax_bits = 0u; c->n_active = 0; c->n_near64 = 0;
     }
     if (i >= D.nv) return;
     const double4_32a T = D.xtil[i];
@@ -101,7 +101,7 @@ template <typename R> __global__ void k_eval_out(Dev<R> D, const double4_32a *xs
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0) {
         Ctrl *c = D.ctrl;
-        c->rebuild = 1; c->cell_bits = 0u; c->n_active_last = c->n_active; c->n_active = 0;
+        c->rebuild = 1; c->cell_bits = 0u; c->xmax_bits = 0u; c->n_active_last = c->n_active; c->n_active = 0;
     }
     if (i >= D.nv) return;
     const double4_32a T = xtsave[i];

@@ -156,3 +156,21 @@ def test_fp32_pairs_below_the_line_are_evaluated_in_double(B):  # noqa: F811
     B.sim_eval_gradient(sim.h, X, X)
     assert sim.state()[2]["n_near_fp64"] == 512
     sim.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_an_evaluation_at_nan_leaves_the_skip_as_it_was(B, prec):  # noqa: F811
+    """An evaluation that fails on a non-finite position does not reach the next step's candidates."""
+    sc = S.two_blocks(0)
+    active = []
+    for bad in (False, True):
+        sim = B.Sim(sc, precision=prec, iters=4)
+        if bad:
+            x = sc.x0.copy()
+            x[5] = np.nan
+            with pytest.raises(B.SimError):
+                B.sim_eval_gradient(sim.h, x, x)
+        sim.step(1)
+        active.append(B.sim_get_trace(sim.h)[:, B.TRACE_COLUMNS.index("n_active")].astype(int).tolist())
+        sim.close()
+    assert active[0] == active[1] and max(active[0]) > 0, active
