@@ -86,7 +86,7 @@ __device__ inline void tet_hvp_edges(const Dev<R> &D, int e, const int4 &tv, con
     if constexpr (sizeof(R) == 4) {
         const float4 q0 = __ldcg(D.tS + e), q1 = __ldcg(D.tS + n + e), q2 = __ldcg(D.tS + 2 * n + e);
         const float4 q3 = __ldcg(D.tS + 3 * n + e);
-        const float k1 = __ldcg(D.tk + e), k2 = q3.w;
+        const float hv = D.hv[e], k1 = hv * __ldcg(D.tk + e), k2 = hv * q3.w;
         const float Z[3][3] = {{q0.x, q0.y, q0.z}, {q0.w, q1.x, q1.y}, {q1.z, q1.w, q2.x}};
         const float S[3][3] = {{q2.y, q2.z, q2.w}, {q2.z, q3.x, q3.y}, {q2.w, q3.y, q3.z}};
         float L[3][3], E[3][3];
