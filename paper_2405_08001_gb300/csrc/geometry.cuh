@@ -186,7 +186,7 @@ template <typename R, bool F64 = false> __host__ __device__ inline void barrier_
     if constexpr (F64) {
         const R L = log1p_tab(r / dhat);
         const R q = r / d;
-        b1 = -r * (R(2) * L + q);
+        b1 = fma(R(-2) * r, L, -(r * q));   // (rms 0.56 to 0.68 units of 2^-53; -r (2 L + q): 0.71 to 0.82)
         b2 = R(-2) * L - R(4) * q + q * q;
     } else {
         const R L = log1p(r / dhat);

@@ -79,12 +79,34 @@ static void quotients(int n)
     std::printf("%d\n", differ);
 }
 
+// b' of the barrier at gaps d = dhat (1 - x), x in [x0, x1]: the rms error, in units of 2^-53, of the FP64 form (whose
+// logarithm is the library's on the host) and of -2 r L - r^2 / d with one fused rounding
+static void barrier(double x0, double x1, int n)
+{
+    std::mt19937_64 g(3);
+    std::uniform_real_distribution<double> U(0, 1);
+    const double dhat = 1e-3;
+    long double e = 0, ref = 0;
+    for (int t = 0; t < n; ++t) {
+        const double d = dhat * (1 - x0 * std::pow(x1 / x0, U(g))), r = d - dhat;
+        const long double b = -2.0L * r * log1pl((long double)r / dhat) - (long double)r * r / d;
+        double b1, b2;
+        barrier_d12r<double, true>(d, r, dhat, b1, b2);
+        const double c1 = std::fma(-2.0 * r, std::log1p(r / dhat), -(r * r / d));
+        e += (b1 / b - 1) * (b1 / b - 1);
+        ref += (c1 / b - 1) * (c1 / b - 1);
+    }
+    std::printf("%.4f %.4f\n", (double)sqrtl(e / n) * 0x1p53, (double)sqrtl(ref / n) * 0x1p53);
+}
+
 int main(int argc, char **argv)
 {
     if (argc == 7 && !std::strcmp(argv[1], "bounds"))
         bounds(std::atoi(argv[2]), std::atof(argv[3]), std::atof(argv[4]), std::atof(argv[5]), std::atoi(argv[6]));
     else if (argc == 3 && !std::strcmp(argv[1], "quotients"))
         quotients(std::atoi(argv[2]));
+    else if (argc == 5 && !std::strcmp(argv[1], "barrier"))
+        barrier(std::atof(argv[2]), std::atof(argv[3]), std::atoi(argv[4]));
     else return 2;
     return 0;
 }

@@ -33,3 +33,12 @@ def test_quotients_by_one_reciprocal_are_the_divisions(program):
     """The FP64 pairs' and beta's quotients, formed from one reciprocal and corrected by their residual, are those of the
     division: by Markstein's theorem for every divisor but the one whose mantissa is all ones."""
     assert program("quotients", 2000000) == ["0"]
+
+
+# x = 1 - d / dhat, from just below dhat to near contact
+@pytest.mark.parametrize("x", [(1e-8, 1e-4), (1e-4, 1e-2), (1e-2, 0.3), (0.3, 0.99)])
+def test_fp64_barrier_slope_rounds_no_more_than_its_formula(program, x):
+    """b' = -2 r L - r^2 / d from r / d, which b'' needs too: as many roundings as the formula's own (200,000 samples give
+    either rms to 1 %, the margin is 5)."""
+    ours, ref = map(float, program("barrier", *x, 200000))
+    assert ours <= 1.05 * ref, (ours, ref)
