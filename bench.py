@@ -144,7 +144,7 @@ def algorithmic_bytes(kernel: str, prec: int, sizes: dict, n_cand: int, n_active
     and the directions are 4-vectors of the element type (16 B float, 32 B double).  Per tet: 4 indices (16 B),
     the constants on edge vectors (FP32: 20 floats, the float-float rest metric and the triangular factor of
     mu h^2 V Dm^-1 Dm^-T; FP64: 8 doubles, and the factor's 6, which the p^T H p pass reads; in FP32 it reads the record
-    instead).  Candidates:
+    and h^2 V instead).  Candidates:
     int4 (16 B); active pairs (64 B float form, 112 B double form) written by the gradient pass and read by p^T H p.
     The persistent step stores P g in the beta pass and forms the direction inside the p^T H p pass.  The per-tet
     p^T H p record (68 B in FP32, 16 B in FP64: written by the gradient pass, read by the p^T H p pass) is counted in
@@ -162,7 +162,7 @@ def algorithmic_bytes(kernel: str, prec: int, sizes: dict, n_cand: int, n_active
     if kernel == "k_dir":
         return V * 4 * v4
     if kernel == "k_pHp":
-        return (T * (16 + rec + (0 if prec == 1 else 48)) + V * ((0 if prec == 1 else xpos) + (5 if persistent else 1) * v4) +
+        return (T * (16 + rec + (4 if prec == 1 else 48)) + V * ((0 if prec == 1 else xpos) + (5 if persistent else 1) * v4) +
                 n_active * act)
     if kernel == "k_update":
         disp = 32 if prec == 1 else 32      # FP32: float copy now + at the build; FP64: x at the build
